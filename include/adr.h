@@ -47,7 +47,8 @@ typedef enum {
     ADR_EGEOM = 5,    /* the curve families do not cover the domain (§3, §6): tracing failed
                          (closed integral curve, |beta| = 0 on a curve), a family has no
                          inflow boundary, or an interior node meets no curve of a family */
-    ADR_ETIMEOUT = 6  /* a bounded device wait gave up (tensor-core network kernels) */
+    ADR_ETIMEOUT = 6  /* a bounded device wait gave up (tensor-core network kernels, grid
+                         barriers of the one-launch iteration) */
 } adr_status;
 
 typedef enum {
@@ -256,7 +257,8 @@ adr_status adr_paper_u0(adr_problem* prob, double* u0);
 /*
  * adr_time_kernels -- device time of the sweep kernels of one split step, each
  * launched reps times back to back on the handle's stream in the launch
- * configuration of the solve, timed with CUDA events on that stream: B gather,
+ * configuration of the solve's graph (small grids solve in one launch, whose
+ * phases are not timed apart), timed with CUDA events on that stream: B gather,
  * B curve solve, B curve->grid map, G gather, G curve solve, G map (+ norms).
  * The gathers are passes of their own through the grid (both precision
  * modes, single handles and batches).  With

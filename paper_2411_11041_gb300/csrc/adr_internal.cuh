@@ -78,6 +78,7 @@ struct Family {
     // soff[curve] + j*T + t, T the curve's block size)
     int n_slots = 0;
     int cmax = 1;             // rows of the longest chunk (a thread's rows) of the family
+    int tmax = 32;            // largest block size T of the family's curves
     int* soff = nullptr;      // [n_lines+1]
     int* ncell = nullptr;     // [n_nodes] the same cells in node order (-1 at the curves' ends;
                               // FP64 through the grid: the separate gather pass)
@@ -130,6 +131,9 @@ struct IterState {
     unsigned long long corr_bits;  // running max |dt d| of the step's corrections (bits)
     double corr;                   // the last step's largest correction (reduced precision)
     int fp32_steps;                // steps done with FP32 corrections
+    int timeout;                   // one-launch iteration: a grid barrier's wait gave up
+    unsigned long long corr_loop[2];  // its running max |dt d| by the step's parity
+    unsigned bar;                  // its barrier arrivals
     int pad;
 };
 
@@ -152,6 +156,8 @@ struct Problem {
     int N = 0;             // nx*ny
     int n_interior = 0;
     int n_sm = 0;
+    bool coop = false;     // the device takes cooperative launches
+    int n_loop_blocks = 0; // blocks of the one-launch iteration the partial sums have room for
     int rows_per_thread = 16;   // launch shape of the curve solve (<= 16 rows per thread)
     int map_blocks_per_sm = 4;  // launch shape of the curve -> grid map
     bool const_beta = false;
@@ -256,6 +262,13 @@ adr_status launch_mask_copy(Problem* p, const double* in, double* out);
 // make the iteration's factorisation family 0's active one (sweep.cu); a
 // batch reads the active buffers once, when it is built
 adr_status ensure_iteration_active(Problem* p);
+// the outer iteration in one cooperative launch (sweep.cu), measured faster up
+// to about 500^2 nodes; larger grids take the graph of separate kernels, whose
+// blocks fill the chip by themselves
+constexpr int kLoopMaxNodes = 1 << 18;
+bool loop_applies(const Problem* p);
+adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
+                             double* half, double tol, int max_iter, bool norms);
 // Anderson extrapolation (accel.cu)
 adr_status launch_anderson(Problem* p);
 adr_status alloc_anderson(Problem* p);

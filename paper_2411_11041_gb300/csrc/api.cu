@@ -3,6 +3,7 @@
 // parabolic time stepping.  See include/adr.h for the contract.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -224,11 +225,15 @@ adr_status run_iteration(adr_problem* h, double theta, double dt, double sig,
         TRY(prepare_family(p, 0, theta * dt, dt, sig, 0));
         TRY(prepare_family(p, 1, theta * dt, dt, sig, 0));
         TRY(load_family(p, fextra, fx_scale));
+        if (!accel && loop_applies(p)) {
+            TRY(launch_solve_loop(p, dt, p->ubuf[0], p->ubuf[1], p->ubuf[0], p->ubuf[2], tol, max_iter, true));
+        } else {
         if (!h->exec || h->g_theta != theta || h->g_dt != dt || h->g_sig != sig ||
             h->g_fextra != fextra || h->g_scale != fx_scale || h->g_tol != tol ||
             h->g_max_iter != max_iter || h->g_accel != accel)
             TRY(build_graph(h, theta, dt, sig, fextra, fx_scale, tol, max_iter, accel));
         ADR_CUDA_TRY(cudaGraphLaunch(h->exec, p->stream));
+        }
     }
     if (p->opts.transfer) TRY(finish_direct(p, max_iter, out, iter_out, midpoint));
     else TRY(launch_finish(p, out, iter_out, midpoint));
@@ -241,6 +246,10 @@ adr_status run_iteration(adr_problem* h, double theta, double dt, double sig,
     ADR_CUDA_TRY(cudaStreamSynchronize(p->stream));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, h->ev0, h->ev1);
+    if (st.timeout) {
+        set_error("the iteration gave up waiting at a grid barrier; its outputs are not valid");
+        return ADR_ETIMEOUT;
+    }
     *converged = st.converged != 0;
     if (st.iter > 0 && !std::isfinite(st.rel)) {
         *converged = false;
@@ -441,6 +450,9 @@ adr_status adr_create(const adr_grid* grid, const uint8_t* mask, double mu, doub
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, dev);
+        int coop = 0;
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        p->coop = coop != 0;
     }
     adr_status s = ADR_OK;
     auto fail = [&](adr_status st) {
@@ -476,7 +488,8 @@ adr_status adr_create(const adr_grid* grid, const uint8_t* mask, double mu, doub
             return fail(cuda_fail(e, "cudaMemsetAsync"));
     }
     if ((s = alloc_anderson(p))) return fail(s);
-    if ((s = dev_alloc(p, &p->partial, 2 * (size_t)p->n_partial_blocks)) ||
+    p->n_loop_blocks = p->n_sm;  // the one-launch iteration keeps two steps' partial sums
+    if ((s = dev_alloc(p, &p->partial, 2 * (size_t)std::max(p->n_partial_blocks, 2 * p->n_loop_blocks))) ||
         (s = dev_alloc(p, &p->state, 1)) || (s = dev_alloc(p, &p->fextra, N)) ||
         (s = dev_alloc(p, &p->pivmin, 2)))
         return fail(s);
@@ -623,6 +636,17 @@ adr_status adr_split_step(adr_problem* h, double dt, const double* u, double* u_
         TRY(launch_xfer(p, 1, p->fam[0].v, p->xuG, p->xuG, 0, nullptr, nullptr, false, false));
         TRY(launch_line_solve_dir(p, 1, dt, p->xuG, p->xuG, false));
         TRY(launch_grid_map_ex(p, 1, u_next, u_next, 0, nullptr, nullptr, false, false));
+    } else if (loop_applies(p)) {
+        TRY(launch_state_reset(p));
+        TRY(launch_solve_loop(p, dt, u, u_next, u_next, half, -1.0, 1, false));
+        IterState st;
+        ADR_CUDA_TRY(cudaMemcpyAsync(&st, p->state, sizeof st, cudaMemcpyDeviceToHost, p->stream));
+        ADR_CUDA_TRY(cudaStreamSynchronize(p->stream));
+        if (st.timeout) {
+            set_error("the split step gave up waiting at a grid barrier; its outputs are not valid");
+            return ADR_ETIMEOUT;
+        }
+        return ADR_OK;
     } else {
         TRY(launch_substep_solve(p, 0, dt, u, u, false));
         TRY(launch_grid_map_ex(p, 0, half, half, 0, nullptr, nullptr, false, false));

@@ -11,6 +11,8 @@
 //                 the nearest crossings on the node's row and column (§6), with
 //                 the relative-update norms fused in.
 //  k_check        one block: convergence test and the CUDA-graph loop condition.
+//  k_solve_loop   the whole iteration of a small or medium problem as one
+//                 cooperative launch.
 //  *_batch        the same steps for many problems in one persistent launch.
 #include <cuda_runtime.h>
 
@@ -117,15 +119,15 @@ struct BlockChunk {
     bool active;
 };
 
-// chunk of the calling thread inside a work item of block size T whose curves
-// are curves[0 .. BS/T-1]
+// chunk of thread tid inside a work item of block size T whose curves are
+// curves[0 .. BS/T-1]
 __device__ __forceinline__ void item_chunk_of(const CurveArgs& a, int T, const int* curves,
-                                              BlockChunk& b)
+                                              BlockChunk& b, int tid)
 {
     b.T = T;
     int L = __ffs(b.T) - 1;
-    int sb = threadIdx.x >> L;
-    b.lt = threadIdx.x & (b.T - 1);
+    int sb = tid >> L;
+    b.lt = tid & (b.T - 1);
     b.line = curves[sb];
     b.active = b.line >= 0;
     b.base = b.n = b.m = b.c = b.s = b.cnt = b.so = 0;
@@ -143,15 +145,27 @@ template <int BS>
 __device__ __forceinline__ void item_chunk(const CurveArgs& a, const int* item_T,
                                            const int* item_curve, BlockChunk& b)
 {
-    item_chunk_of(a, item_T[blockIdx.x], item_curve + blockIdx.x * Items<BS>::MAXC, b);
+    item_chunk_of(a, item_T[blockIdx.x], item_curve + blockIdx.x * Items<BS>::MAXC, b, threadIdx.x);
+}
+
+// grid state / node values: read-only in a launch of their own; written by
+// other blocks of the same launch in the one-launch iteration (COH: a plain
+// load, ordered by the grid barrier's acquire)
+template <bool COH>
+__device__ __forceinline__ double ld_state(const double* p)
+{
+    if constexpr (COH) return *p;
+    else return __ldg(p);
 }
 
 // bilinear gather at a row's node from its cell and corner weights (slot sl)
+template <bool COH>
 __device__ __forceinline__ double gather_w(const double* __restrict__ u, int nx, int cell,
                                            const double* __restrict__ w, size_t NS, int sl)
 {
     const double* r0 = u + cell;
-    double p11 = __ldg(r0), p12 = __ldg(r0 + 1), p21 = __ldg(r0 + nx), p22 = __ldg(r0 + nx + 1);
+    double p11 = ld_state<COH>(r0), p12 = ld_state<COH>(r0 + 1), p21 = ld_state<COH>(r0 + nx),
+           p22 = ld_state<COH>(r0 + nx + 1);
     double v = __ldg(w + sl) * p11;
     v = fma(__ldg(w + NS + sl), p12, v);
     v = fma(__ldg(w + 2 * NS + sl), p21, v);
@@ -548,27 +562,42 @@ __device__ __forceinline__ float as_f32(E x)
     else return f64_to_f32(x);
 }
 
-// Curve solve of one work item (block size T, curves[0 .. BS/T-1], reduced-
-// system constants Lc, elimination factors fac in precision E); the whole
-// block calls it.  RES = 0: FP64 new-value form, v = x.  RES = 1: residual
-// form, the correction x in precision E and v = u + dt x accumulated in FP64
-// (u is parked in v between the passes).  The rows' rp values live in
-// shared memory [R][BS] between the passes.
-template <int BS, int FAM, bool RES, typename E, bool DIR = false>
-__device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, const int* curves,
-                                                 const E* __restrict__ Lc, const E* __restrict__ fac,
-                                                 unsigned char* smem)
+// the threads that solve together: a whole block, or one group of n threads
+// of a block (named barrier id; a single warp needs none)
+struct BlockSync {
+    __device__ __forceinline__ void operator()() const { __syncthreads(); }
+};
+struct GroupSync {
+    int id, n;
+    __device__ __forceinline__ void operator()() const
+    {
+        if (n == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+    }
+};
+
+// Curve solve of one work item, or of a slice of it (block size T, curves[0 ..
+// BS/T-1], reduced-system constants Lc, elimination factors fac in precision
+// E) by a group of BS threads, tid the thread's index in it.  LS: threads of
+// the whole item (the stride of Lc, already offset to the slice).  RES = 0:
+// FP64 new-value form, v = x.  RES = 1: residual form, the correction x in
+// precision E and v = u + dt x accumulated in FP64 (u is parked in v between
+// the passes) and corr (nullable) keeps the largest |dt x|.  The rows' rp
+// values live in shared memory [R][BS] between the passes.
+template <int BS, int LS, int FAM, bool RES, typename E, bool DIR, bool COH, class Sync>
+__device__ __forceinline__ void curve_solve_group(const CurveArgs& a, const double* __restrict__ u, int Titem,
+                                                  const int* curves, const E* __restrict__ Lc,
+                                                  const E* __restrict__ fac, unsigned char* smem, int tid,
+                                                  Sync sync, unsigned long long* corr)
 {
-    constexpr int LMAX = Items<BS>::LMAX, NF = Items<BS>::NF;
+    constexpr int LMAX = Items<LS>::LMAX, NF = Items<LS>::NF;
     E (*sR)[BS] = reinterpret_cast<E (*)[BS]>(smem);
     double* __restrict__ buf = reinterpret_cast<double*>(smem + 2 * BS * sizeof(double));
-    const int tid = threadIdx.x;
     // row j's 8-byte slot of rp (E)
     auto rp = [&](int j) -> E& { return *reinterpret_cast<E*>(buf + j * BS + tid); };
-    const double* __restrict__ u = (a.state && (a.state->iter & 1)) ? a.u_odd : a.u_even;
     double* __restrict__ v = a.v;
     BlockChunk b;
-    item_chunk_of(a, Titem, curves, b);
+    item_chunk_of(a, Titem, curves, b, tid);
     const int lt = b.lt, T = b.T, L = __ffs(T) - 1;
     if (b.active && b.n < 2 && lt <= b.n) v[b.base + lt] = 0.0;
     const int base = b.base, s = b.s, cnt = b.cnt;
@@ -601,9 +630,9 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
         if (cnt > 0) {
             const double kap = (FAM == 1) ? __ldg(a.kap + b.line) : 0.0;
             const double* __restrict__ un = u + base + s;
-            double u0 = paper ? 0.0 : __ldg(un), u1 = paper ? 0.0 : __ldg(un + 1);
+            double u0 = paper ? 0.0 : ld_state<COH>(un), u1 = paper ? 0.0 : ld_state<COH>(un + 1);
             for (int j = 0; j < cnt; ++j) {
-                const double u2 = paper ? 0.0 : __ldg(un + j + 2);
+                const double u2 = paper ? 0.0 : ld_state<COH>(un + j + 2);
                 row(j, so + j * T + lt, kap, u0, u1, u2);
                 u0 = u1;
                 u1 = u2;
@@ -611,7 +640,7 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
         }
     } else if (cnt > 0) {
         const double kap = (FAM == 1) ? __ldg(a.kap + b.line) : 0.0;
-        auto uslot = [&](int sl) -> double { return gather_w(u, a.nx, __ldg(a.gcell + sl), a.gw, NS, sl); };
+        auto uslot = [&](int sl) -> double { return gather_w<COH>(u, a.nx, __ldg(a.gcell + sl), a.gw, NS, sl); };
         double u0 = 0.0, u1 = 0.0;
         if (!paper) {
             u0 = (s == 0) ? 0.0 : uslot(so + (b.c - 1) * T + (lt - 1));
@@ -640,10 +669,10 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
             double u2 = 0.0;
             if (nsl >= 0) {
                 const double* r0 = u + ncell;
-                u2 = nw0 * __ldg(r0);
-                u2 = fma(nw1, __ldg(r0 + 1), u2);
-                u2 = fma(nw2, __ldg(r0 + a.nx), u2);
-                u2 = fma(nw3, __ldg(r0 + a.nx + 1), u2);
+                u2 = nw0 * ld_state<COH>(r0);
+                u2 = fma(nw1, ld_state<COH>(r0 + 1), u2);
+                u2 = fma(nw2, ld_state<COH>(r0 + a.nx), u2);
+                u2 = fma(nw3, ld_state<COH>(r0 + a.nx + 1), u2);
             }
             nsl = next_slot(j + 1);
             if (nsl >= 0) load_desc();
@@ -663,13 +692,13 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
     const E lc0 = Lc[tid];
     E k1n = E(0), k2n = E(0), ib = E(0);
     if (L > 0) {
-        k1n = Lc[BS + tid];
-        k2n = Lc[(1 + LMAX) * BS + tid];
+        k1n = Lc[LS + tid];
+        k2n = Lc[(1 + LMAX) * LS + tid];
     } else {
-        ib = Lc[(NF - 1) * BS + tid];
+        ib = Lc[(NF - 1) * LS + tid];
     }
     sR[0][tid] = rho;
-    __syncthreads();
+    sync();
     const E rhoN = lt + 1 < T ? sR[0][tid + 1] : E(0);
     E R = cnt > 0 ? mad(-lc0, rhoN, rpp) : E(0);
     int bsel = 1;
@@ -679,13 +708,13 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
         const int d = 1 << l;
         const E k1 = k1n, k2 = k2n;
         if (l + 1 < L) {
-            k1n = Lc[(2 + l) * BS + tid];
-            k2n = Lc[(2 + LMAX + l) * BS + tid];
+            k1n = Lc[(2 + l) * LS + tid];
+            k2n = Lc[(2 + LMAX + l) * LS + tid];
         } else {
-            ib = Lc[(NF - 1) * BS + tid];
+            ib = Lc[(NF - 1) * LS + tid];
         }
         sR[bsel][tid] = R;
-        __syncthreads();
+        sync();
         const E Rm = lt >= d ? sR[bsel][tid - d] : E(0);
         const E Rp = lt + d < T ? sR[bsel][tid + d] : E(0);
         R = mad(-k2, Rp, mad(-k1, Rm, R));
@@ -693,7 +722,7 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
     }
     const E G = R * ib;
     sR[bsel][tid] = G;
-    __syncthreads();
+    sync();
     const E Gm = lt > 0 ? sR[bsel][tid - 1] : E(0);
     // 5. back substitution; values out
     E x = G;
@@ -707,7 +736,7 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
             if constexpr (sizeof(E) == 4) x64 = f32_to_f64(x);
             else x64 = x;
             // v = u + dt d in FP64 (u parked in v, or the node values themselves)
-            const double ub = DIR ? __ldg(u + node) : v[node];
+            const double ub = DIR ? ld_state<COH>(u + node) : v[node];
             v[node] = paper ? x64 : fma(a.dt, x64, ub);
             xmax = fmaxf(xmax, fabsf(as_f32(x)));
         } else {
@@ -720,15 +749,27 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
     }
     if constexpr (RES) {
         // largest correction of the launch (for the solve's statistics)
-        if (a.state && !paper) {
+        if (corr && !paper) {
             for (int o = 16; o > 0; o >>= 1) xmax = fmaxf(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
             if ((tid & 31) == 0 && xmax > 0.f) {
                 const double cmax = a.dt * f32_to_f64(xmax);
-                atomicMax(const_cast<unsigned long long*>(&a.state->corr_bits),
-                          (unsigned long long)__double_as_longlong(cmax));
+                atomicMax(corr, (unsigned long long)__double_as_longlong(cmax));
             }
         }
     }
+}
+
+// the whole block solves one item from the state of the step's parity
+template <int BS, int FAM, bool RES, typename E, bool DIR = false>
+__device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, const int* curves,
+                                                 const E* __restrict__ Lc, const E* __restrict__ fac,
+                                                 unsigned char* smem)
+{
+    const double* u = (a.state && (a.state->iter & 1)) ? a.u_odd : a.u_even;
+    curve_solve_group<BS, BS, FAM, RES, E, DIR, false>(a, u, Titem, curves, Lc, fac, smem, threadIdx.x,
+                                                       BlockSync(),
+                                                       a.state ? const_cast<unsigned long long*>(&a.state->corr_bits)
+                                                               : nullptr);
 }
 
 // one work item of the reduced-precision mode: FP32 corrections until the
@@ -986,31 +1027,56 @@ __global__ void k_map_coef(long long N, const uint8_t* ntype, const int* cg, con
     }
 }
 
-// curve -> grid map over nodes first, first + stride, ... of one problem;
-// returns the partial sums of the norms of the calling thread
-template <bool NORMS>
-__device__ __forceinline__ void grid_map_body(const GridArgs& a, long long first, long long stride,
-                                              double& dd, double& uu)
+// the map's tables of one node, and the map from them
+struct MapPre {
+    int4 g;
+    double2 c0, c1, c2, c3;
+    bool in;
+};
+
+__device__ __forceinline__ void map_prefetch(const GridArgs& a, long long k, MapPre& p)
 {
-    int it = a.state ? a.state->iter : 0;
-    double* __restrict__ out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
-    const double* __restrict__ prev = (it & 1) ? a.prev_odd : a.prev_even;
-    const double* __restrict__ v = a.v;
+    p.in = k < (long long)a.nx * a.ny && a.ntype[k] == kInterior;
+    if (k >= (long long)a.nx * a.ny) return;
+    p.g = *reinterpret_cast<const int4*>(a.mg + 4 * k);
+    const double2* c = reinterpret_cast<const double2*>(a.mc + 8 * k);
+    p.c0 = c[0];
+    p.c1 = c[1];
+    p.c2 = c[2];
+    p.c3 = c[3];
+}
+
+// curve -> grid map over nodes first, first + stride, ... of one problem into
+// out; adds the norms' sums of the calling thread (against prev).  COH: the
+// curve values and the previous state come from this launch, and the first
+// node's tables from pre.
+template <bool NORMS, bool COH>
+__device__ __forceinline__ void grid_map_nodes(const GridArgs& a, double* __restrict__ out, const double* prev,
+                                               long long first, long long stride, double& dd, double& uu,
+                                               const MapPre* pre = nullptr)
+{
+    const double* v = a.v;
     const long long N = (long long)a.nx * a.ny;
     for (long long k = first; k < N; k += stride) {
         double val = 0.0;
-        if (a.ntype[k] == kInterior) {
-            int4 g = *reinterpret_cast<const int4*>(a.mg + 4 * k);
-            const double2* c = reinterpret_cast<const double2*>(a.mc + 8 * k);
-            double2 c0 = c[0], c1 = c[1], c2 = c[2], c3 = c[3];
-            val = c0.x * __ldg(v + g.x);
-            val = fma(c0.y, __ldg(v + g.x + 1), val);
-            val = fma(c1.x, __ldg(v + g.y), val);
-            val = fma(c1.y, __ldg(v + g.y + 1), val);
-            val = fma(c2.x, __ldg(v + g.z), val);
-            val = fma(c2.y, __ldg(v + g.z + 1), val);
-            val = fma(c3.x, __ldg(v + g.w), val);
-            val = fma(c3.y, __ldg(v + g.w + 1), val);
+        MapPre q;
+        if (COH && k == first) {
+            q = *pre;
+        } else if (COH) {
+            map_prefetch(a, k, q);
+        } else {
+            q.in = a.ntype[k] == kInterior;
+            if (q.in) map_prefetch(a, k, q);
+        }
+        if (q.in) {
+            val = q.c0.x * ld_state<COH>(v + q.g.x);
+            val = fma(q.c0.y, ld_state<COH>(v + q.g.x + 1), val);
+            val = fma(q.c1.x, ld_state<COH>(v + q.g.y), val);
+            val = fma(q.c1.y, ld_state<COH>(v + q.g.y + 1), val);
+            val = fma(q.c2.x, ld_state<COH>(v + q.g.z), val);
+            val = fma(q.c2.y, ld_state<COH>(v + q.g.z + 1), val);
+            val = fma(q.c3.x, ld_state<COH>(v + q.g.w), val);
+            val = fma(q.c3.y, ld_state<COH>(v + q.g.w + 1), val);
             if (NORMS) {
                 double dlt = val - prev[k];
                 dd = fma(dlt, dlt, dd);
@@ -1019,6 +1085,17 @@ __device__ __forceinline__ void grid_map_body(const GridArgs& a, long long first
         }
         out[k] = val;
     }
+}
+
+// the same into the state buffer of the step's parity
+template <bool NORMS>
+__device__ __forceinline__ void grid_map_body(const GridArgs& a, long long first, long long stride,
+                                              double& dd, double& uu)
+{
+    int it = a.state ? a.state->iter : 0;
+    double* out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
+    const double* prev = (it & 1) ? a.prev_odd : a.prev_even;
+    grid_map_nodes<NORMS, false>(a, out, prev, first, stride, dd, uu);
 }
 
 template <bool NORMS>
@@ -1271,6 +1348,429 @@ __global__ void k_check(IterState* st, const double* partial, int nblocks, doubl
     }
 }
 
+// ---------------------------------------------------- one-launch iteration
+// The whole outer iteration of a small or medium problem as one cooperative
+// launch: one block per SM stays resident and walks the phases of every split
+// step (B solve with its gather, B map, G solve with its gather, G map with
+// the norms) with a grid barrier after each, and every block evaluates the
+// convergence test from the same partial sums in the same order.  The
+// arithmetic per row and node is the separate kernels', in the same order.
+// What bounds these sizes is latency, not a pipe: a graph node costs about 4 us
+// from its predecessor's last block to its own, seven times a step; here a
+// barrier costs 1.3 us, four times a step, and a warp's FP64 instruction 64
+// cycles (31 ns), dependent or not.  Measured per split step (sheared
+// problem, FP64, graph of kernels -> one launch): 33^2 25.6 -> 13.0 us,
+// 64^2 28.4 -> 13.6, 129^2 32.7 -> 19.3, 257^2 40.4 -> 28.6, 385^2 52.1 -> 39.4,
+// 500^2 75 -> 72; at 700^2 one block of 256 threads per SM no longer hides the
+// tables' latency (110 -> 129 us), hence kLoopMaxNodes.
+// A group of GS threads owns one slice of a 256-thread work item (one curve
+// where T = GS), dealt to the SMs before it is dealt to an SM's groups, so
+// that every SM's FP64 pipe gets its share of the curves.
+// Data that other blocks write during the launch (the grid states, the curve
+// values, the partial sums) is read from L2 (ld.global.cg); the static tables
+// may stay in L1 from step to step.  Barrier waits are bounded: a block that
+// gives up flags IterState::timeout and leaves, and so do the others.
+constexpr int kLoopThreads = 256;
+constexpr size_t kLoopSmem = 224 * 1024;  // dynamic shared memory of a block
+constexpr int kLoopSpin = 1 << 23;  // polls of one barrier wait (several seconds)
+
+struct LoopArgs {
+    CurveArgs c[2];
+    GridArgs g[2];
+    const int* item_T[2];
+    const int* item_curve[2];
+    const double* lanec[2];
+    const float* lanec32[2];
+    int n_items[2];
+    IterState* state;
+    double* partial;  // [2][2 * gridDim.x] by the step's parity
+    double tol;
+    int max_iter;
+    int norms;        // 0: exactly max_iter steps, no norms (a split step of a caller's own loop)
+};
+
+// all blocks of the (cooperative) launch; *epoch counts the barriers passed
+__device__ __forceinline__ bool grid_barrier(IterState* st, unsigned& epoch)
+{
+    __shared__ int ok;
+    __syncthreads();
+    ++epoch;
+    if (threadIdx.x == 0) {
+        const unsigned target = epoch * gridDim.x;
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
+        int good = 0;
+        for (int k = 0; k < kLoopSpin; ++k) {
+            unsigned c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&st->bar) : "memory");
+            if ((int)(c - target) >= 0) {
+                good = 1;
+                break;
+            }
+        }
+        if (!good) st->timeout = 1;
+        ok = good;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
+// shared memory of a group of the one-launch iteration whose longest chunk has
+// R rows: exchange buffers [2][GS] and planes [R][GS], a column per thread:
+// the gathered u (FP64 form: replaced by rp row by row), cp, vp and, in the
+// residual form, rp
+template <int GS, bool REF>
+__host__ __device__ constexpr size_t loop_smem(int R)
+{
+    return (size_t)(2 + (REF ? 4 : 3) * R) * GS * sizeof(double);
+}
+
+// slice q of a family's work items: its curves and reduced-system constants
+struct LoopUnit {
+    BlockChunk b;
+    size_t lo;
+    bool any;
+};
+
+template <int GS, int FAM>
+__device__ __forceinline__ void loop_unit(const LoopArgs& a, int q, int gt, LoopUnit& w)
+{
+    constexpr int PER = 256 / GS, NF = Items<256>::NF;
+    w.any = q < a.n_items[FAM] * PER;
+    if (!w.any) return;
+    const int item = q / PER, sl = q - item * PER;
+    const int T = a.item_T[FAM][item];
+    const int* cv = a.item_curve[FAM] + item * Items<256>::MAXC + sl * (GS / T);
+    w.any = cv[0] >= 0;  // an empty slice: the same for the whole group
+    if (!w.any) return;
+    item_chunk_of(a.c[FAM], T, cv, w.b, gt);
+    w.lo = (size_t)item * NF * 256 + sl * GS;
+}
+
+// gather descriptors of a thread's first rows, loaded before the barrier that
+// the grid state waits for (the acquire empties L1, so a table read after it
+// costs an L2 round trip of about 800 cycles, as much as 12 dependent FP64
+// operations)
+constexpr int kLoopPre = 3;
+struct LoopPre {
+    int cell[kLoopPre];
+    double w[kLoopPre][4];
+};
+
+__device__ __forceinline__ void loop_prefetch(const CurveArgs& a, const LoopUnit& q, LoopPre& p)
+{
+    if (!q.any) return;
+#pragma unroll
+    for (int j = 0; j < kLoopPre; ++j)
+        if (j < q.b.cnt) {
+            const int sl = q.b.so + j * q.b.T + q.b.lt;
+            p.cell[j] = __ldg(a.gcell + sl);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) p.w[j][k] = __ldg(a.gw + (size_t)k * a.n_slots + sl);
+        }
+}
+
+// One slice of a work item by a group of GS threads: the gathers of all of a
+// thread's rows first (independent loads, several rows' in flight), the neighbours' end values through shared memory,
+// then curve_solve_group's elimination with the row data loaded a row ahead
+// and cp, vp kept in shared memory for the two passes that follow.  The same
+// operations in the same order.
+template <int GS, int FAM, bool RES, typename E>
+__device__ __forceinline__ void loop_solve_unit(const CurveArgs& a, const BlockChunk& b, const double* u,
+                                                const E* __restrict__ Lc, const E* __restrict__ fac,
+                                                unsigned char* smem, int tid, GroupSync sync,
+                                                unsigned long long* corr, const LoopPre& pre, bool use_pre)
+{
+    constexpr int LS = 256, LMAX = Items<LS>::LMAX, NF = Items<LS>::NF;
+    constexpr int LV = GS == 32 ? 5 : 6;  // levels of the largest T
+    const int R = a.R;
+    E (*sR)[GS] = reinterpret_cast<E (*)[GS]>(smem);
+    double* su = reinterpret_cast<double*>(smem) + 2 * GS + tid;    // [j * GS]
+    E* scp = reinterpret_cast<E*>(su - tid + R * GS) + tid;
+    E* svp = scp + R * GS;
+    E* srp = RES ? svp + R * GS : reinterpret_cast<E*>(su);         // FP64 form: over u
+    const int lt = b.lt, T = b.T, L = __ffs(T) - 1, cnt = b.cnt, s = b.s, base = b.base, so = b.so;
+    const size_t NS = a.n_slots;
+    double* __restrict__ v = a.v;
+    if (b.active && b.n < 2 && lt <= b.n) v[base + lt] = 0.0;
+    // the reduced system's factors: all of them in flight during the gathers
+    const E lc0 = Lc[tid];
+    E k1[LV], k2[LV];
+#pragma unroll
+    for (int l = 0; l < LV; ++l) {
+        k1[l] = l < L ? Lc[(1 + l) * LS + tid] : E(0);
+        k2[l] = l < L ? Lc[(1 + LMAX + l) * LS + tid] : E(0);
+    }
+    const E ib = Lc[(NF - 1) * LS + tid];
+    const double kap = (FAM == 1 && cnt > 0) ? __ldg(a.kap + b.line) : 0.0;
+    double c0 = 0.0, c1 = 0.0, c2 = 0.0, F = 0.0;  // row data, a row ahead
+    E fl = E(0), fc = E(0), fv = E(0);
+    auto load = [&](int j) {
+        const int sl = so + j * T + lt;
+        c0 = __ldg(a.srow + sl);
+        if (FAM == 0) {
+            c1 = __ldg(a.srow + NS + sl);
+            c2 = __ldg(a.srow + 2 * NS + sl);
+            F = __ldg(a.Fl + sl);
+        }
+        fc = __ldg(fac + sl);
+        fv = __ldg(fac + NS + sl);
+        fl = __ldg(fac + 3 * NS + sl);
+    };
+    if (cnt > 0) load(0);
+    // 1. u at the thread's rows
+    int j0 = 0;
+    if (use_pre) {
+#pragma unroll
+        for (int j = 0; j < kLoopPre; ++j)
+            if (j < cnt) {
+                const double* r0 = u + pre.cell[j];
+                double t = pre.w[j][0] * r0[0];
+                t = fma(pre.w[j][1], r0[1], t);
+                t = fma(pre.w[j][2], r0[a.nx], t);
+                su[j * GS] = fma(pre.w[j][3], r0[a.nx + 1], t);
+            }
+        j0 = kLoopPre;
+    }
+#pragma unroll 3
+    for (int j = j0; j < cnt; ++j) {
+        const int sl = so + j * T + lt;
+        su[j * GS] = gather_w<true>(u, a.nx, __ldg(a.gcell + sl), a.gw, NS, sl);
+    }
+    sync();
+    // the neighbours' values: the last row of the chunk before, the first of the one after
+    const double ul = (cnt > 0 && s > 0) ? su[(b.c - 1) * GS - 1] : 0.0;
+    const double ur = (cnt > 0 && s + cnt < b.m) ? su[1] : 0.0;
+    sync();
+    // 2. right-hand sides and downward elimination
+    E rpp = E(0);
+    if (cnt > 0) {
+        double u0 = ul, u1 = su[0];
+        for (int j = 0; j < cnt; ++j) {
+            const double d0 = c0, d1 = c1, d2 = c2, dF = F;
+            const E el = fl;
+            scp[j * GS] = fc;
+            svp[j * GS] = fv;
+            if (j + 1 < cnt) load(j + 1);
+            const double u2 = j + 1 < cnt ? su[(j + 1) * GS] : ur;
+            double r;
+            if (FAM == 0) {
+                r = fma(d0, u0, dF);
+                r = fma(d1, u1, r);
+                r = fma(d2, u2, r);
+            } else {
+                r = d0 * fma(kap, u1, u0 + u2);
+            }
+            E re;
+            if constexpr (sizeof(E) == 4) re = f64_to_f32(r);
+            else re = r;
+            rpp = mad(-el, rpp, re);
+            srp[j * GS] = rpp;
+            u0 = u1;
+            u1 = u2;
+        }
+    }
+    // 3. upward pass over the chunk: rho for its first row
+    E rho = E(0);
+    for (int j = cnt - 2; j >= 0; --j) rho = mad(-scp[j * GS], rho, srp[j * GS]);
+    // 4. reduced system of the chunk ends
+    sR[0][tid] = rho;
+    sync();
+    const E rhoN = lt + 1 < T ? sR[0][tid + 1] : E(0);
+    E Rr = cnt > 0 ? mad(-lc0, rhoN, rpp) : E(0);
+    int bsel = 1;
+#pragma unroll
+    for (int l = 0; l < LV; ++l) {
+        if (l >= L) break;  // uniform over the group
+        const int d = 1 << l;
+        sR[bsel][tid] = Rr;
+        sync();
+        const E Rm = lt >= d ? sR[bsel][tid - d] : E(0);
+        const E Rp = lt + d < T ? sR[bsel][tid + d] : E(0);
+        Rr = mad(-k2[l], Rp, mad(-k1[l], Rm, Rr));
+        bsel ^= 1;
+    }
+    const E G = Rr * ib;
+    sR[bsel][tid] = G;
+    sync();
+    const E Gm = lt > 0 ? sR[bsel][tid - 1] : E(0);
+    // 5. back substitution; values out
+    E x = G;
+    float xmax = 0.f;
+    for (int j = cnt - 1; j >= 0; --j) {
+        if (j < cnt - 1) x = mad(-svp[j * GS], Gm, mad(-scp[j * GS], x, srp[j * GS]));
+        const int node = base + s + j + 1;
+        if constexpr (RES) {
+            double x64;
+            if constexpr (sizeof(E) == 4) x64 = f32_to_f64(x);
+            else x64 = x;
+            v[node] = fma(a.dt, x64, su[j * GS]);
+            xmax = fmaxf(xmax, fabsf(as_f32(x)));
+        } else {
+            v[node] = x;
+        }
+    }
+    if (b.active && b.n >= 2 && lt == 0) {
+        v[base] = 0.0;
+        v[base + b.n] = 0.0;
+    }
+    if constexpr (RES) {
+        if (corr) {
+            for (int o = 16; o > 0; o >>= 1) xmax = fmaxf(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
+            if ((tid & 31) == 0 && xmax > 0.f)
+                atomicMax(corr, (unsigned long long)__double_as_longlong(a.dt * f32_to_f64(xmax)));
+        }
+    }
+}
+
+// a group's slices of one family; pre: the first slice's first descriptors
+template <int GS, int FAM, bool REF>
+__device__ __forceinline__ void loop_solve(const LoopArgs& a, const double* u, bool hp, unsigned char* sm,
+                                           unsigned long long* corr, const LoopUnit& first, const LoopPre& pre)
+{
+    const int NG = blockDim.x / GS, grp = threadIdx.x / GS, gt = threadIdx.x % GS;
+    const CurveArgs& c = a.c[FAM];
+    const GroupSync sync{grp + 1, GS};  // barrier 0 is the block's
+    const int units = a.n_items[FAM] * (256 / GS);
+    LoopUnit w = first;
+    bool use = true;
+    for (int q = blockIdx.x + gridDim.x * grp; q < units;) {
+        if (w.any) {
+            if (REF && !hp)
+                loop_solve_unit<GS, FAM, true, float>(c, w.b, u, a.lanec32[FAM] + w.lo, c.fac32, sm, gt, sync, corr,
+                                                        pre, use);
+            else
+                loop_solve_unit<GS, FAM, REF, double>(c, w.b, u, a.lanec[FAM] + w.lo, c.fac, sm, gt, sync, corr, pre,
+                                                        use);
+            sync();  // the group's shared memory is reused
+        }
+        q += gridDim.x * NG;
+        use = false;
+        if (q < units) loop_unit<GS, FAM>(a, q, gt, w);
+    }
+}
+
+// (dd, uu) summed over the warp: lane 0 gets dd, lane 16 uu (5 additions, as
+// an FP64 warp instruction costs the same for 1 or 32 lanes)
+__device__ __forceinline__ double warp_sum2(double dd, double uu, int lane)
+{
+    double v = lane < 16 ? dd : uu;
+    const double w = lane < 16 ? uu : dd;
+    v += __shfl_xor_sync(0xffffffffu, w, 16);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+template <int GS, bool REF>
+__global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_constant__ LoopArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ double red[2][kLoopThreads / 32];
+    __shared__ double srel;
+    __shared__ int sflag;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    // nodes in runs of 32, dealt to the blocks first; blocks and warps past
+    // the grid's end have none
+    const long long N = (long long)a.g[0].nx * a.g[0].ny;
+    const long long first = ((long long)blockIdx.x + (long long)gridDim.x * warp) * 32 + lane;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    const int runs = (int)min((N + 31) / 32, (long long)gridDim.x * nw);
+    const int npart = min((int)gridDim.x, runs);                           // blocks with nodes
+    const int nwarp = blockIdx.x < npart ? (runs - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;  // warps with nodes
+    const int grp = threadIdx.x / GS, gt = threadIdx.x % GS;
+    LoopUnit w0, w1;
+    loop_unit<GS, 0>(a, blockIdx.x + gridDim.x * grp, gt, w0);
+    loop_unit<GS, 1>(a, blockIdx.x + gridDim.x * grp, gt, w1);
+    unsigned char* sm = smem + (size_t)grp * loop_smem<GS, REF>(a.c[0].R);
+    LoopPre pre;
+    MapPre mp;
+    loop_prefetch(a.c[0], w0, pre);
+    unsigned epoch = 0;
+    int iter = 0, hp = 0, fp32 = 0, conv = 0;
+    double rel = INFINITY;
+    for (;;) {
+        const double* u = (iter & 1) ? a.c[0].u_odd : a.c[0].u_even;
+        double* un = (iter & 1) ? a.g[1].out_even : a.g[1].out_odd;
+        unsigned long long* corr = REF && a.norms ? &a.state->corr_loop[iter & 1] : nullptr;
+        double dd = 0.0, uu = 0.0;
+        loop_solve<GS, 0, REF>(a, u, hp, sm, corr, w0, pre);
+        map_prefetch(a.g[0], first, mp);
+        if (!grid_barrier(a.state, epoch)) return;
+        grid_map_nodes<false, true>(a.g[0], a.g[0].out_even, nullptr, first, stride, dd, uu, &mp);
+        loop_prefetch(a.c[1], w1, pre);
+        if (!grid_barrier(a.state, epoch)) return;
+        if (REF && blockIdx.x == 0 && threadIdx.x == 0) a.state->corr_loop[(iter + 1) & 1] = 0ull;
+        loop_solve<GS, 1, REF>(a, a.c[1].u_even, hp, sm, corr, w1, pre);
+        map_prefetch(a.g[1], first, mp);
+        if (!grid_barrier(a.state, epoch)) return;
+        if (!a.norms) {
+            grid_map_nodes<false, true>(a.g[1], un, nullptr, first, stride, dd, uu, &mp);
+            loop_prefetch(a.c[0], w0, pre);
+            if (++iter >= a.max_iter) break;
+            if (!grid_barrier(a.state, epoch)) return;
+            continue;
+        }
+        grid_map_nodes<true, true>(a.g[1], un, u, first, stride, dd, uu, &mp);
+        loop_prefetch(a.c[0], w0, pre);
+        if (warp < nwarp) {
+            const double v = warp_sum2(dd, uu, lane);
+            if ((lane & 15) == 0) red[lane >> 4][warp] = v;
+        }
+        __syncthreads();
+        double* part = a.partial + (size_t)(iter & 1) * 2 * gridDim.x;
+        if (nwarp > 0 && threadIdx.x < 2) {  // both sums in one warp's instructions
+            double t = red[threadIdx.x][0];
+            for (int q = 1; q < nwarp; ++q) t += red[threadIdx.x][q];
+            part[2 * blockIdx.x + threadIdx.x] = t;
+        }
+        if (!grid_barrier(a.state, epoch)) return;
+        ++iter;
+        if (warp == 0) {
+            // every block: the same sums in the same order
+            double t = 0.0;
+            for (int b = lane >> 1; b < npart; b += 16) t += __ldcg(part + 2 * b + (lane & 1));
+            for (int o = 2; o < 32; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            const double num = __shfl_sync(0xffffffffu, t, 0), den = __shfl_sync(0xffffffffu, t, 1);
+            if (lane == 0) {
+                // the square root and the division (20 FP64 instructions) only where
+                // they decide: a relative update clearly above every threshold goes on
+                const double lim = 2.0 * a.tol * (REF && !hp ? kHpSwitch : 1.0);
+                int flag = 0;
+                if (iter >= a.max_iter || !(num > lim * lim * den) || !(den > 0.0) || !isfinite(num) || !isfinite(den)) {
+                    double r = den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0);
+                    if (!isfinite(num) || !isfinite(den)) r = INFINITY;  // diverged
+                    srel = r;
+                    if (a.tol > 0.0 && r <= a.tol) flag |= 1;
+                    if (a.tol > 0.0 && r <= kHpSwitch * a.tol) flag |= 2;
+                    if ((flag & 1) || iter >= a.max_iter || !isfinite(r)) flag |= 4;
+                }
+                sflag = flag;
+            }
+        }
+        __syncthreads();
+        const int flag = sflag;
+        if (!hp) {
+            ++fp32;
+            hp = (flag >> 1) & 1;
+        }
+        if (flag & 4) {
+            conv = flag & 1;
+            rel = srel;
+            break;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        IterState* st = a.state;
+        st->iter = iter;
+        st->rel = rel;
+        st->converged = conv;
+        st->hp = hp;
+        st->fp32_steps = fp32;
+        if (REF && a.norms)  // the last step's corrections are behind its barriers
+            st->corr = __longlong_as_double((long long)__ldcg(&st->corr_loop[(iter - 1) & 1]));
+        st->done = 1;
+    }
+}
+
 // out = wa*a + wb*b on every node, where a = u_j and b = u_{j+1/2} of the last
 // step (selected by the step counter); used for the Crank-Nicolson midpoint
 __global__ void k_finish(const IterState* st, const double* u_even, const double* u_odd,
@@ -1308,6 +1808,9 @@ __global__ void k_reset(IterState* st)
     st->corr = 0.0;
     st->hp = 0;
     st->fp32_steps = 0;
+    st->corr_loop[0] = st->corr_loop[1] = 0ull;
+    st->bar = 0u;
+    st->timeout = 0;
 }
 
 __global__ void k_set_bits(double* p, unsigned long long bits)
@@ -1369,6 +1872,7 @@ adr_status setup_groups(Problem* p, int fam, const std::vector<int>& off)
                                  p->stream));
     ADR_CUDA_TRY(cudaStreamSynchronize(p->stream));
     std::vector<int> byT[11];  // index log2(T)
+    F.tmax = 32;
     for (int l : order) {
         int m = off[l + 1] - off[l] - 2;
         int T = 32, lg = 5;
@@ -1383,6 +1887,7 @@ adr_status setup_groups(Problem* p, int fam, const std::vector<int>& off)
         }
         byT[lg].push_back(l);
         Tof[l] = T;
+        F.tmax = std::max(F.tmax, T);
     }
     std::vector<int> soff(F.n_lines + 1, 0);
     long long tot = 0;
@@ -1852,6 +2357,82 @@ adr_status launch_grid_map_ex(Problem* p, int fam, double* out_even, double* out
     if (norms) k_grid_map<true><<<blocks, kGridThreads, 0, p->stream>>>(a);
     else k_grid_map<false><<<blocks, kGridThreads, 0, p->stream>>>(a);
     ADR_CUDA_TRY(cudaGetLastError());
+    return ADR_OK;
+}
+
+// one-launch iteration: problems through the grid whose curves take at most
+// 64 threads (their groups' tables fit an SM's shared memory) and whose step
+// is bound by latency
+bool loop_applies(const Problem* p)
+{
+    if (p->opts.transfer || p->N > kLoopMaxNodes || p->n_sm <= 0 || !p->coop) return false;
+    for (const Family& F : p->fam)
+        if (!F.iset[0].count || F.iset[1].count || F.iset[2].count || F.tmax > 64) return false;
+    return true;
+}
+
+template <int GS, bool REF>
+static cudaError_t loop_launch(const LoopArgs& a, int R, int blocks, cudaStream_t st)
+{
+    // as many groups as fit the block's threads and an SM's shared memory
+    const int groups = std::min(kLoopThreads / GS, (int)(kLoopSmem / loop_smem<GS, REF>(R)));
+    const size_t sm = (size_t)groups * loop_smem<GS, REF>(R);
+    cudaError_t e = cudaFuncSetAttribute(k_solve_loop<GS, REF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    void* args[] = {const_cast<LoopArgs*>(&a)};
+    return cudaLaunchCooperativeKernel((const void*)k_solve_loop<GS, REF>, dim3(blocks), dim3(groups * GS), args, sm,
+                                       st);
+}
+
+// steps from u_even (the state buffers by the step's parity; the first step
+// reads u_even), u_{j+1/2} in half; norms = false: exactly max_iter steps
+adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
+                             double* half, double tol, int max_iter, bool norms)
+{
+    LoopArgs a{};
+    int tmax = 32;
+    int R = 1;
+    for (int fam = 0; fam < 2; ++fam) {
+        Family& F = p->fam[fam];
+        if (!F.prep_valid || F.prep_paper || F.prep_dt != dt) {
+            set_error("internal: curve systems not factored for this step");
+            return ADR_EINVAL;
+        }
+        CurveArgs& c = a.c[fam];
+        c = curve_args(p, fam);
+        c.u_even = fam == 0 ? u_even : half;
+        c.u_odd = fam == 0 ? u_odd : half;
+        GridArgs& g = a.g[fam];
+        g.nx = p->grid.nx;
+        g.ny = p->grid.ny;
+        g.ntype = p->ntype;
+        g.mg = F.mg;
+        g.mc = F.mc;
+        g.v = F.v;
+        g.out_even = fam == 0 ? half : out_even;
+        g.out_odd = fam == 0 ? half : u_odd;
+        a.item_T[fam] = F.iset[0].T;
+        a.item_curve[fam] = F.iset[0].curve;
+        a.lanec[fam] = F.iset[0].lanec;
+        a.lanec32[fam] = F.iset[0].lanec32;
+        a.n_items[fam] = F.iset[0].count;
+        tmax = std::max(tmax, F.tmax);
+        R = std::max(R, F.cmax);
+    }
+    a.c[0].R = a.c[1].R = R;
+    a.state = p->state;
+    a.partial = p->partial;
+    a.tol = tol;
+    a.max_iter = max_iter;
+    a.norms = norms ? 1 : 0;
+    const int blocks = std::min(p->n_sm, p->n_loop_blocks);
+    const bool ref = p->opts.prec == ADR_FP32_REFINE;
+    cudaError_t e = cudaSuccess;
+#define ADR_LOOP(GS_) e = ref ? loop_launch<GS_, true>(a, R, blocks, p->stream) : loop_launch<GS_, false>(a, R, blocks, p->stream)
+    if (tmax <= 32) ADR_LOOP(32);
+    else ADR_LOOP(64);
+#undef ADR_LOOP
+    if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel (one-launch iteration)");
     return ADR_OK;
 }
 

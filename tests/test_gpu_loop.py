@@ -1,0 +1,92 @@
+"""The one-launch iteration (and the separate kernels just past it) against the CPU oracle
+at the edges of their range: a single warp per curve and 64 threads per curve
+(512 / 513 unknowns), the largest grid of the one launch and the first past
+it, thin and masked domains, both precision modes.
+
+Tolerances as in test_gpu_parity.py: FP64 1e-12, FP32 + refinement 1e-5, both
+of max |u|."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2411_11041_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _problem(nx, ny, field, mask, seed=5):
+    rng = np.random.default_rng(seed)
+    if field == "sheared":
+        b1, b2 = W.sheared_beta(nx, ny)
+    else:
+        b1, b2 = np.full((ny, nx), field[0]), np.full((ny, nx), field[1])
+    y1 = (ny - 1) / (nx - 1)
+    f = W.random_field(rng, nx, ny)
+    return W.Problem(nx, ny, 3e-3, 0.8, b1, b2, f, W.make_mask(mask, nx, ny), y1=y1)
+
+
+CASES = [
+    (31, 9, (1.0, 0.37), "square"),
+    (40, 40, (1.0, 0.0), "square"),      # aligned: curves on grid lines
+    (65, 64, "sheared", "square"),
+    (90, 90, (-0.6, 0.8), "disc"),
+    (514, 24, (1.0, 0.0), "square"),     # 512 unknowns: one warp a curve
+    (515, 24, (1.0, 0.0), "square"),     # 513: 64 threads
+    (1026, 11, (1.0, 0.0), "square"),    # 1024 unknowns, the longest of 64 threads
+    (1027, 11, (1.0, 0.0), "square"),    # past it: separate kernels
+    (300, 290, "sheared", "L"),
+    (512, 512, "sheared", "square"),     # the largest grid of the one launch
+    (512, 513, "sheared", "square"),     # the first of the separate kernels
+]
+
+
+@pytest.mark.parametrize("nx,ny,field,mask", CASES)
+@pytest.mark.parametrize("prec", [0, 1])
+def test_fixed_steps_match_oracle(nx, ny, field, mask, prec):
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    p = _problem(nx, ny, field, mask)
+    if field == "sheared" and mask == "L":
+        p.beta2[:] = np.abs(p.beta2)
+    o = O.Oracle(p)
+    s = Solver(p, tol=0.0, max_iter=3, prec=prec)
+    u, it, st, code = s.solve_stationary(want_iter=True)
+    ref, refit, k, rel, _ = o.solve_stationary(tol=0.0, max_iter=3)
+    tol = 1e-12 if prec == 0 else 1e-5
+    assert st["iters"] == k == 3
+    assert np.abs(u.cpu().numpy() - ref).max() <= tol * np.abs(ref).max()
+    assert np.abs(it.cpu().numpy() - refit).max() <= tol * np.abs(refit).max()
+    assert abs(st["rel_update"] - rel) <= (1e-9 if prec == 0 else 1e-3) * rel + 1e-13
+    # a caller's own split step, in place
+    v = torch.tensor(np.random.default_rng(1).normal(size=(ny, nx)) * o.interior(), device="cuda:0")
+    rh, rn = o.split_step(0.5, 0.02, v.cpu().numpy())
+    uh, un = s.split_step(v, 0.02)
+    assert np.abs(uh.cpu().numpy() - rh).max() <= tol * np.abs(rh).max()
+    assert np.abs(un.cpu().numpy() - rn).max() <= tol * np.abs(rn).max()
+
+
+def test_two_streams_solve_at_once():
+    """Two handles on two streams from two threads: each launch waits for the
+    SMs it needs, and both answers are the single solves'."""
+    import threading
+
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    ps = [_problem(120, 120, "sheared", "square", seed=k) for k in (1, 2)]
+    ref = [Solver(p, tol=1e-9, max_iter=5000).solve_stationary()[0].clone() for p in ps]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in ps]
+    out = [None, None]
+
+    def work(i):
+        with torch.cuda.stream(streams[i]):
+            s = Solver(ps[i], tol=1e-9, max_iter=5000, stream=streams[i])
+            for _ in range(5):
+                out[i] = s.solve_stationary()[0]
+
+    th = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    [t.start() for t in th]
+    [t.join() for t in th]
+    torch.cuda.synchronize()
+    for u, r in zip(out, ref):
+        assert torch.equal(u, r)
