@@ -851,6 +851,35 @@ __global__ void __launch_bounds__(BS, BS == 256 ? 4 : (BS == 512 ? 2 : 1)) k_cur
     else curve_solve_body<BS, FAM, false, double, true>(a, item_T[blockIdx.x], cv, lanec + lo, a.fac, smem);
 }
 
+// the same with a block of GS threads per slice of a 256-thread item (curves of
+// T <= GS).  The bound is the SM's FP64 pipe, so an SM with two items where
+// others have one doubles the launch: at 513^2 180 items meet 152 SMs, at
+// 1024^2 429.  Slices of one curve each even that out (725 blocks of 64
+// threads, 858 of 128).  Measured whole items -> slices, a solve pass: 513^2
+// 16.8 -> 14.5 us, 257^2 12.5 -> 10.5, 1024^2 29.0 -> 28.1; curves of T = 256
+// (2048^2) have nothing to slice.
+template <int GS, int FAM, bool REF>
+__global__ void __launch_bounds__(GS, 1024 / GS) k_curve_solve_slice(CurveArgs a, const int* item_T,
+                                                                     const int* item_curve, const double* lanec,
+                                                                     const float* lanec32)
+{
+    if (a.state && a.state->done) return;
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int PER = 256 / GS, NF = Items<256>::NF;
+    const int item = blockIdx.x / PER, sl = blockIdx.x - item * PER, T = item_T[item];
+    const int* cv = item_curve + item * Items<256>::MAXC + sl * (GS / T);
+    if (cv[0] < 0) return;  // an empty slice
+    const size_t lo = (size_t)item * NF * 256 + sl * GS;
+    const double* u = (a.state && (a.state->iter & 1)) ? a.u_odd : a.u_even;
+    unsigned long long* corr = a.state ? const_cast<unsigned long long*>(&a.state->corr_bits) : nullptr;
+    if (REF && !(a.state && a.state->hp))
+        curve_solve_group<GS, 256, FAM, true, float, true, false>(a, u, T, cv, lanec32 + lo, a.fac32, smem,
+                                                                  threadIdx.x, BlockSync(), corr);
+    else
+        curve_solve_group<GS, 256, FAM, REF, double, true, false>(a, u, T, cv, lanec + lo, a.fac, smem, threadIdx.x,
+                                                                  BlockSync(), corr);
+}
+
 // DIR: the table's u pointers are the families' node values (the batched
 // gather pass before the solve fills them)
 template <int BS, int FAM, bool REF, bool DIR = false>
@@ -2197,6 +2226,13 @@ adr_status launch_line_solve(Problem* p, int fam, double dt, const double* u_eve
     return ADR_OK;
 }
 
+// threads of a block of the sliced solve; 256: whole items
+static int solve_slice(const Family& F)
+{
+    if (F.tmax > 128 || !F.iset[0].count) return 256;
+    return F.tmax;
+}
+
 // the curve solve of the direct transfer: u_even / u_odd are node arrays of
 // the family (selected by the step's parity when use_state)
 adr_status launch_line_solve_dir(Problem* p, int fam, double dt, const double* u_even,
@@ -2228,7 +2264,25 @@ adr_status launch_line_solve_dir(Problem* p, int fam, double dt, const double* u
     }
     ADR_SOLVE_DIR(1024, F.iset[2])
     ADR_SOLVE_DIR(512, F.iset[1])
-    ADR_SOLVE_DIR(256, F.iset[0])
+    const ItemSet& I0 = F.iset[0];
+    const int gs = solve_slice(F);
+#define ADR_SLICE(GS_)                                                                             \
+    {                                                                                              \
+        const size_t sm = solve_smem<GS_>(R);                                                      \
+        const int nb = I0.count * (256 / GS_);                                                     \
+        if (ref) {                                                                                 \
+            if (fam == 0) k_curve_solve_slice<GS_, 0, true><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32); \
+            else k_curve_solve_slice<GS_, 1, true><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32);         \
+        } else {                                                                                   \
+            if (fam == 0) k_curve_solve_slice<GS_, 0, false><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32); \
+            else k_curve_solve_slice<GS_, 1, false><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32);         \
+        }                                                                                          \
+    }
+    if (gs == 32) ADR_SLICE(32)
+    else if (gs == 64) ADR_SLICE(64)
+    else if (gs == 128) ADR_SLICE(128)
+    else ADR_SOLVE_DIR(256, F.iset[0])
+#undef ADR_SLICE
 #undef ADR_SOLVE_DIR
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
