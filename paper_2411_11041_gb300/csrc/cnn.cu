@@ -67,12 +67,6 @@ __device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const void* p)
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(smem_u32(p)));
 }
-__device__ __forceinline__ void ldsm_x4_t(unsigned (&r)[4], const void* p)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(p)));
-}
 __device__ __forceinline__ void ldsm_x2_t(unsigned (&r)[2], const void* p)
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
@@ -97,6 +91,8 @@ struct ConvArgs {
     const float* bias;  // [Cout] or null
     bf16* y;            // [B][H][W][Cout] or null
     float* y32;         // [B][H][W][Cout] FP32 output or null
+    const bf16* mask;   // [B][H][W][Cout] or null: the output is 0 where the mask is not positive
+                        // (the ReLU's backward pass, tensor-core kernels)
     int relu;
     long long spin;     // tensor-core kernels: bound of their mbarrier waits in polls
                         // (0: the default bound)
@@ -269,6 +265,19 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     return false;
 }
 
+// 16 BF16 values set to 0 where the mask's are not positive (sign set, zero or NaN)
+__device__ __forceinline__ void relu_mask16(uint32_t (&v)[8], const bf16* mask)
+{
+    const uint4 a = *reinterpret_cast<const uint4*>(mask), b = *reinterpret_cast<const uint4*>(mask + 8);
+    const uint32_t m[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    auto pos = [](uint32_t h) { return h - 1u < 0x7f80u; };  // 1 .. 0x7f80: positive, infinity included
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        if (!pos(m[j] & 0xffffu)) v[j] &= 0xffff0000u;
+        if (!pos(m[j] >> 16)) v[j] &= 0x0000ffffu;
+    }
+}
+
 template <int N>
 __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
 {
@@ -403,6 +412,7 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
                     __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
                     packed[j] = *reinterpret_cast<uint32_t*>(&h);
                 }
+                if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
                 uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
                 dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                 dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
@@ -583,6 +593,7 @@ __global__ void __launch_bounds__(TmaConv<N>::THREADS) k_conv_tma(const __grid_c
                 __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
                 packed[j] = *reinterpret_cast<uint32_t*>(&h);
             }
+            if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
             uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
             dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
             dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
@@ -594,108 +605,295 @@ __global__ void __launch_bounds__(TmaConv<N>::THREADS) k_conv_tma(const __grid_c
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(MT * N));
 }
 
+// ------------------------------------------------ weight gradient (tcgen05)
+// dW[tap][ci][co] = sum over pixels p of x[p + tap][ci] dy[p][co].  The
+// reduction runs over pixels, so both operands are MN-major as they lie in
+// memory (NHWC: a pixel's channels are contiguous): one TMA load brings 64
+// channels of 64 pixels (a 4 x 16 window, shifted by the tap's offset for x;
+// the image border and the channels past Cin come as zero fill) as a
+// 64-row x 128-byte plane in the 128-byte swizzle, which is the MN-major
+// operand layout as it stands: 64 channels along a row, 8 pixels per swizzle
+// group (groups 1024 bytes apart: the stride offset), the next 64 channels a
+// plane further (the leading offset).
+// Two planes make one M = 128 operand: the two channel halves of a tap where
+// Cin = 128, two taps where Cin <= 64.  A CTA holds the accumulators of G such
+// pairs in tensor memory and walks its share of the pixel windows, each dy tile
+// serving all G pairs; partial sums per CTA are reduced in a fixed order
+// afterwards, so the gradient is deterministic.  What bounds it is the planes'
+// traffic from L2: (2 G + N / 64) 8 KB per 4 G MMAs of 128 x N x 16.
+// Measured for a 64-problem batch: 128 -> 128 channels 672 us on mma.sync, 103
+// us here (0.75 PFLOP/s); 64 -> 64 channels 201 -> 60 us.
 struct WgradArgs {
     int B, H, W, Cin, Cout, dil;
-    const bf16* x;   // layer input [B][H][W][Cin]
-    const bf16* dy;  // gradient at the pre-activation [B][H][W][Cout]
-    float* part;     // [splits][9 Cin][Cout]
-    long long pchunk;
+    float* part;       // [splits][9 Cin][Cout]
+    int G;             // operand pairs of a CTA (blockIdx.y: its first pair / G)
+    int npair;         // pairs in all: 9 (Cin = 128) or 5 (Cin <= 64, the tenth plane unused)
+    int tiles;         // pixel windows in all
+    int per;           // windows of a split (blockIdx.x)
+    int stages;
+    long long spin;
 };
 
-// dW[k][co] = sum_p X_patch[p][k] dY[p][co]: M = 9 Cin, N = Cout, reduction
-// over pixels (split over blockIdx.z; partial sums reduced afterwards)
-template <int BN>
-__global__ void __launch_bounds__(128) k_conv_wgrad(WgradArgs a)
+constexpr int kWgPlane = 64 * 128;    // bytes of a plane: 64 pixels x 64 channels
+constexpr int kWgThreads = 128;
+constexpr int kWgMaxStages = 8;
+constexpr int kWgSmem = 216 * 1024;   // stages, without the alignment slack
+
+// MN-major shared-memory descriptor, 128-byte swizzle: 64-element blocks `lbo`
+// bytes apart, 8-pixel groups 1024 bytes apart
+__device__ __forceinline__ uint64_t umma_sdesc_mn(uint32_t addr, uint32_t lbo)
 {
-    constexpr int BM = 64, BP = 32, AS = BM + 8, BSTR = BN + 8;
-    constexpr int WN = BN >= 64 ? 2 : 1, WM = 4 / WN, TM = BM / WM, TN = BN / WN;
-    constexpr int MI = TM / 16, NI = TN / 8;
-    __shared__ __align__(16) bf16 As[2][BP][AS];
-    __shared__ __align__(16) bf16 Bs[2][BP][BSTR];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int wm = warp / WN, wn = warp % WN;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int HW = a.H * a.W;
-    const long long M = (long long)a.B * HW;
-    const int K = 9 * a.Cin;
-    const long long pbeg = (long long)blockIdx.z * a.pchunk;
-    const long long pend = pbeg + a.pchunk < M ? pbeg + a.pchunk : M;
-    float acc[MI][NI][4];
+    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
+           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+template <int N>
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ CUtensorMap tx,
+                                                            const __grid_constant__ CUtensorMap ty, WgradArgs a,
+                                                            int tmem_cols, int* err)
+{
+    constexpr int NB = N / 64;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    __shared__ uint64_t full[kWgMaxStages], empty[kWgMaxStages];
+    __shared__ uint32_t tmem_base;
+    __shared__ int consumed;
+    const int tid = threadIdx.x, warp = tid >> 5, S = a.stages;
+    const int g0 = blockIdx.y * a.G, ng = min(a.G, a.npair - g0);
+    const int t0 = blockIdx.x * a.per, t1 = min(t0 + a.per, a.tiles), nk = max(t1 - t0, 0);
+    const int stage = (2 * a.G + NB) * kWgPlane, bytes = (2 * ng + NB) * kWgPlane;
+    const int tiles_x = a.W / 16, per_img = tiles_x * (a.H / 4);
+    const bool wide = a.Cin > 64;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         smem_u32(&tmem_base)),
+                     "r"(tmem_cols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[s])));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+    const uint32_t tmem = tmem_base;
+    bool ok = true;
+    int issued = 0;
+    if (tid == 0) {
+        const uint64_t px = reinterpret_cast<uint64_t>(&tx), py = reinterpret_cast<uint64_t>(&ty);
+        for (int k = 0; k < nk; ++k) {
+            const int s = k % S, t = t0 + k;
+            if (k >= S && !(ok = mbar_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin))) break;
+            const int b = t / per_img, r = t - b * per_img;
+            const int y0 = (r / tiles_x) * 4, x0 = (r - (r / tiles_x) * tiles_x) * 16;
+            const uint32_t sa = sbase + s * stage, bar = smem_u32(&full[s]);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
+                         : "memory");
+            for (int q = 0; q < 2 * ng + NB; ++q) {
+                int c, dx = 0, dy = 0;
+                const bool isx = q < 2 * ng;
+                if (isx) {
+                    const int p = 2 * g0 + q;  // plane: (tap, half) or tap
+                    const int tap = min(wide ? p >> 1 : p, 8);
+                    c = wide ? (p & 1) * 64 : 0;
+                    dy = (tap / 3 - 1) * a.dil;
+                    dx = (tap % 3 - 1) * a.dil;
+                } else {
+                    c = (q - 2 * ng) * 64;
+                }
+                const uint32_t dst = sa + (isx ? q : 2 * a.G + q - 2 * ng) * kWgPlane;
+                asm volatile(
+                    "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+                    "%4, %5}], [%6];\n" ::"r"(dst),
+                    "l"(isx ? px : py), "r"(c), "r"(x0 + dx), "r"(y0 + dy), "r"(b), "r"(bar)
+                    : "memory");
+            }
+            issued = k + 1;
+        }
+    } else if (tid == 32) {
+        // FP32 accumulator, BF16 operands, both MN-major
+        const uint32_t idesc = umma_idesc(128, N) | (1u << 15) | (1u << 16);
+        int k = 0;
+        for (; k < nk; ++k) {
+            const int s = k % S;
+            if (!(ok = mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const uint32_t sa = sbase + s * stage, sb = sa + 2 * a.G * kWgPlane;
+            for (int g = 0; g < ng; ++g) {
 #pragma unroll
-    for (int i = 0; i < MI; ++i)
-#pragma unroll
-        for (int j = 0; j < NI; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
-    auto load = [&](int st, long long p0) {
-        for (int v = tid; v < BP * (BM / 8); v += 128) {
-            int row = v / (BM / 8), kg = v % (BM / 8);
-            long long p = p0 + row;
-            int k = m0 + kg * 8;
-            const bf16* src = a.x;
-            bool ok = false;
-            if (p < pend && k < K) {
-                int tap = k / a.Cin, ci = k - tap * a.Cin;
-                int b = (int)(p / HW), rem = (int)(p - (long long)b * HW);
-                int r = rem / a.W, c = rem - r * a.W;
-                int rr = r + (tap / 3 - 1) * a.dil, cc = c + (tap % 3 - 1) * a.dil;
-                if (rr >= 0 && rr < a.H && cc >= 0 && cc < a.W) {
-                    src = a.x + (((long long)b * a.H + rr) * a.W + cc) * a.Cin + ci;
-                    ok = true;
+                for (int ks = 0; ks < 4; ++ks) {  // 16 pixels each
+                    const uint64_t ad = umma_sdesc_mn(sa + 2 * g * kWgPlane + ks * 2048, kWgPlane);
+                    const uint64_t bd = umma_sdesc_mn(sb + ks * 2048, kWgPlane);
+                    const uint32_t acc = (k > 0 || ks > 0) ? 1u : 0u;
+                    asm volatile(
+                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+                            tmem + (uint32_t)(g * N)),
+                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
                 }
             }
-            cp_async16(&As[st][row][kg * 8], src, ok);
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                smem_u32(&empty[s])));
         }
-        for (int v = tid; v < BP * (BN / 8); v += 128) {
-            int row = v / (BN / 8), ng = v % (BN / 8);
-            long long p = p0 + row;
-            int n = n0 + ng * 8;
-            bool ok = p < pend && n < a.Cout;
-            cp_async16(&Bs[st][row][ng * 8], ok ? a.dy + p * a.Cout + n : a.dy, ok);
-        }
-        cp_async_commit();
-    };
-    const long long np = pend > pbeg ? (pend - pbeg + BP - 1) / BP : 0;
-    if (np > 0) load(0, pbeg);
-    for (long long pt = 0; pt < np; ++pt) {
-        const int st = (int)(pt & 1);
-        if (pt + 1 < np) {
-            load(st ^ 1, pbeg + (pt + 1) * BP);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BP; kk += 16) {
-            unsigned af[MI][4], bfr[NI][2];
-#pragma unroll
-            for (int i = 0; i < MI; ++i)
-                ldsm_x4_t(af[i], &As[st][kk + (lane & 7) + ((lane >> 4) << 3)]
-                                    [wm * TM + i * 16 + ((lane >> 3) & 1) * 8]);
-#pragma unroll
-            for (int j = 0; j < NI; ++j) ldsm_x2_t(bfr[j], &Bs[st][kk + (lane & 15)][wn * TN + j * 8]);
-#pragma unroll
-            for (int i = 0; i < MI; ++i)
-#pragma unroll
-                for (int j = 0; j < NI; ++j) mma_bf16(acc[i][j], af[i], bfr[j]);
-        }
-        __syncthreads();
+        consumed = k;
     }
-    const int g = lane >> 2, t = lane & 3;
-    float* part = a.part + (size_t)blockIdx.z * K * a.Cout;
+    const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    if (!all_ok && tid == 0) {
+        // a wait gave up: let the loads this CTA issued and no MMA consumed land
+        for (int k = consumed; k < issued; ++k) mbar_wait(smem_u32(&full[k % S]), (k / S) & 1, err);
+    }
+    ok = all_ok;
+    const int nc = consumed;
+    if (nc >= 1) {
+        const uint32_t bar = smem_u32(&empty[(nc - 1) % S]), par = ((nc - 1) / S) & 1;
+        bool w = ok && mbar_wait(bar, par, err, a.spin);
+        if (!w) mbar_wait(bar, par, err);
+        ok = __syncthreads_and((ok && w) ? 1 : 0) != 0;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+    if (ok) {
+        // accumulator row m of pair g: channel m of the tap (Cin = 128), or
+        // channel m % 64 of tap 2 g + m / 64
+        const int m = tid;
+        const uint32_t lane = (uint32_t)(warp * 32) << 16;
+        for (int g = 0; g < ng; ++g) {
+            const int p = 2 * (g0 + g) + (m >> 6), tap = wide ? p >> 1 : p, ci = wide ? m : m & 63;
+            const bool out = tap < 9 && ci < a.Cin;
+            float* dst = a.part + ((size_t)blockIdx.x * 9 * a.Cin + (size_t)tap * a.Cin + ci) * N;
 #pragma unroll
-    for (int i = 0; i < MI; ++i)
+            for (int c0 = 0; c0 < N; c0 += 16) {
+                uint32_t v[16];
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+                      "=r"(v[15])
+                    : "r"(tmem + lane + (uint32_t)(g * N + c0)));
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if (out) {
+                    uint4* d4 = reinterpret_cast<uint4*>(dst + c0);
 #pragma unroll
-        for (int j = 0; j < NI; ++j) {
-            int n = n0 + wn * TN + j * 8 + 2 * t;
-            if (n >= a.Cout) continue;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                int k = m0 + wm * TM + i * 16 + g + h * 8;
-                if (k >= K) continue;
-                part[(size_t)k * a.Cout + n] = acc[i][j][2 * h];
-                part[(size_t)k * a.Cout + n + 1] = acc[i][j][2 * h + 1];
+                    for (int j = 0; j < 4; ++j)
+                        d4[j] = nk > 0 ? make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3])
+                                       : make_uint4(0u, 0u, 0u, 0u);
+                }
             }
         }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(tmem_cols));
+}
+
+// -------------------------------------------- the last layer's backward pass
+// Only channel 0 of the output enters the loss, so the output gradient is one
+// value per pixel (dy0) and both gradients of the 64 -> 8 layer are sums over
+// 9 taps of a scalar times 64 channels: bound by reading and writing the 64
+// channels once, not by arithmetic, and no tensor core is needed (161 us for
+// the weight gradient on mma.sync and 49 us for the data gradient as a tcgen05
+// convolution with 8 input channels, before the ReLU pass; 39 and 48 us here
+// with the ReLU mask included, 64 problems).
+constexpr int kLastBlocks = 608;
+
+// dx[p][ci] = sum_tap dy0[p + shift] W[8 - tap][ci][0] where act > 0, else 0; a
+// thread takes 8 channels of a pixel
+__global__ void __launch_bounds__(256) k_last_dgrad(const bf16* __restrict__ dy0, const bf16* __restrict__ w,
+                                                    const bf16* __restrict__ act, long long M, int H, int W,
+                                                    bf16* __restrict__ dx)
+{
+    __shared__ float sw[9][64];
+    for (int i = threadIdx.x; i < 576; i += 256) sw[8 - i / 64][i & 63] = __bfloat162float(w[(size_t)i * kCout]);
+    __syncthreads();
+    const int cg = (threadIdx.x & 7) * 8;
+    for (long long p = (blockIdx.x * 256LL + threadIdx.x) >> 3; p < M; p += gridDim.x * 32LL) {
+        const int rem = (int)(p % (H * W)), r = rem / W, c = rem - r * W;
+        float acc[8] = {};
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int dr = tap / 3 - 1, dc = tap % 3 - 1;
+            const bool in = r + dr >= 0 && r + dr < H && c + dc >= 0 && c + dc < W;
+            const float d = in ? __bfloat162float(dy0[p + dr * W + dc]) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] = fmaf(d, sw[tap][cg + j], acc[j]);
+        }
+        const uint4 av = *reinterpret_cast<const uint4*>(act + p * 64 + cg);
+        const bf16* ab = reinterpret_cast<const bf16*>(&av);
+        uint4 ov;
+        bf16* ob = reinterpret_cast<bf16*>(&ov);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            ob[j] = __bfloat162float(ab[j]) > 0.f ? __float2bfloat16(acc[j]) : __float2bfloat16(0.f);
+        *reinterpret_cast<uint4*>(dx + p * 64 + cg) = ov;
+    }
+}
+
+// block partials of dW[tap][ci][0] = sum_q x[q][ci] dy0[q - shift] (577 per
+// block: the last is the sum of dy0, the bias gradient); a block takes a run of
+// pixels, a thread 8 channels of every 32nd pixel
+__global__ void __launch_bounds__(256) k_last_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dy0,
+                                                    long long M, int H, int W, float* __restrict__ part)
+{
+    const int cgi = threadIdx.x & 7, cg = cgi * 8, pl = threadIdx.x >> 3;
+    const long long chunk = ((M + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
+    const long long p0 = blockIdx.x * chunk, p1 = p0 + chunk < M ? p0 + chunk : M;
+    float acc[9][8] = {};
+    float bs = 0.f;
+    for (long long p = p0 + pl; p < p1; p += 32) {
+        const int rem = (int)(p % (H * W)), r = rem / W, c = rem - r * W;
+        const uint4 xv = *reinterpret_cast<const uint4*>(x + p * 64 + cg);
+        const bf16* xb = reinterpret_cast<const bf16*>(&xv);
+        float xf[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) xf[j] = __bfloat162float(xb[j]);
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+            const int dr = tap / 3 - 1, dc = tap % 3 - 1;
+            const bool in = r - dr >= 0 && r - dr < H && c - dc >= 0 && c - dc < W;
+            const float d = in ? __bfloat162float(dy0[p - dr * W - dc]) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[tap][j] = fmaf(d, xf[j], acc[tap][j]);
+            if (tap == 4) bs += d;
+        }
+    }
+    // over the warp's 4 pixels, then over the 8 warps
+    __shared__ float red[8][577];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float v = acc[tap][j];
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            if (lane < 8) red[warp][tap * 64 + cg + j] = v;
+        }
+    bs += __shfl_xor_sync(0xffffffffu, bs, 8);
+    bs += __shfl_xor_sync(0xffffffffu, bs, 16);
+    if (lane == 0) red[warp][576] = bs;
+    __syncthreads();
+    for (int i = threadIdx.x; i < 577; i += 256) {
+        float v = 0.f;
+        for (int q = 0; q < 8; ++q) v += red[q][i];
+        part[(size_t)blockIdx.x * 577 + i] = v;
+    }
+}
+
+// the block partials summed into the layer's gradient (channel 0; the other
+// channels' gradients are 0): one warp per entry, a fixed order
+__global__ void k_last_sum(const float* __restrict__ part, int blocks, float* __restrict__ gw, float* __restrict__ gb)
+{
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (i >= 577) return;
+    float v = 0.f;
+    for (int b = lane; b < blocks; b += 32) v += part[(size_t)b * 577 + i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    float* dst = i < 576 ? gw + (size_t)i * kCout : gb;
+    if (lane < kCout) dst[lane] = lane == 0 ? v : 0.f;
 }
 
 // grad[i] = sum over splits of part[s][i]  (fixed order: deterministic)
@@ -708,41 +906,59 @@ __global__ void k_sum_splits(const float* part, int splits, long long n, float* 
     grad[i] = s;
 }
 
-// bias gradient: per channel sum over pixels (one block per channel)
-__global__ void k_bias_grad(const bf16* dy, long long M, int C, float* grad)
+// bias gradient: per channel sum over pixels.  Every block sums a run of
+// pixels, a thread 8 channels (16 bytes) of every (256 C / 8)th pixel, so that
+// a warp reads whole rows; block partials in a fixed order.  Bound by reading
+// dy once; one block per channel with a stride of C between its reads took 176
+// us for 64 problems x 64 channels.
+constexpr int kBiasBlocks = 304;
+template <int C>
+__global__ void __launch_bounds__(256) k_bias_part(const bf16* __restrict__ dy, long long M, float* __restrict__ part)
 {
-    int c = blockIdx.x;
-    float s = 0.f;
-    for (long long p = threadIdx.x; p < M; p += blockDim.x) s += __bfloat162float(dy[p * C + c]);
-    __shared__ float sh[256];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
+    constexpr int TC = C / 8, PL = 256 / TC;  // threads across the channels, pixels per pass
+    const int cg = (threadIdx.x % TC) * 8, pl = threadIdx.x / TC;
+    const long long chunk = (M + gridDim.x - 1) / gridDim.x;
+    const long long p0 = blockIdx.x * chunk, p1 = p0 + chunk < M ? p0 + chunk : M;
+    float acc[8] = {};
+#pragma unroll 4
+    for (long long p = p0 + pl; p < p1; p += PL) {
+        const uint4 v = *reinterpret_cast<const uint4*>(dy + p * C + cg);
+        const bf16* b = reinterpret_cast<const bf16*>(&v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(b[j]);
     }
-    if (threadIdx.x == 0) grad[c] = sh[0];
+    __shared__ float red[PL][C];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) red[pl][cg + j] = acc[j];
+    __syncthreads();
+    for (int c = threadIdx.x; c < C; c += 256) {
+        float s = 0.f;
+        for (int q = 0; q < PL; ++q) s += red[q][c];
+        part[(size_t)blockIdx.x * C + c] = s;
+    }
 }
 
-// dYpre = dY where the layer's ReLU output is positive, else 0
-__global__ void k_relu_bwd(const bf16* dy, const bf16* y, long long n, bf16* out)
+__global__ void k_bias_sum(const float* __restrict__ part, int blocks, int C, float* __restrict__ grad)
 {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    out[i] = __bfloat162float(y[i]) > 0.f ? dy[i] : __float2bfloat16(0.f);
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (c >= C) return;
+    float v = 0.f;
+    for (int b = lane; b < blocks; b += 32) v += part[(size_t)b * C + c];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) grad[c] = v;
 }
 
-// loss = 1/2 mean over the M cells of (y[p][0] - t[p])^2, dY[p][0] = (y - t) / M,
-// other channels 0; per-block partial sums of the loss (FP64)
-__global__ void k_loss(const float* y32, int C, const float* t, long long M, bf16* dy, double* part)
+// loss = 1/2 mean over the M cells of (y[p][0] - t[p])^2, dy0[p] = (y - t) / M
+// (the gradient of the other channels is 0); per-block partial sums of the
+// loss (FP64)
+__global__ void k_loss(const float* y32, int C, const float* t, long long M, bf16* dy0, double* part)
 {
     long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     double e2 = 0.0;
     if (p < M) {
         float e = y32[p * C] - t[p];
         e2 = 0.5 * (double)e * (double)e;
-        dy[p * C] = __float2bfloat16(e / (float)M);
-        for (int c = 1; c < C; ++c) dy[p * C + c] = __float2bfloat16(0.f);
+        dy0[p] = __float2bfloat16(e / (float)M);
     }
     __shared__ double sh[256];
     sh[threadIdx.x] = e2;
@@ -754,11 +970,19 @@ __global__ void k_loss(const float* y32, int C, const float* t, long long M, bf1
     if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+// one block of 256 threads (one thread took 63 us for 1024 partials)
 __global__ void k_sum_loss(const double* part, int n, long long count, double* loss)
 {
+    __shared__ double sh[256];
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    *loss = s / (double)count;
+    for (int i = threadIdx.x; i < n; i += 256) s += part[i];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = sh[0] / (double)count;
 }
 
 struct LayerTab {
@@ -926,7 +1150,9 @@ struct adr_cnn {
     long long spin = 0;  // bound of those waits (adr_cnn_set_wait_limit; 0: default)
     bf16* act[kLayers] = {};  // post-activation outputs of layers 0..6 (bf16)
     float* y32 = nullptr;     // last layer output (fp32) [M][8]
-    bf16 *dA = nullptr, *dB = nullptr, *dpre = nullptr;
+    bf16 *dA = nullptr, *dB = nullptr, *dy0 = nullptr;
+    float* spart = nullptr;   // block partials of the bias and last-layer gradients
+    int n_sm = 0;
     float* part = nullptr;
     long long part_size = 0;
     double* lpart = nullptr;
@@ -1065,62 +1291,91 @@ adr_status cnn_forward(adr_cnn* c, int batch, const bf16* x)
     return ADR_OK;
 }
 
+// tensor map of an activation [B][H][W][C] with a box of 64 channels x 16 x 4
+// pixels, 128-byte swizzle
+bool wgrad_map(CUtensorMap* m, const bf16* x, int B, int H, int W, int C)
+{
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
+    if (!enc) return false;
+    cuuint64_t d[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+    cuuint64_t st[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
+    cuuint32_t box[4] = {64, 16, 4, 1}, e[4] = {1, 1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(x), d, st, box, e,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// weight and bias gradients of a layer of 64 or 128 output channels from its
+// input and its pre-activation gradient
+adr_status layer_grad(adr_cnn* c, int batch, int l, const bf16* xin, const bf16* dy)
+{
+    cudaStream_t st = c->stream;
+    const int cin = kCh[l], cout = kCh[l + 1];
+    const long long M = (long long)batch * c->hw * c->hw;
+    CUtensorMap tx, ty;
+    if (!wgrad_map(&tx, xin, batch, c->hw, c->hw, cin) || !wgrad_map(&ty, dy, batch, c->hw, c->hw, cout)) {
+        adr::set_error("the driver refused a tensor map of the weight gradient");
+        return ADR_ECUDA;
+    }
+    WgradArgs w{};
+    w.B = batch;
+    w.H = w.W = c->hw;
+    w.Cin = cin;
+    w.Cout = cout;
+    w.dil = kDil[l];
+    w.part = c->part;
+    w.spin = c->spin;
+    w.npair = cin > 64 ? 9 : 5;
+    w.G = cout == 128 ? 3 : 5;  // accumulators: G x cout of 512 columns of tensor memory
+    const int groups = (w.npair + w.G - 1) / w.G;
+    const int stage = (2 * w.G + cout / 64) * kWgPlane;
+    w.stages = std::min(kWgMaxStages, kWgSmem / stage);
+    w.tiles = (int)(M / 64);
+    int splits = std::max(1, std::min(c->n_sm / groups, w.tiles));
+    splits = (int)std::min<long long>(splits, c->part_size / (9LL * cin * cout));
+    w.per = (w.tiles + splits - 1) / splits;
+    splits = (w.tiles + w.per - 1) / w.per;
+    const int cols = w.G * cout <= 256 ? 256 : 512, smem = w.stages * stage + 1024;
+    const dim3 grid((unsigned)splits, (unsigned)groups);
+    if (cout == 128) k_wgrad_tc<128><<<grid, kWgThreads, smem, st>>>(tx, ty, w, cols, c->err);
+    else k_wgrad_tc<64><<<grid, kWgThreads, smem, st>>>(tx, ty, w, cols, c->err);
+    const long long nw = 9LL * cin * cout;
+    k_sum_splits<<<(int)((nw + 255) / 256), 256, 0, st>>>(c->part, splits, nw, c->grad + c->T.woff[l]);
+    const int nb = (int)std::min<long long>(kBiasBlocks, (M + 63) / 64);
+    if (cout == 128) k_bias_part<128><<<nb, 256, 0, st>>>(dy, M, c->spart);
+    else k_bias_part<64><<<nb, 256, 0, st>>>(dy, M, c->spart);
+    k_bias_sum<<<(cout * 32 + 255) / 256, 256, 0, st>>>(c->spart, nb, cout, c->grad + c->T.boff[l]);
+    return ADR_OK;
+}
+
 adr_status cnn_backward(adr_cnn* c, int batch, const bf16* x, const float* t)
 {
     cudaStream_t st = c->stream;
     const long long M = (long long)batch * c->hw * c->hw;
-    int nb = (int)((M + 255) / 256);
+    const int nb = (int)((M + 255) / 256), last = kLayers - 1;
+    k_loss<<<nb, 256, 0, st>>>(c->y32, kCout, t, M, c->dy0, c->lpart);
+    k_sum_loss<<<1, 256, 0, st>>>(c->lpart, nb, M, c->loss);
+    // the last layer: channel 0 alone
+    const int lb = (int)std::min<long long>(kLastBlocks, (M + 31) / 32);
+    k_last_wgrad<<<lb, 256, 0, st>>>(c->act[last - 1], c->dy0, M, c->hw, c->hw, c->spart);
+    k_last_sum<<<(577 * 32 + 255) / 256, 256, 0, st>>>(c->spart, lb, c->grad + c->T.woff[last],
+                                                      c->grad + c->T.boff[last]);
     bf16* dy = c->dA;
-    k_loss<<<nb, 256, 0, st>>>(c->y32, kCout, t, M, dy, c->lpart);
-    k_sum_loss<<<1, 1, 0, st>>>(c->lpart, nb, M, c->loss);
-    for (int l = kLayers - 1; l >= 0; --l) {
-        const int cin = kCh[l], cout = kCh[l + 1];
-        const bf16* dyp = dy;
-        if (l < kLayers - 1) {
-            k_relu_bwd<<<(int)((M * cout + 255) / 256), 256, 0, st>>>(dy, c->act[l], M * cout, c->dpre);
-            dyp = c->dpre;
-        }
-        const bf16* xin = l == 0 ? x : c->act[l - 1];
-        // weight gradient, split over pixels
-        WgradArgs w{};
-        w.B = batch;
-        w.H = w.W = c->hw;
-        w.Cin = cin;
-        w.Cout = cout;
-        w.dil = kDil[l];
-        w.x = xin;
-        w.dy = dyp;
-        w.part = c->part;
-        long long K = 9LL * cin;
-        int splits = (int)std::min<long long>(64, (M + 1023) / 1024);
-        if (splits < 1) splits = 1;
-        while ((long long)splits * K * cout > c->part_size) splits--;
-        w.pchunk = ((M + splits - 1) / splits + 31) / 32 * 32;
-        splits = (int)((M + w.pchunk - 1) / w.pchunk);
-        dim3 grid((unsigned)((K + 63) / 64), 1, (unsigned)splits);
-        if (cout >= 64) {
-            grid.y = (cout + 63) / 64;
-            k_conv_wgrad<64><<<grid, 128, 0, st>>>(w);
-        } else if (cout % 16 == 0) {
-            grid.y = cout / 16;
-            k_conv_wgrad<16><<<grid, 128, 0, st>>>(w);
-        } else {
-            grid.y = (cout + 7) / 8;
-            k_conv_wgrad<8><<<grid, 128, 0, st>>>(w);
-        }
-        long long nw = K * cout;
-        k_sum_splits<<<(int)((nw + 255) / 256), 256, 0, st>>>(c->part, splits, nw, c->grad + c->T.woff[l]);
-        k_bias_grad<<<cout, 256, 0, st>>>(dyp, M, cout, c->grad + c->T.boff[l]);
+    k_last_dgrad<<<lb, 256, 0, st>>>(c->dy0, c->wb + c->T.woff[last], c->act[last - 1], M, c->hw, c->hw, dy);
+    for (int l = last - 1; l >= 0; --l) {
+        TRY_S(layer_grad(c, batch, l, l == 0 ? x : c->act[l - 1], dy));
         if (l > 0) {
-            // data gradient: correlation with the flipped, transposed weights
+            // data gradient: correlation with the flipped, transposed weights,
+            // masked by the ReLU of the layer below
             ConvArgs a{};
             a.B = batch;
             a.H = a.W = c->hw;
-            a.Cin = cout;
-            a.Cout = cin;
+            a.Cin = kCh[l + 1];
+            a.Cout = kCh[l];
             a.dil = kDil[l];
-            a.x = dyp;
+            a.x = dy;
             a.w = c->wt + c->T.woff[l];
+            a.mask = c->act[l - 1];
             a.spin = c->spin;
             a.y = dy == c->dA ? c->dB : c->dA;
             launch_conv(st, a, c->wtk + c->T.woff[l], c->err);
@@ -1224,6 +1479,11 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
         c->T.cout[l] = kCh[l + 1];
     }
     const long long M = (long long)max_batch * c->hw * c->hw;
+    {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
+    }
     adr_status s = ADR_OK;
     auto fail = [&](adr_status st) {
         adr_cnn_destroy(c);
@@ -1235,7 +1495,8 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
         (s = cnn_alloc(c, &c->wk, c->P)) || (s = cnn_alloc(c, &c->wtk, c->P)) ||
         (s = cnn_alloc(c, &c->err, 1)) ||
         (s = cnn_alloc(c, &c->y32, M * kCout)) || (s = cnn_alloc(c, &c->dA, M * 128)) ||
-        (s = cnn_alloc(c, &c->dB, M * 128)) || (s = cnn_alloc(c, &c->dpre, M * 128)) ||
+        (s = cnn_alloc(c, &c->dB, M * 128)) || (s = cnn_alloc(c, &c->dy0, M)) ||
+        (s = cnn_alloc(c, &c->spart, (size_t)kLastBlocks * 577)) ||
         (s = cnn_alloc(c, &c->lpart, (M + 255) / 256 + 1)) || (s = cnn_alloc(c, &c->loss, 1)))
         return fail(s);
     for (int l = 0; l < kLayers - 1; ++l)
@@ -1248,6 +1509,8 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
                                       tc_smem_bytes<64>()));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       tc_smem_bytes<128>()));
+    ADR_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem + 1024));
+    ADR_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem + 1024));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tma<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       TmaConv<64>::SMEM));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tma<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -282,3 +282,30 @@ def test_bounded_wait_timeout_is_reported_and_the_handle_recovers(torch_cuda):
     ref = CNN.forward(pb, xh[0])
     assert _rel(y[0], ref) <= 2e-2
     net.loss_grad(x, t)  # no error left behind
+
+
+@pytest.mark.parametrize("batch", [2, 4, 64])
+def test_gradient_of_a_batch_is_the_mean_of_its_samples(torch_cuda, batch):
+    """The weight gradient's pixel splits, from one window per split to many:
+    1 / batch is a power of two, so every stored value of the single-sample
+    passes scales exactly and only the FP32 summation order differs: about
+    sqrt(262144) 2^-24 = 3e-5 of the terms' norm, times 30 for the terms'
+    cancellation in the sums."""
+    torch = torch_cuda
+    from paper_2411_11041_gb300 import Network
+    net = Network(batch, W.cnn_init_params(7, last_scale=1.0))
+    x, t, _, _ = _rand_inputs(batch, 3, torch)
+    x[:, :3] *= 3.0  # unlike borders
+    mean = torch.zeros(net.grad.shape, dtype=torch.float64, device="cuda:0")
+    losses = []
+    for b in range(batch):
+        loss, g = net.loss_grad(x[b:b + 1].contiguous(), t[b:b + 1].contiguous())
+        mean += g.double() / batch
+        losses.append(loss)
+    loss, g = net.loss_grad(x, t)
+    assert abs(loss - np.mean(losses)) <= 1e-12 * loss
+    assert torch.equal(g, net.loss_grad(x, t)[1])  # deterministic
+    for l in range(CNN.LAYERS):
+        for lo, hi in ((CNN.offset(l), CNN.offset(l, True)), (CNN.offset(l, True), CNN.offset(l + 1))):
+            a, r = g[lo:hi].double(), mean[lo:hi]
+            assert (a - r).norm() <= 1e-3 * r.norm(), (l, lo)
