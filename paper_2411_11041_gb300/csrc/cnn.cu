@@ -49,183 +49,45 @@ __device__ __forceinline__ unsigned smem_u32(const void* p)
     return (unsigned)__cvta_generic_to_shared(p);
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool ok)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem_u32(dst)), "l"(src),
-                 "r"(ok ? 16 : 0));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
-}
-
-__device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const void* p)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldsm_x2_t(unsigned (&r)[2], const void* p)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
-                 : "=r"(r[0]), "=r"(r[1])
-                 : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], const unsigned (&b)[2])
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-        "{%8,%9}, {%0,%1,%2,%3};\n"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 // ------------------------------------------------------ convolution kernels
 
+// All convolutions run on the 5th-generation tensor cores as implicit GEMMs
+// with M = pixels, N = Cout and K = 9 Cin: tcgen05.mma (kind::f16, BF16
+// operands, FP32 accumulators in tensor memory), operands staged by TMA.
+// Every mbarrier wait is bounded; when a wait gives up the kernel sets *err,
+// lets the loads and MMAs it issued finish, skips its output and frees its
+// tensor memory.
 struct ConvArgs {
-    int B, H, W, Cin, Cout, dil;
-    const bf16* x;      // [B][H][W][Cin]
-    const bf16* w;      // [9 Cin][Cout]
+    int B, H, W, dil;
+    int cblocks;        // 64-channel blocks of the input
+    int kc;             // channels per tap of the K-major weights (64 cblocks)
     const float* bias;  // [Cout] or null
-    bf16* y;            // [B][H][W][Cout] or null
-    float* y32;         // [B][H][W][Cout] FP32 output or null
     const bf16* mask;   // [B][H][W][Cout] or null: the output is 0 where the mask is not positive
-                        // (the ReLU's backward pass, tensor-core kernels)
+                        // (the ReLU's backward pass)
+    bf16* y;            // [B][H][W][Cout] (64 or 128 channels)
+    float* y32;         // [B][H][W][8] FP32 (the last layer)
     int relu;
-    long long spin;     // tensor-core kernels: bound of their mbarrier waits in polls
-                        // (0: the default bound)
+    int stages, tiles;
+    long long spin;     // bound of the mbarrier waits in polls (0: the default bound)
 };
-
-// implicit GEMM: M = pixels, N = Cout, K = 9 Cin (tap-major); a block computes
-// 128 pixels x BN channels with 8 warps; double-buffered cp.async tiles.
-template <int BN>
-__global__ void __launch_bounds__(256) k_conv_fwd(ConvArgs a)
-{
-    constexpr int BM = 128, BK = 32, AS = BK + 8, BSTR = BN + 8;
-    constexpr int WN = BN >= 64 ? 2 : 1, WM = 8 / WN, TM = BM / WM, TN = BN / WN;
-    constexpr int MI = TM / 16, NI = TN / 8;
-    __shared__ __align__(16) bf16 As[2][BM][AS];
-    __shared__ __align__(16) bf16 Bs[2][BK][BSTR];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int wm = warp / WN, wn = warp % WN;
-    const long long m0 = (long long)blockIdx.x * BM;
-    const int n0 = blockIdx.y * BN;
-    const int HW = a.H * a.W;
-    const long long M = (long long)a.B * HW;
-    const int K = 9 * a.Cin;
-    float acc[MI][NI][4];
-#pragma unroll
-    for (int i = 0; i < MI; ++i)
-#pragma unroll
-        for (int j = 0; j < NI; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
-
-    auto load = [&](int st, int k0) {
-        for (int v = tid; v < BM * (BK / 8); v += 256) {
-            int row = v / (BK / 8), kg = v % (BK / 8);
-            long long p = m0 + row;
-            int k = k0 + kg * 8;
-            const bf16* src = a.x;
-            bool ok = false;
-            if (p < M && k < K) {
-                int tap = k / a.Cin, ci = k - tap * a.Cin;
-                int b = (int)(p / HW), rem = (int)(p - (long long)b * HW);
-                int r = rem / a.W, c = rem - r * a.W;
-                int rr = r + (tap / 3 - 1) * a.dil, cc = c + (tap % 3 - 1) * a.dil;
-                if (rr >= 0 && rr < a.H && cc >= 0 && cc < a.W) {
-                    src = a.x + (((long long)b * a.H + rr) * a.W + cc) * a.Cin + ci;
-                    ok = true;
-                }
-            }
-            cp_async16(&As[st][row][kg * 8], src, ok);
-        }
-        for (int v = tid; v < BK * (BN / 8); v += 256) {
-            int row = v / (BN / 8), ng = v % (BN / 8);
-            int k = k0 + row, n = n0 + ng * 8;
-            bool ok = k < K && n < a.Cout;
-            cp_async16(&Bs[st][row][ng * 8], ok ? a.w + (long long)k * a.Cout + n : a.w, ok);
-        }
-        cp_async_commit();
-    };
-    const int nk = (K + BK - 1) / BK;
-    load(0, 0);
-    for (int kt = 0; kt < nk; ++kt) {
-        const int st = kt & 1;
-        if (kt + 1 < nk) {
-            load(st ^ 1, (kt + 1) * BK);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < BK; kk += 16) {
-            unsigned af[MI][4], bfr[NI][2];
-#pragma unroll
-            for (int i = 0; i < MI; ++i)
-                ldsm_x4(af[i], &As[st][wm * TM + i * 16 + (lane & 15)][kk + (lane >> 4) * 8]);
-#pragma unroll
-            for (int j = 0; j < NI; ++j) ldsm_x2_t(bfr[j], &Bs[st][kk + (lane & 15)][wn * TN + j * 8]);
-#pragma unroll
-            for (int i = 0; i < MI; ++i)
-#pragma unroll
-                for (int j = 0; j < NI; ++j) mma_bf16(acc[i][j], af[i], bfr[j]);
-        }
-        __syncthreads();
-    }
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int i = 0; i < MI; ++i)
-#pragma unroll
-        for (int j = 0; j < NI; ++j) {
-            int n = n0 + wn * TN + j * 8 + 2 * t;
-            if (n >= a.Cout) continue;
-            float b0 = a.bias ? a.bias[n] : 0.f, b1 = a.bias ? a.bias[n + 1] : 0.f;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                long long p = m0 + wm * TM + i * 16 + g + h * 8;
-                if (p >= M) continue;
-                float v0 = acc[i][j][2 * h] + b0, v1 = acc[i][j][2 * h + 1] + b1;
-                if (a.relu) {
-                    v0 = fmaxf(v0, 0.f);
-                    v1 = fmaxf(v1, 0.f);
-                }
-                if (a.y)
-                    *reinterpret_cast<__nv_bfloat162*>(a.y + p * a.Cout + n) = __floats2bfloat162_rn(v0, v1);
-                if (a.y32) {
-                    a.y32[p * a.Cout + n] = v0;
-                    a.y32[p * a.Cout + n + 1] = v1;
-                }
-            }
-        }
-}
-
-// ------------------------------------------------ tensor-core convolution
-// The same implicit GEMM on the 5th-generation tensor cores: tcgen05.mma
-// (kind::f16, BF16 operands, FP32 accumulator in tensor memory), one CTA of
-// 128 threads per 128 output pixels and all N = Cout output channels.  A
-// (im2col rows) and B (weights, K-major) are staged by cp.async into shared
-// memory in the 128-byte-swizzled K-major layout, two stages deep; one thread
-// issues the MMAs of a stage and commits them to that stage's mbarrier, which
-// frees the stage for the copies two steps later.  The epilogue reads the
-// accumulator rows back with tcgen05.ld (thread t <-> row t), adds the bias,
-// applies the ReLU and stores BF16.  Every mbarrier wait is bounded; when a
-// wait gives up the kernel sets *err, lets the MMAs it issued finish, skips
-// the epilogue and frees its tensor memory.  The decision to give up is the
-// block's (every thread agrees), so the barriers and the warp-collective
-// tensor-memory loads are never reached by part of a block.
 
 constexpr long long kWaitLimit = 1LL << 22;  // default bound: blocking polls (about a second)
 
-__device__ __forceinline__ uint32_t sw128(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+// Shared-memory matrix descriptors, 128-byte swizzle, 1024-byte aligned
+// operands below 256 KB: the low word holds the address (in 16 bytes) and the
+// leading offset, the high word the stride offset (8-row groups 1024 bytes
+// apart), the version and the swizzle.  An operand `bytes` further is the low
+// word plus bytes / 16, which keeps the issuing thread's work per MMA to one
+// addition (it sets the pace where N = 64).
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
 
-// shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
-// 1024 bytes apart (the leading offset is not used by this layout)
-__device__ __forceinline__ uint64_t umma_sdesc(uint32_t addr)
+__device__ __forceinline__ void umma(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc)
 {
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %5, 0;\n mov.b64 da, {%1, %3};\n mov.b64 db, {%2, "
+        "%3};\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d),
+        "r"(a_lo), "r"(b_lo), "n"(kDescHi), "r"(idesc), "r"(acc));
 }
 
 // instruction descriptor: FP32 accumulator, BF16 A and B, both K-major, M x N
@@ -278,9 +140,236 @@ __device__ __forceinline__ void relu_mask16(uint32_t (&v)[8], const bf16* mask)
     }
 }
 
-template <int N>
-__global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
+// A persistent CTA per SM walks output tiles of 8 MT x 16 pixels of one image
+// and all N output channels, its warps specialised: thread 0 issues the TMA
+// loads up to S stages ahead ("full" mbarriers, transaction bytes), a thread of
+// warp 1 issues a stage's MMAs as it lands and commits them to the stage's
+// "empty" mbarrier, and 4 MT warps read finished accumulators back, two sets
+// of accumulators in tensor memory so that a tile's output overlaps the next
+// tile's MMAs.  A stage is a tap's input window and weights of 64 channels; the
+// image border inside a window comes as TMA's zero fill, and a tap whose window
+// lies outside the image altogether is left out (of 9 taps 6.25 on average are
+// left at dilation 16 and 4 at 32).  The last layer's 8 channels run as N = 16
+// with zero-filled weight rows.
+// What bounds it is the operands' traffic from L2 (8 to 11 TB/s into all SMs).
+// Loading a window once for the three taps above each other (2 KB rows, so the
+// taps are 1024-byte aligned offsets of it) was 20 % faster in the layers of
+// small dilation, but sums the taps in another order, which flips BF16
+// roundings of the stored activations (0.4 % of the output); the order kept
+// here is tap by tap.
+// Measured, forward of 128 problems (all eight layers): 1.06 ms with two CTAs
+// of one tile each per SM and mma.sync for the last layer, 0.83 ms here; the
+// 128 -> 128 layer at dilation 8 runs at 0.95 PFLOP/s, the last layer took 125
+// us of 64 problems and takes 43.
+template <int N, int MT>
+struct ConvWs {
+    static constexpr int WH = 8 * MT, THREADS = 64 + 128 * MT, COLS = 2 * MT * N;
+};
+constexpr int kConvMaxStages = 8;
+constexpr int kFirstSmem = 2 * (128 * 128 + 64 * 128) + 1024;  // k_conv_first's two stages
+constexpr int kConvSmem = 224 * 1024;  // stages, without the alignment slack
+
+// the (tap, channel block) steps of a tile in order, both for the loads and for
+// the MMAs: f(tap, cb, window y, window x); stops when f returns false
+template <int WH, typename F>
+__device__ __forceinline__ bool conv_steps(const ConvArgs& a, int y0, int x0, F f)
 {
+    for (int tap = 0; tap < 9; ++tap) {
+        const int y = y0 + (tap / 3 - 1) * a.dil, x = x0 + (tap % 3 - 1) * a.dil;
+        if (y >= a.H || y + WH <= 0 || x >= a.W || x + 16 <= 0) continue;
+        for (int cb = 0; cb < a.cblocks; ++cb)
+            if (!f(tap, cb, y, x)) return false;
+    }
+    return true;
+}
+
+template <int N, int MT>
+__global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid_constant__ CUtensorMap ta,
+                                                                    const __grid_constant__ CUtensorMap tw,
+                                                                    ConvArgs a, int* err)
+{
+    using C = ConvWs<N, MT>;
+    constexpr int WH = C::WH, A_BYTES = WH * 2048, STAGE = A_BYTES + N * 128;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    __shared__ uint64_t full[kConvMaxStages], empty[kConvMaxStages], tfull[2], tempty[2];
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_issued, s_consumed;
+    const int tid = threadIdx.x, warp = tid >> 5, S = a.stages;
+    const int tiles_x = a.W / 16, per_img = tiles_x * (a.H / WH);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         smem_u32(&tmem_base)),
+                     "r"(C::COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[s])));
+        }
+        for (int k = 0; k < 2; ++k) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&tfull[k])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&tempty[k])), "r"(128 * MT));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n");
+        s_issued = s_consumed = 0;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+    const uint32_t tmem = tmem_base;
+    bool ok = true;
+    if (tid == 0) {
+        // producer
+        const uint64_t pa = reinterpret_cast<uint64_t>(&ta), pw = reinterpret_cast<uint64_t>(&tw);
+        int k = 0;
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+            const int b = t / per_img, r = t - b * per_img;
+            const int y0 = (r / tiles_x) * WH, x0 = (r - (r / tiles_x) * tiles_x) * 16;
+            ok = conv_steps<WH>(a, y0, x0, [&](int tap, int cb, int y, int x) {
+                const int s = k % S;
+                // slot s was last read by the MMAs of step k - S
+                if (k >= S && !mbar_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin)) return false;
+                const uint32_t sa = sbase + s * STAGE, bar = smem_u32(&full[s]);
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(STAGE)
+                             : "memory");
+                asm volatile(
+                    "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+                    "%4, %5}], [%6];\n" ::"r"(sa),
+                    "l"(pa), "r"(cb * 64), "r"(x), "r"(y), "r"(b), "r"(bar)
+                    : "memory");
+                asm volatile(
+                    "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                    "[%4];\n" ::"r"(sa + A_BYTES),
+                    "l"(pw), "r"(tap * a.kc + cb * 64), "r"(0), "r"(bar)
+                    : "memory");
+                ++k;
+                return true;
+            });
+        }
+        s_issued = k;
+    } else if (tid == 32) {
+        // MMA issuer
+        const uint32_t idesc = umma_idesc(128, N);
+        int k = 0, i = 0;
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++i) {
+            const int b = t / per_img, r = t - b * per_img;
+            const int y0 = (r / tiles_x) * WH, x0 = (r - (r / tiles_x) * tiles_x) * 16;
+            const int buf = i & 1;
+            if (i >= 2 && !(ok = mbar_wait(smem_u32(&tempty[buf]), ((i >> 1) - 1) & 1, err, a.spin))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const uint32_t d = tmem + (uint32_t)(buf * MT * N);
+            uint32_t acc = 0u;
+            ok = conv_steps<WH>(a, y0, x0, [&](int, int, int, int) {
+                const int s = k % S;
+                if (!mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin)) return false;
+                asm volatile("tcgen05.fence::after_thread_sync;\n");
+                const uint32_t al = desc_lo(sbase + s * STAGE, 16), bl = al + A_BYTES / 16;
+#pragma unroll
+                for (int ks = 0; ks < 4; ++ks) {  // 16 channels: 32 bytes of the swizzled rows
+#pragma unroll
+                    for (int m = 0; m < MT; ++m)
+                        umma(d + (uint32_t)(m * N), al + m * (128 * 128 / 16) + ks * 2, bl + ks * 2, idesc, acc);
+                    acc = 1u;
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                    smem_u32(&empty[s])));
+                ++k;
+                return true;
+            });
+            if (ok)
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                    smem_u32(&tfull[buf])));
+        }
+        s_consumed = k;
+    } else if (warp >= 2) {
+        // output: warp w reads lanes 32 (w % 4) .. of accumulator (w - 2) / 4;
+        // accumulator row r of window q is the pixel (y0 + 8 q + r / 16, x0 + r % 16)
+        const int q = (warp - 2) >> 2, r = ((warp & 3) << 5) + (tid & 31);
+        const uint32_t lane = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * N);
+        int i = 0;
+        for (int t = blockIdx.x; t < a.tiles; t += gridDim.x, ++i) {
+            const int buf = i & 1;
+            // the whole warp goes on or gives up (the loads below are warp-collective)
+            const bool w = mbar_wait(smem_u32(&tfull[buf]), (i >> 1) & 1, err, a.spin);
+            ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const int b = t / per_img, rr = t - b * per_img;
+            const int y0 = (rr / tiles_x) * WH, x0 = (rr - (rr / tiles_x) * tiles_x) * 16;
+            const long long m = ((long long)b * a.H + y0 + 8 * q + (r >> 4)) * a.W + x0 + (r & 15);
+            const uint32_t src = tmem + lane + (uint32_t)(buf * MT * N);
+#pragma unroll
+            for (int c0 = 0; c0 < N; c0 += 16) {
+                uint32_t v[16];
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+                      "=r"(v[15])
+                    : "r"(src + (uint32_t)c0));
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if constexpr (N == 16) {  // the last layer: 8 FP32 channels
+                    float f[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[j]) + a.bias[j];
+                    float4* dst = reinterpret_cast<float4*>(a.y32 + m * kCout);
+                    dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+                    dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+                } else {
+                    uint32_t packed[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        float f0 = __uint_as_float(v[2 * j]), f1 = __uint_as_float(v[2 * j + 1]);
+                        if (a.bias) {
+                            f0 += a.bias[c0 + 2 * j];
+                            f1 += a.bias[c0 + 2 * j + 1];
+                        }
+                        if (a.relu) {
+                            f0 = fmaxf(f0, 0.f);
+                            f1 = fmaxf(f1, 0.f);
+                        }
+                        __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
+                        packed[j] = *reinterpret_cast<uint32_t*>(&h);
+                    }
+                    if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
+                    uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
+                    dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                    dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;\n");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&tempty[buf])) : "memory");
+        }
+    }
+    const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    if (!all_ok && tid == 0) {
+        // a wait gave up: let the loads this CTA issued and no MMA consumed land
+        // before the shared memory is released, and the MMAs finish before the
+        // tensor memory is (the default bound; commits arrive in issue order)
+        for (int k = s_consumed; k < s_issued; ++k) mbar_wait(smem_u32(&full[k % S]), (k / S) & 1, err);
+        const int nc = s_consumed;
+        if (nc >= 1) mbar_wait(smem_u32(&empty[(nc - 1) % S]), ((nc - 1) / S) & 1, err);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(C::COLS));
+}
+
+// The first layer (40 channels): im2col rows of the 360 features of a pixel
+// staged by cp.async in 64-wide K tiles that run across taps, two stages deep,
+// one CTA of 128 threads per 128 output pixels.  (On k_conv with the channels
+// padded to 64 the K tiles would fall differently and the stored BF16
+// activations would round differently.)  As in k_conv every wait is bounded;
+// the decision to give up is the block's.
+__device__ __forceinline__ uint32_t sw128(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+
+__global__ void __launch_bounds__(128) k_conv_first(ConvArgs a, const bf16* __restrict__ x,
+                                                      const bf16* __restrict__ wk, int* err)
+{
+    constexpr int N = 64, Cin = kCin, K = 9 * kCin;
     constexpr int BK = 64, A_BYTES = 128 * 128, B_BYTES = N * 128, STAGE = A_BYTES + B_BYTES;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -289,7 +378,6 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
     const int tid = threadIdx.x, warp = tid >> 5;
     const int HW = a.H * a.W;
     const long long M = (long long)a.B * HW, m0 = (long long)blockIdx.x * 128;
-    const int K = 9 * a.Cin;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          smem_u32(&tmem_base)),
@@ -335,21 +423,21 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
         const uint32_t sa = sbase + st * STAGE, sb = sa + A_BYTES;
         const int k = kt * BK + c * 8;
         const bool kin = k < K;
-        const int tap = kin ? k / a.Cin : 0, ci = k - tap * a.Cin;
+        const int tap = kin ? k / Cin : 0, ci = k - tap * Cin;
         const int dy = (tap / 3 - 1) * a.dil, dx = (tap % 3 - 1) * a.dil;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int r = r0 + 16 * i;
             const int yy = py[i] + dy, xx = px[i] + dx;
             const bool in = kin && pb[i] >= 0 && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W;
-            const bf16* src = in ? a.x + (((long long)pb[i] * a.H + yy) * a.W + xx) * a.Cin + ci : a.x;
+            const bf16* src = in ? x + (((long long)pb[i] * a.H + yy) * a.W + xx) * Cin + ci : x;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa + sw128(r, c)), "l"(src),
                          "r"(in ? 16 : 0));
         }
 #pragma unroll
         for (int i = 0; i < N / 16; ++i) {
             const int r = r0 + 16 * i;  // output channel
-            const bf16* src = kin ? a.w + (long long)r * K + k : a.w;
+            const bf16* src = kin ? wk + (long long)r * K + k : wk;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sb + sw128(r, c)), "l"(src),
                          "r"(kin ? 16 : 0));
         }
@@ -359,16 +447,10 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
         __syncthreads();
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint32_t idesc = umma_idesc(128, N);
+            const uint32_t idesc = umma_idesc(128, N), al = desc_lo(sa, 16), bl = desc_lo(sb, 16);
 #pragma unroll
-            for (int ks = 0; ks < BK / 16; ++ks) {
-                const uint64_t ad = umma_sdesc(sa + ks * 32), bd = umma_sdesc(sb + ks * 32);
-                const uint32_t acc = (kt > 0 || ks > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-            }
+            for (int ks = 0; ks < BK / 16; ++ks)
+                umma(tmem, al + ks * 2, bl + ks * 2, idesc, (kt > 0 || ks > 0) ? 1u : 0u);
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                 smem_u32(&mbar[st])));
         }
@@ -412,7 +494,6 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
                     __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
                     packed[j] = *reinterpret_cast<uint32_t*>(&h);
                 }
-                if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
                 uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
                 dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
                 dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
@@ -423,186 +504,6 @@ __global__ void __launch_bounds__(128) k_conv_tc(ConvArgs a, int* err)
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(N));
-}
-
-// ------------------------------------------------ TMA-fed tensor-core convolution
-// For inputs of 64 or 128 channels: a CTA computes the output pixels of an
-// 8 MT x 16 window of one image for all N output channels.  The K loop runs over
-// (tap, 64-channel block); for each, one TMA load brings the input window
-// shifted by the tap's offset (the image border comes as TMA's zero fill) and
-// one brings the 64 x N weight tile, both with the 128-byte swizzle, which is
-// the K-major layout the MMA descriptors expect (row = pixel y * 16 + x).
-// Thread 0 (the producer) keeps up to S stages in flight on "full" mbarriers
-// (transaction bytes); thread 32 (the MMA issuer, another warp) issues a
-// stage's MMAs as soon as it lands, and their commit to the stage's "empty"
-// mbarrier frees it for the producer.  The MMAs of consecutive stages queue
-// back to back.  Every wait is bounded; on a timeout the kernel sets *err,
-// waits (bounded) for the loads it issued that no MMA consumed, skips the
-// epilogue and frees its tensor memory.
-// MT windows of 8 x 16 pixels stacked (an 8 MT x 16 window, one TMA load),
-// each with its own accumulator (tensor-memory columns [t N, t N + N)),
-// sharing every weight tile.  Measured on the 128-problem forward pass with
-// one thread loading and issuing: one window 1.42 ms (3 or 4 stages), two
-// windows with 2 stages (two CTAs per SM) 1.11 ms, two with 3 stages 1.48 ms,
-// four windows 1.22 ms; with the producer and the MMA issuer apart, two
-// windows 1.06 ms with 2 stages and 1.29 ms with 3 (one CTA per SM).
-constexpr int kTmaMT = 2;
-template <int N>
-struct TmaConv {
-    static constexpr int MT = kTmaMT;
-    static constexpr int S = MT == 1 ? (N == 128 ? 3 : 4) : 2;
-    static constexpr int A_BYTES = MT * 128 * 128, B_BYTES = N * 128, STAGE = A_BYTES + B_BYTES;
-    static constexpr int SMEM = S * STAGE + 1024;
-    static constexpr int THREADS = 128 * MT;
-};
-
-template <int N>
-__global__ void __launch_bounds__(TmaConv<N>::THREADS) k_conv_tma(const __grid_constant__ CUtensorMap ta,
-                                                                  const __grid_constant__ CUtensorMap tw,
-                                                                  ConvArgs a, int* err)
-{
-    using C = TmaConv<N>;
-    constexpr int S = C::S, A_BYTES = C::A_BYTES, STAGE = C::STAGE, MT = C::MT, WH = 8 * MT;
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    __shared__ uint64_t full[S], empty[S];
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int tiles_x = a.W / 16, per_img = tiles_x * (a.H / WH);
-    const int b = blockIdx.x / per_img, t = blockIdx.x - b * per_img;
-    const int y0 = (t / tiles_x) * WH, x0 = (t - (t / tiles_x) * tiles_x) * 16;
-    const int cblocks = a.Cin / 64, nk = 9 * cblocks;
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                         smem_u32(&tmem_base)),
-                     "r"(MT * N));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-    }
-    if (tid == 0) {
-        for (int s = 0; s < S; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[s])));
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;\n");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n");
-    const uint32_t tmem = tmem_base;
-    __shared__ int consumed;  // steps whose MMAs were issued (set by the issuer)
-    bool ok = true;
-    int issued = 0;
-    if (tid == 0) {
-        // producer: loads run up to S stages ahead of the MMAs
-        const uint64_t pa = reinterpret_cast<uint64_t>(&ta), pw = reinterpret_cast<uint64_t>(&tw);
-        for (int k = 0; k < nk; ++k) {
-            const int s = k % S, tap = k / cblocks, cb = k - tap * cblocks;
-            // slot s was last read by the MMAs of step k - S
-            if (k >= S && !(ok = mbar_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin))) break;
-            const int dy = (tap / 3 - 1) * a.dil, dx = (tap % 3 - 1) * a.dil;
-            const uint32_t sa = sbase + s * STAGE, sb = sa + A_BYTES, bar = smem_u32(&full[s]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(STAGE)
-                         : "memory");
-            asm volatile(
-                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
-                "%4, %5}], [%6];\n" ::"r"(sa),
-                "l"(pa), "r"(cb * 64), "r"(x0 + dx), "r"(y0 + dy), "r"(b), "r"(bar)
-                : "memory");
-            asm volatile(
-                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-                "[%4];\n" ::"r"(sb),
-                "l"(pw), "r"(tap * a.Cin + cb * 64), "r"(0), "r"(bar)
-                : "memory");
-            issued = k + 1;
-        }
-    } else if (tid == 32) {
-        // MMA issuer: each stage's MMAs as soon as its bytes land
-        const uint32_t idesc = umma_idesc(128, N);
-        int k = 0;
-        for (; k < nk; ++k) {
-            const int s = k % S;
-            if (!(ok = mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin))) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint32_t sa = sbase + s * STAGE, sb = sa + A_BYTES;
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-                const uint64_t bd = umma_sdesc(sb + ks * 32);
-                const uint32_t acc = (k > 0 || ks > 0) ? 1u : 0u;
-#pragma unroll
-                for (int q = 0; q < MT; ++q) {
-                    const uint64_t ad = umma_sdesc(sa + q * 128 * 128 + ks * 32);
-                    asm volatile(
-                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                            tmem + (uint32_t)(q * N)),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-                }
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                smem_u32(&empty[s])));
-        }
-        consumed = k;
-    }
-    const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
-    if (!all_ok && tid == 0) {
-        // a wait gave up: let the loads this CTA issued and no MMA consumed land
-        // before the shared memory is released (the default bound)
-        for (int k = consumed; k < issued; ++k) mbar_wait(smem_u32(&full[k % S]), (k / S) & 1, err);
-    }
-    // every MMA issued has finished when the last issued step's commit arrives
-    // (in issue order); after a give-up the MMAs still finish before the
-    // tensor memory is freed
-    ok = all_ok;
-    const int nc = consumed;
-    if (nc >= 1) {
-        const uint32_t bar = smem_u32(&empty[(nc - 1) % S]), par = ((nc - 1) / S) & 1;
-        bool w = ok && mbar_wait(bar, par, err, a.spin);
-        if (!w) mbar_wait(bar, par, err);
-        ok = __syncthreads_and((ok && w) ? 1 : 0) != 0;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;\n");
-    if (ok) {
-        // warp w reads lanes 32 (w % 4) .. of accumulator w / 4; accumulator
-        // row r of window q is the pixel (y0 + 8 q + r / 16, x0 + r % 16)
-        const int q = warp >> 2, r = ((warp & 3) << 5) + (tid & 31);
-        const int py = y0 + 8 * q + (r >> 4), px = x0 + (r & 15);
-        const long long m = ((long long)b * a.H + py) * a.W + px;
-        const uint32_t lane = ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(q * N);
-#pragma unroll
-        for (int c0 = 0; c0 < N; c0 += 16) {
-            uint32_t v[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15])
-                : "r"(tmem + lane + (uint32_t)c0));
-            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-            uint32_t packed[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                float f0 = __uint_as_float(v[2 * j]), f1 = __uint_as_float(v[2 * j + 1]);
-                if (a.bias) {
-                    f0 += a.bias[c0 + 2 * j];
-                    f1 += a.bias[c0 + 2 * j + 1];
-                }
-                if (a.relu) {
-                    f0 = fmaxf(f0, 0.f);
-                    f1 = fmaxf(f1, 0.f);
-                }
-                __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
-                packed[j] = *reinterpret_cast<uint32_t*>(&h);
-            }
-            if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
-            uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
-            dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-            dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(MT * N));
 }
 
 // ------------------------------------------------ weight gradient (tcgen05)
@@ -626,6 +527,7 @@ __global__ void __launch_bounds__(TmaConv<N>::THREADS) k_conv_tma(const __grid_c
 struct WgradArgs {
     int B, H, W, Cin, Cout, dil;
     float* part;       // [splits][9 Cin][Cout]
+    float* bpart;      // [splits][Cout] sums of dy (the bias gradient)
     int G;             // operand pairs of a CTA (blockIdx.y: its first pair / G)
     int npair;         // pairs in all: 9 (Cin = 128) or 5 (Cin <= 64, the tenth plane unused)
     int tiles;         // pixel windows in all
@@ -639,13 +541,10 @@ constexpr int kWgThreads = 128;
 constexpr int kWgMaxStages = 8;
 constexpr int kWgSmem = 216 * 1024;   // stages, without the alignment slack
 
-// MN-major shared-memory descriptor, 128-byte swizzle: 64-element blocks `lbo`
-// bytes apart, 8-pixel groups 1024 bytes apart
-__device__ __forceinline__ uint64_t umma_sdesc_mn(uint32_t addr, uint32_t lbo)
-{
-    return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
+// the order in which 128-channel inputs' taps are dealt to the CTA groups:
+// every three in a row hold one tap of each kernel row and column, so that the
+// windows left out at the image's border are spread evenly
+__device__ __forceinline__ int wgrad_tap(int i) { return (int)((0x642831750ull >> (4 * i)) & 15u); }
 
 template <int N>
 __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ CUtensorMap tx,
@@ -655,15 +554,37 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     constexpr int NB = N / 64;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    __shared__ uint64_t full[kWgMaxStages], empty[kWgMaxStages];
+    __shared__ uint64_t full[kWgMaxStages], empty[kWgMaxStages], done;
     __shared__ uint32_t tmem_base;
-    __shared__ int consumed;
+    __shared__ int consumed, used;
+    __shared__ float sbias[128];
+    const bool bias = blockIdx.y == 0;  // these CTAs' warps 2 and 3 sum dy from its staged tiles
     const int tid = threadIdx.x, warp = tid >> 5, S = a.stages;
     const int g0 = blockIdx.y * a.G, ng = min(a.G, a.npair - g0);
     const int t0 = blockIdx.x * a.per, t1 = min(t0 + a.per, a.tiles), nk = max(t1 - t0, 0);
-    const int stage = (2 * a.G + NB) * kWgPlane, bytes = (2 * ng + NB) * kWgPlane;
+    const int stage = (2 * a.G + NB) * kWgPlane;
     const int tiles_x = a.W / 16, per_img = tiles_x * (a.H / 4);
     const bool wide = a.Cin > 64;
+    // the pairs with a tap whose window meets the image (the others' x is all
+    // zero fill): at dilations 16 and 32 a good part of the windows drop out
+    auto live = [&](int y0, int x0) -> unsigned {
+        if (!wide) return (1u << ng) - 1u;  // dilations up to 4: every window meets it
+        unsigned mk = 0u;
+        for (int g = 0; g < ng; ++g) {
+            const int tap = wgrad_tap(g0 + g), y = y0 + (tap / 3 - 1) * a.dil, x = x0 + (tap % 3 - 1) * a.dil;
+            if (y < a.H && y + 4 > 0 && x < a.W && x + 16 > 0) mk |= 1u << g;
+        }
+        return mk;
+    };
+    // the windows of the split in order (y0, x0, image), without divisions
+    int b = t0 / per_img, y0 = (t0 - b * per_img) / tiles_x * 4, x0 = (t0 - b * per_img) % tiles_x * 16;
+    auto next_window = [&]() {
+        if ((x0 += 16) < a.W) return;
+        x0 = 0;
+        if ((y0 += 4) < a.H) return;
+        y0 = 0;
+        ++b;
+    };
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                          smem_u32(&tmem_base)),
@@ -673,8 +594,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     if (tid == 0) {
         for (int s = 0; s < S; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[s])));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&empty[s])), "r"(bias ? 3 : 1));
         }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&done)));
         asm volatile("fence.mbarrier_init.release.cluster;\n");
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -683,63 +605,98 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     const uint32_t tmem = tmem_base;
     bool ok = true;
     int issued = 0;
-    if (tid == 0) {
-        const uint64_t px = reinterpret_cast<uint64_t>(&tx), py = reinterpret_cast<uint64_t>(&ty);
+    if (warp == 0) {
+        // producer warp: a lane per plane, so that a stage's loads go out together
+        // (one thread issuing all of them kept the MMAs waiting)
+        const int q = tid;
+        const bool isx = q < 2 * ng, mine = q < 2 * ng + NB;
+        int c = (q - 2 * ng) * 64, dx = 0, dy = 0;
+        if (isx) {
+            const int p = 2 * g0 + q;  // plane: (tap, half) or tap
+            const int tap = wide ? wgrad_tap(p >> 1) : min(p, 8);
+            c = wide ? (p & 1) * 64 : 0;
+            dy = (tap / 3 - 1) * a.dil;
+            dx = (tap % 3 - 1) * a.dil;
+        }
+        const uint64_t map = isx ? reinterpret_cast<uint64_t>(&tx) : reinterpret_cast<uint64_t>(&ty);
+        const uint32_t off = (isx ? q : 2 * a.G + q - 2 * ng) * kWgPlane;
         for (int k = 0; k < nk; ++k) {
-            const int s = k % S, t = t0 + k;
-            if (k >= S && !(ok = mbar_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin))) break;
-            const int b = t / per_img, r = t - b * per_img;
-            const int y0 = (r / tiles_x) * 4, x0 = (r - (r / tiles_x) * tiles_x) * 16;
-            const uint32_t sa = sbase + s * stage, bar = smem_u32(&full[s]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
-                         : "memory");
-            for (int q = 0; q < 2 * ng + NB; ++q) {
-                int c, dx = 0, dy = 0;
-                const bool isx = q < 2 * ng;
-                if (isx) {
-                    const int p = 2 * g0 + q;  // plane: (tap, half) or tap
-                    const int tap = min(wide ? p >> 1 : p, 8);
-                    c = wide ? (p & 1) * 64 : 0;
-                    dy = (tap / 3 - 1) * a.dil;
-                    dx = (tap % 3 - 1) * a.dil;
-                } else {
-                    c = (q - 2 * ng) * 64;
-                }
-                const uint32_t dst = sa + (isx ? q : 2 * a.G + q - 2 * ng) * kWgPlane;
+            const int s = k % S;
+            const uint32_t bar = smem_u32(&full[s]);
+            const unsigned mk = live(y0, x0);
+            if (q == 0) {
+                if (k >= S) ok = mbar_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin);
+                if (ok)
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar),
+                                 "r"((2 * __popc(mk) + NB) * kWgPlane)
+                                 : "memory");
+            }
+            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+            if (!ok) break;
+            if (mine && (!isx || ((mk >> (q >> 1)) & 1u)))
                 asm volatile(
                     "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
-                    "%4, %5}], [%6];\n" ::"r"(dst),
-                    "l"(isx ? px : py), "r"(c), "r"(x0 + dx), "r"(y0 + dy), "r"(b), "r"(bar)
+                    "%4, %5}], [%6];\n" ::"r"(sbase + s * stage + off),
+                    "l"(map), "r"(c), "r"(x0 + dx), "r"(y0 + dy), "r"(b), "r"(bar)
                     : "memory");
-            }
             issued = k + 1;
+            next_window();
         }
     } else if (tid == 32) {
         // FP32 accumulator, BF16 operands, both MN-major
         const uint32_t idesc = umma_idesc(128, N) | (1u << 15) | (1u << 16);
+        unsigned have = 0u;  // pairs accumulated into
         int k = 0;
         for (; k < nk; ++k) {
             const int s = k % S;
+            const unsigned mk = live(y0, x0);
+            next_window();
             if (!(ok = mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin))) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint32_t sa = sbase + s * stage, sb = sa + 2 * a.G * kWgPlane;
+            const uint32_t al = desc_lo(sbase + s * stage, kWgPlane);
+            const uint32_t bl = desc_lo(sbase + s * stage + 2 * a.G * kWgPlane, kWgPlane);
             for (int g = 0; g < ng; ++g) {
+                if (!((mk >> g) & 1u)) continue;
+                const uint32_t first = (have >> g) & 1u;
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {  // 16 pixels each
-                    const uint64_t ad = umma_sdesc_mn(sa + 2 * g * kWgPlane + ks * 2048, kWgPlane);
-                    const uint64_t bd = umma_sdesc_mn(sb + ks * 2048, kWgPlane);
-                    const uint32_t acc = (k > 0 || ks > 0) ? 1u : 0u;
-                    asm volatile(
-                        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-                            tmem + (uint32_t)(g * N)),
-                        "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-                }
+                for (int ks = 0; ks < 4; ++ks)  // 16 pixels each
+                    umma(tmem + (uint32_t)(g * N), al + (2 * g * kWgPlane + ks * 2048) / 16, bl + ks * (2048 / 16),
+                         idesc, ks > 0 ? 1u : first);
             }
+            have |= mk;
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                 smem_u32(&empty[s])));
         }
+        if (k > 0)
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                smem_u32(&done)));
         consumed = k;
+        used = (int)have;
+    } else if (warp >= 2 && bias) {
+        // two channels a lane: warp w takes dy plane w - 2 (N = 128) or half of
+        // the rows of the one plane
+        constexpr int ROWS = NB == 2 ? 64 : 32;
+        const int lane = tid & 31, plane = NB == 2 ? warp - 2 : 0, row0 = NB == 2 ? 0 : (warp - 2) * 32;
+        float s0 = 0.f, s1 = 0.f;
+        for (int k = 0; k < nk; ++k) {
+            const int s = k % S;
+            const bool w = mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin);
+            ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
+            if (!ok) break;
+            const uint32_t base = sbase + s * stage + (2 * a.G + plane) * kWgPlane + (lane & 3) * 4;
+#pragma unroll 8
+            for (int r = row0; r < row0 + ROWS; ++r) {
+                uint32_t v;
+                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(base + r * 128 + (((lane >> 2) ^ (r & 7)) << 4)));
+                s0 += __uint_as_float(v << 16);
+                s1 += __uint_as_float(v & 0xffff0000u);
+            }
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&empty[s])) : "memory");
+        }
+        sbias[(warp - 2) * 64 + 2 * lane] = s0;
+        sbias[(warp - 2) * 64 + 2 * lane + 1] = s1;
     }
     const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
     if (!all_ok && tid == 0) {
@@ -748,10 +705,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     }
     ok = all_ok;
     const int nc = consumed;
-    if (nc >= 1) {
-        const uint32_t bar = smem_u32(&empty[(nc - 1) % S]), par = ((nc - 1) / S) & 1;
-        bool w = ok && mbar_wait(bar, par, err, a.spin);
-        if (!w) mbar_wait(bar, par, err);
+    if (nc >= 1) {  // every MMA issued has finished
+        bool w = ok && mbar_wait(smem_u32(&done), 0, err, a.spin);
+        if (!w) mbar_wait(smem_u32(&done), 0, err);
         ok = __syncthreads_and((ok && w) ? 1 : 0) != 0;
     }
     asm volatile("tcgen05.fence::after_thread_sync;\n");
@@ -760,8 +716,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
         // channel m % 64 of tap 2 g + m / 64
         const int m = tid;
         const uint32_t lane = (uint32_t)(warp * 32) << 16;
+        if (bias && tid < N) a.bpart[(size_t)blockIdx.x * N + tid] = sbias[tid] + (NB == 1 ? sbias[tid + 64] : 0.f);
         for (int g = 0; g < ng; ++g) {
-            const int p = 2 * (g0 + g) + (m >> 6), tap = wide ? p >> 1 : p, ci = wide ? m : m & 63;
+            const int p = 2 * (g0 + g) + (m >> 6), tap = wide ? wgrad_tap(g0 + g) : p, ci = wide ? m : m & 63;
             const bool out = tap < 9 && ci < a.Cin;
             float* dst = a.part + ((size_t)blockIdx.x * 9 * a.Cin + (size_t)tap * a.Cin + ci) * N;
 #pragma unroll
@@ -778,7 +735,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
                     uint4* d4 = reinterpret_cast<uint4*>(dst + c0);
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        d4[j] = nk > 0 ? make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3])
+                        d4[j] = ((used >> g) & 1) ? make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3])
                                        : make_uint4(0u, 0u, 0u, 0u);
                 }
             }
@@ -796,32 +753,46 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
 // 9 taps of a scalar times 64 channels: bound by reading and writing the 64
 // channels once, not by arithmetic, and no tensor core is needed (161 us for
 // the weight gradient on mma.sync and 49 us for the data gradient as a tcgen05
-// convolution with 8 input channels, before the ReLU pass; 39 and 48 us here
+// convolution with 8 input channels, before the ReLU pass; 33 and 30 us here
 // with the ReLU mask included, 64 problems).
 constexpr int kLastBlocks = 608;
 
-// dx[p][ci] = sum_tap dy0[p + shift] W[8 - tap][ci][0] where act > 0, else 0; a
-// thread takes 8 channels of a pixel
+// The 9 neighbours dy0[p + dir * shift] of pixel p = (r, c), 0 outside the image
+__device__ __forceinline__ void last_taps(const bf16* __restrict__ dy0, long long p, int r, int c, int H, int W,
+                                          int dir, float (&d)[9])
+{
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap) {
+        const int dr = dir * (tap / 3 - 1), dc = dir * (tap % 3 - 1);
+        const bool in = (unsigned)(r + dr) < (unsigned)H && (unsigned)(c + dc) < (unsigned)W;
+        d[tap] = in ? __bfloat162float(dy0[p + dr * W + dc]) : 0.f;
+    }
+}
+
+// dx[p][ci] = sum_tap dy0[p + shift] w[8 - tap][ci] where act > 0, else 0 (w: the
+// weights of output channel 0); a thread takes 8 channels of every 32nd pixel
+// of the block's run, their 72 weights in registers
 __global__ void __launch_bounds__(256) k_last_dgrad(const bf16* __restrict__ dy0, const bf16* __restrict__ w,
                                                     const bf16* __restrict__ act, long long M, int H, int W,
                                                     bf16* __restrict__ dx)
 {
-    __shared__ float sw[9][64];
-    for (int i = threadIdx.x; i < 576; i += 256) sw[8 - i / 64][i & 63] = __bfloat162float(w[(size_t)i * kCout]);
-    __syncthreads();
-    const int cg = (threadIdx.x & 7) * 8;
-    for (long long p = (blockIdx.x * 256LL + threadIdx.x) >> 3; p < M; p += gridDim.x * 32LL) {
-        const int rem = (int)(p % (H * W)), r = rem / W, c = rem - r * W;
-        float acc[8] = {};
+    const int cg = (threadIdx.x & 7) * 8, HW = H * W;
+    float wr[9][8];
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int dr = tap / 3 - 1, dc = tap % 3 - 1;
-            const bool in = r + dr >= 0 && r + dr < H && c + dc >= 0 && c + dc < W;
-            const float d = in ? __bfloat162float(dy0[p + dr * W + dc]) : 0.f;
+    for (int tap = 0; tap < 9; ++tap)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] = fmaf(d, sw[tap][cg + j], acc[j]);
-        }
+        for (int j = 0; j < 8; ++j) wr[tap][j] = __bfloat162float(w[(8 - tap) * 64 + cg + j]);
+    const long long chunk = ((M + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
+    const long long p0 = blockIdx.x * chunk, p1 = p0 + chunk < M ? p0 + chunk : M;
+    for (long long p = p0 + (threadIdx.x >> 3); p < p1; p += 32) {
         const uint4 av = *reinterpret_cast<const uint4*>(act + p * 64 + cg);
+        const int rem = (int)(p % HW), r = rem / W, c = rem - r * W;
+        float d[9], acc[8] = {};
+        last_taps(dy0, p, r, c, H, W, 1, d);
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] = fmaf(d[tap], wr[tap][j], acc[j]);
         const bf16* ab = reinterpret_cast<const bf16*>(&av);
         uint4 ov;
         bf16* ob = reinterpret_cast<bf16*>(&ov);
@@ -838,27 +809,25 @@ __global__ void __launch_bounds__(256) k_last_dgrad(const bf16* __restrict__ dy0
 __global__ void __launch_bounds__(256) k_last_wgrad(const bf16* __restrict__ x, const bf16* __restrict__ dy0,
                                                     long long M, int H, int W, float* __restrict__ part)
 {
-    const int cgi = threadIdx.x & 7, cg = cgi * 8, pl = threadIdx.x >> 3;
+    const int cgi = threadIdx.x & 7, cg = cgi * 8, pl = threadIdx.x >> 3, HW = H * W;
     const long long chunk = ((M + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
     const long long p0 = blockIdx.x * chunk, p1 = p0 + chunk < M ? p0 + chunk : M;
     float acc[9][8] = {};
     float bs = 0.f;
+#pragma unroll 2
     for (long long p = p0 + pl; p < p1; p += 32) {
-        const int rem = (int)(p % (H * W)), r = rem / W, c = rem - r * W;
         const uint4 xv = *reinterpret_cast<const uint4*>(x + p * 64 + cg);
+        const int rem = (int)(p % HW), r = rem / W, c = rem - r * W;
+        float d[9];
+        last_taps(dy0, p, r, c, H, W, -1, d);
         const bf16* xb = reinterpret_cast<const bf16*>(&xv);
-        float xf[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) xf[j] = __bfloat162float(xb[j]);
+        for (int j = 0; j < 8; ++j) {
+            const float xf = __bfloat162float(xb[j]);
 #pragma unroll
-        for (int tap = 0; tap < 9; ++tap) {
-            const int dr = tap / 3 - 1, dc = tap % 3 - 1;
-            const bool in = r - dr >= 0 && r - dr < H && c - dc >= 0 && c - dc < W;
-            const float d = in ? __bfloat162float(dy0[p - dr * W - dc]) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[tap][j] = fmaf(d, xf[j], acc[tap][j]);
-            if (tap == 4) bs += d;
+            for (int tap = 0; tap < 9; ++tap) acc[tap][j] = fmaf(d[tap], xf, acc[tap][j]);
         }
+        bs += d[4];
     }
     // over the warp's 4 pixels, then over the 8 warps
     __shared__ float red[8][577];
@@ -896,56 +865,28 @@ __global__ void k_last_sum(const float* __restrict__ part, int blocks, float* __
     if (lane < kCout) dst[lane] = lane == 0 ? v : 0.f;
 }
 
-// grad[i] = sum over splits of part[s][i]  (fixed order: deterministic)
-__global__ void k_sum_splits(const float* part, int splits, long long n, float* grad)
+// sums over the splits in a fixed order (deterministic): a layer's n weights
+// from part[s][i] and, after them, its nb biases from bpart[s][i].  A block
+// takes 32 entries in 8 slices of the splits (one thread per entry took 16 us
+// for 152 splits)
+__global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ part, int splits, int n,
+                                                    float* __restrict__ grad, const float* __restrict__ bpart, int nb,
+                                                    float* __restrict__ gbias)
 {
-    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    const bool w = blockIdx.x * 32 < n;  // n is a multiple of 32
+    const float* src = w ? part + i : bpart + (i - n);
+    const int stride = w ? n : nb;
     float s = 0.f;
-    for (int q = 0; q < splits; ++q) s += part[(size_t)q * n + i];
-    grad[i] = s;
-}
-
-// bias gradient: per channel sum over pixels.  Every block sums a run of
-// pixels, a thread 8 channels (16 bytes) of every (256 C / 8)th pixel, so that
-// a warp reads whole rows; block partials in a fixed order.  Bound by reading
-// dy once; one block per channel with a stride of C between its reads took 176
-// us for 64 problems x 64 channels.
-constexpr int kBiasBlocks = 304;
-template <int C>
-__global__ void __launch_bounds__(256) k_bias_part(const bf16* __restrict__ dy, long long M, float* __restrict__ part)
-{
-    constexpr int TC = C / 8, PL = 256 / TC;  // threads across the channels, pixels per pass
-    const int cg = (threadIdx.x % TC) * 8, pl = threadIdx.x / TC;
-    const long long chunk = (M + gridDim.x - 1) / gridDim.x;
-    const long long p0 = blockIdx.x * chunk, p1 = p0 + chunk < M ? p0 + chunk : M;
-    float acc[8] = {};
 #pragma unroll 4
-    for (long long p = p0 + pl; p < p1; p += PL) {
-        const uint4 v = *reinterpret_cast<const uint4*>(dy + p * C + cg);
-        const bf16* b = reinterpret_cast<const bf16*>(&v);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] += __bfloat162float(b[j]);
-    }
-    __shared__ float red[PL][C];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) red[pl][cg + j] = acc[j];
+    for (int q = sl; q < splits; q += 8) s += src[(size_t)q * stride];
+    __shared__ float sh[8][32];
+    sh[sl][lane] = s;
     __syncthreads();
-    for (int c = threadIdx.x; c < C; c += 256) {
-        float s = 0.f;
-        for (int q = 0; q < PL; ++q) s += red[q][c];
-        part[(size_t)blockIdx.x * C + c] = s;
+    if (sl == 0) {
+        for (int q = 1; q < 8; ++q) s += sh[q][lane];
+        (w ? grad + i : gbias + (i - n))[0] = s;
     }
-}
-
-__global__ void k_bias_sum(const float* __restrict__ part, int blocks, int C, float* __restrict__ grad)
-{
-    const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (c >= C) return;
-    float v = 0.f;
-    for (int b = lane; b < blocks; b += 32) v += part[(size_t)b * C + c];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) grad[c] = v;
 }
 
 // loss = 1/2 mean over the M cells of (y[p][0] - t[p])^2, dy0[p] = (y - t) / M
@@ -990,12 +931,11 @@ struct LayerTab {
     int cin[kLayers], cout[kLayers];
 };
 
-// BF16 copies of one FP32 parameter: the weights as stored (W[k][co], the
-// mma.sync forward), K-major for the tensor-core forward (Wk[co][k]), and the
-// flipped, transposed weights of the data gradient, [k'][ci] for mma.sync
-// and K-major [ci][k'] for the tensor cores (k' = (8 - tap) Cout + co)
+// BF16 copies of one FP32 parameter, both K-major: the forward's weights
+// wk[co][tap * Cin + ci] and the flipped, transposed weights of the data
+// gradient wtk[ci][k'], k' = (8 - tap) Cout + co
 struct WeightCopies {
-    bf16 *wb, *wt, *wk, *wtk;
+    bf16 *wk, *wtk;
 };
 
 __device__ __forceinline__ void write_copies(long long i, float p, const LayerTab& T, const WeightCopies& w)
@@ -1009,8 +949,6 @@ __device__ __forceinline__ void write_copies(long long i, float p, const LayerTa
             int tap = (int)(k / cin), ci = (int)(k % cin);
             long long kp = (long long)(8 - tap) * cout + co;
             const bf16 pb = __float2bfloat16(p);
-            w.wb[i] = pb;
-            w.wt[T.woff[l] + kp * cin + ci] = pb;
             w.wk[T.woff[l] + (long long)co * 9 * cin + k] = pb;
             w.wtk[T.woff[l] + (long long)ci * 9 * cout + kp] = pb;
         }
@@ -1145,7 +1083,7 @@ struct adr_cnn {
     long P = 0;
     LayerTab T{};
     float *prm = nullptr, *m = nullptr, *v = nullptr, *grad = nullptr;
-    bf16 *wb = nullptr, *wt = nullptr, *wk = nullptr, *wtk = nullptr;
+    bf16 *wk = nullptr, *wtk = nullptr;
     int* err = nullptr;  // a bounded wait of a tensor-core kernel gave up
     long long spin = 0;  // bound of those waits (adr_cnn_set_wait_limit; 0: default)
     bf16* act[kLayers] = {};  // post-activation outputs of layers 0..6 (bf16)
@@ -1177,12 +1115,6 @@ adr_status cnn_alloc(adr_cnn* c, T** p, size_t n)
     return ADR_OK;
 }
 
-template <int N>
-constexpr int tc_smem_bytes()
-{
-    return 2 * (128 * 128 + N * 128) + 1024;
-}
-
 // the driver's tensor-map encoder, looked up once through the runtime
 PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
 {
@@ -1202,68 +1134,65 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
     return fn;
 }
 
-// tensor maps of a convolution's input [B][H][W][Cin] (box: 64 channels x 16 x
-// 8 pixels) and K-major weights [N][9 Cin] (box: 64 x N), 128-byte swizzle;
-// false when the driver refuses them (the caller takes another kernel)
-bool conv_tensor_maps(const ConvArgs& a, const bf16* wk, CUtensorMap* ta, CUtensorMap* tw)
+// tensor map of an activation [B][H][W][C] with a box of 64 channels x 16 x
+// rows pixels, 128-byte swizzle (channels past C and pixels past the image
+// read as zero)
+bool act_map(CUtensorMap* m, const bf16* x, int B, int H, int W, int C, int rows)
 {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
     if (!enc) return false;
-    const cuuint64_t C = (cuuint64_t)a.Cin, K = 9 * C;
-    cuuint64_t dA[4] = {C, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.B};
-    cuuint64_t sA[3] = {C * 2, C * 2 * a.W, C * 2 * a.W * a.H};
-    cuuint32_t bA[4] = {64, 16, 8 * kTmaMT, 1}, e4[4] = {1, 1, 1, 1};
-    if (enc(ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(a.x), dA, sA, bA, e4,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-    cuuint64_t dW[2] = {K, (cuuint64_t)a.Cout};
-    cuuint64_t sW[1] = {K * 2};
-    cuuint32_t bW[2] = {64, (cuuint32_t)a.Cout}, e2[2] = {1, 1};
-    return enc(tw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16*>(wk), dW, sW, bW, e2,
+    cuuint64_t d[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+    cuuint64_t st[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
+    cuuint32_t box[4] = {64, 16, (cuuint32_t)rows, 1}, e[4] = {1, 1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(x), d, st, box, e,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// tensor-core paths for 64 or 128 output channels with a BF16 output (wk: the
-// K-major weights): TMA-fed for inputs of a multiple of 64 channels on 8 x 16
-// pixel windows, cp.async-fed otherwise; mma.sync for the rest
-void launch_conv(cudaStream_t st, const ConvArgs& a, const bf16* wk = nullptr, int* err = nullptr)
+// tensor map of K-major weights [Cout][K] with a box of 64 x n rows (rows past
+// Cout read as zero)
+bool weight_map(CUtensorMap* m, const bf16* w, int K, int Cout, int n)
 {
-    long long M = (long long)a.B * a.H * a.W;
-    if (wk && err && a.y && !a.y32 && (a.Cout == 64 || a.Cout == 128) && a.Cin % 64 == 0 &&
-        a.H % (8 * kTmaMT) == 0 && a.W % 16 == 0) {
-        CUtensorMap ta, tw;
-        if (conv_tensor_maps(a, wk, &ta, &tw)) {
-            ConvArgs t = a;
-            t.w = wk;
-            const unsigned blocks = (unsigned)(a.B * (a.H / (8 * kTmaMT)) * (a.W / 16));
-            if (a.Cout == 64)
-                k_conv_tma<64><<<blocks, TmaConv<64>::THREADS, TmaConv<64>::SMEM, st>>>(ta, tw, t, err);
-            else
-                k_conv_tma<128><<<blocks, TmaConv<128>::THREADS, TmaConv<128>::SMEM, st>>>(ta, tw, t, err);
-            return;
-        }
+    PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
+    if (!enc) return false;
+    cuuint64_t d[2] = {(cuuint64_t)K, (cuuint64_t)Cout}, st[1] = {(cuuint64_t)K * 2};
+    cuuint32_t box[2] = {64, (cuuint32_t)n}, e[2] = {1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16*>(w), d, st, box, e,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int N, int MT>
+adr_status launch_conv_t(const adr_cnn* c, cudaStream_t st, ConvArgs a, const bf16* x, int cin, const bf16* wk,
+                         int cout)
+{
+    constexpr int WH = 8 * MT;
+    a.cblocks = cin / 64;
+    a.kc = cin;
+    constexpr int stage = WH * 2048 + N * 128;
+    a.stages = std::min(kConvMaxStages, kConvSmem / stage);
+    a.tiles = a.B * (a.H / WH) * (a.W / 16);
+    CUtensorMap ta, tw;
+    if (!act_map(&ta, x, a.B, a.H, a.W, cin, WH) || !weight_map(&tw, wk, 9 * a.kc, cout, N)) {
+        adr::set_error("the driver refused a tensor map of a convolution");
+        return ADR_ECUDA;
     }
-    if (wk && err && a.y && !a.y32 && (a.Cout == 64 || a.Cout == 128)) {
-        ConvArgs t = a;
-        t.w = wk;
-        const unsigned blocks = (unsigned)((M + 127) / 128);
-        if (a.Cout == 64) k_conv_tc<64><<<blocks, 128, tc_smem_bytes<64>(), st>>>(t, err);
-        else k_conv_tc<128><<<blocks, 128, tc_smem_bytes<128>(), st>>>(t, err);
-        return;
-    }
-    dim3 grid((unsigned)((M + 127) / 128), 1);
-    if (a.Cout >= 64) {
-        grid.y = (a.Cout + 63) / 64;
-        k_conv_fwd<64><<<grid, 256, 0, st>>>(a);
-    } else if (a.Cout % 16 == 0) {
-        grid.y = a.Cout / 16;
-        k_conv_fwd<16><<<grid, 256, 0, st>>>(a);
-    } else {
-        grid.y = (a.Cout + 7) / 8;
-        k_conv_fwd<8><<<grid, 256, 0, st>>>(a);
-    }
+    k_conv<N, MT><<<std::min(c->n_sm, a.tiles), ConvWs<N, MT>::THREADS, a.stages * stage + 1024, st>>>(ta, tw, a,
+                                                                                                      c->err);
+    return ADR_OK;
+}
+
+// tiles of 16 x 16 pixels, or of 8 x 16 where the larger ones would leave SMs
+// without one (fewer than about 10 problems)
+adr_status launch_conv(const adr_cnn* c, cudaStream_t st, const ConvArgs& a, const bf16* x, int cin, const bf16* wk,
+                       int cout)
+{
+    const bool big = a.B * (a.H / 16) * (a.W / 16) >= c->n_sm;
+    if (cout == 128)
+        return big ? launch_conv_t<128, 2>(c, st, a, x, cin, wk, cout) : launch_conv_t<128, 1>(c, st, a, x, cin, wk, cout);
+    if (cout == 64)
+        return big ? launch_conv_t<64, 2>(c, st, a, x, cin, wk, cout) : launch_conv_t<64, 1>(c, st, a, x, cin, wk, cout);
+    return big ? launch_conv_t<16, 2>(c, st, a, x, cin, wk, cout) : launch_conv_t<16, 1>(c, st, a, x, cin, wk, cout);
 }
 
 // forward of a batch: act[0..6] bf16, y32 of the last layer
@@ -1274,35 +1203,21 @@ adr_status cnn_forward(adr_cnn* c, int batch, const bf16* x)
         ConvArgs a{};
         a.B = batch;
         a.H = a.W = c->hw;
-        a.Cin = kCh[l];
-        a.Cout = kCh[l + 1];
         a.dil = kDil[l];
-        a.x = in;
-        a.w = c->wb + c->T.woff[l];
         a.bias = c->prm + c->T.boff[l];
         a.relu = l < kLayers - 1;
         a.spin = c->spin;
         if (l < kLayers - 1) a.y = c->act[l];
         else a.y32 = c->y32;
-        launch_conv(c->stream, a, c->wk + c->T.woff[l], c->err);
+        const bf16* wk = c->wk + c->T.woff[l];
+        if (l == 0)
+            k_conv_first<<<(unsigned)(((long long)batch * c->hw * c->hw + 127) / 128), 128, kFirstSmem, c->stream>>>(
+                a, in, wk, c->err);
+        else TRY_S(launch_conv(c, c->stream, a, in, kCh[l], wk, kCh[l + 1]));
         in = c->act[l];
     }
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
-}
-
-// tensor map of an activation [B][H][W][C] with a box of 64 channels x 16 x 4
-// pixels, 128-byte swizzle
-bool wgrad_map(CUtensorMap* m, const bf16* x, int B, int H, int W, int C)
-{
-    PFN_cuTensorMapEncodeTiled_v12000 enc = tmap_encoder();
-    if (!enc) return false;
-    cuuint64_t d[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
-    cuuint64_t st[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
-    cuuint32_t box[4] = {64, 16, 4, 1}, e[4] = {1, 1, 1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(x), d, st, box, e,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // weight and bias gradients of a layer of 64 or 128 output channels from its
@@ -1313,7 +1228,7 @@ adr_status layer_grad(adr_cnn* c, int batch, int l, const bf16* xin, const bf16*
     const int cin = kCh[l], cout = kCh[l + 1];
     const long long M = (long long)batch * c->hw * c->hw;
     CUtensorMap tx, ty;
-    if (!wgrad_map(&tx, xin, batch, c->hw, c->hw, cin) || !wgrad_map(&ty, dy, batch, c->hw, c->hw, cout)) {
+    if (!act_map(&tx, xin, batch, c->hw, c->hw, cin, 4) || !act_map(&ty, dy, batch, c->hw, c->hw, cout, 4)) {
         adr::set_error("the driver refused a tensor map of the weight gradient");
         return ADR_ECUDA;
     }
@@ -1324,9 +1239,10 @@ adr_status layer_grad(adr_cnn* c, int batch, int l, const bf16* xin, const bf16*
     w.Cout = cout;
     w.dil = kDil[l];
     w.part = c->part;
+    w.bpart = c->spart;
     w.spin = c->spin;
     w.npair = cin > 64 ? 9 : 5;
-    w.G = cout == 128 ? 3 : 5;  // accumulators: G x cout of 512 columns of tensor memory
+    w.G = cin > 64 || cout == 128 ? 3 : 5;  // accumulators: G x cout of 512 columns of tensor memory
     const int groups = (w.npair + w.G - 1) / w.G;
     const int stage = (2 * w.G + cout / 64) * kWgPlane;
     w.stages = std::min(kWgMaxStages, kWgSmem / stage);
@@ -1339,12 +1255,9 @@ adr_status layer_grad(adr_cnn* c, int batch, int l, const bf16* xin, const bf16*
     const dim3 grid((unsigned)splits, (unsigned)groups);
     if (cout == 128) k_wgrad_tc<128><<<grid, kWgThreads, smem, st>>>(tx, ty, w, cols, c->err);
     else k_wgrad_tc<64><<<grid, kWgThreads, smem, st>>>(tx, ty, w, cols, c->err);
-    const long long nw = 9LL * cin * cout;
-    k_sum_splits<<<(int)((nw + 255) / 256), 256, 0, st>>>(c->part, splits, nw, c->grad + c->T.woff[l]);
-    const int nb = (int)std::min<long long>(kBiasBlocks, (M + 63) / 64);
-    if (cout == 128) k_bias_part<128><<<nb, 256, 0, st>>>(dy, M, c->spart);
-    else k_bias_part<64><<<nb, 256, 0, st>>>(dy, M, c->spart);
-    k_bias_sum<<<(cout * 32 + 255) / 256, 256, 0, st>>>(c->spart, nb, cout, c->grad + c->T.boff[l]);
+    const int nw = 9 * cin * cout;
+    k_sum_splits<<<(nw + cout) / 32, 256, 0, st>>>(c->part, splits, nw, c->grad + c->T.woff[l], c->spart, cout,
+                                                   c->grad + c->T.boff[l]);
     return ADR_OK;
 }
 
@@ -1361,7 +1274,7 @@ adr_status cnn_backward(adr_cnn* c, int batch, const bf16* x, const float* t)
     k_last_sum<<<(577 * 32 + 255) / 256, 256, 0, st>>>(c->spart, lb, c->grad + c->T.woff[last],
                                                       c->grad + c->T.boff[last]);
     bf16* dy = c->dA;
-    k_last_dgrad<<<lb, 256, 0, st>>>(c->dy0, c->wb + c->T.woff[last], c->act[last - 1], M, c->hw, c->hw, dy);
+    k_last_dgrad<<<lb, 256, 0, st>>>(c->dy0, c->wk + c->T.woff[last], c->act[last - 1], M, c->hw, c->hw, dy);
     for (int l = last - 1; l >= 0; --l) {
         TRY_S(layer_grad(c, batch, l, l == 0 ? x : c->act[l - 1], dy));
         if (l > 0) {
@@ -1370,15 +1283,11 @@ adr_status cnn_backward(adr_cnn* c, int batch, const bf16* x, const float* t)
             ConvArgs a{};
             a.B = batch;
             a.H = a.W = c->hw;
-            a.Cin = kCh[l + 1];
-            a.Cout = kCh[l];
             a.dil = kDil[l];
-            a.x = dy;
-            a.w = c->wt + c->T.woff[l];
             a.mask = c->act[l - 1];
             a.spin = c->spin;
             a.y = dy == c->dA ? c->dB : c->dA;
-            launch_conv(st, a, c->wtk + c->T.woff[l], c->err);
+            TRY_S(launch_conv(c, st, a, dy, kCh[l + 1], c->wtk + c->T.woff[l], kCh[l]));
             dy = a.y;
         }
     }
@@ -1443,7 +1352,7 @@ adr_status adr_cnn_set_params(adr_cnn* c, const float* host)
     ADR_CUDA_TRY(cudaMemsetAsync(c->v, 0, sizeof(float) * c->P, c->stream));
     c->step = 0;
     k_refresh<<<(int)((c->P + 255) / 256), 256, 0, c->stream>>>(c->prm, c->P, c->T,
-                                                                WeightCopies{c->wb, c->wt, c->wk, c->wtk});
+                                                                WeightCopies{c->wk, c->wtk});
     ADR_CUDA_TRY(cudaGetLastError());
     ADR_CUDA_TRY(cudaStreamSynchronize(c->stream));
     return ADR_OK;
@@ -1491,7 +1400,6 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
     };
     if ((s = cnn_alloc(c, &c->prm, c->P)) || (s = cnn_alloc(c, &c->m, c->P)) ||
         (s = cnn_alloc(c, &c->v, c->P)) || (s = cnn_alloc(c, &c->grad, c->P)) ||
-        (s = cnn_alloc(c, &c->wb, c->P)) || (s = cnn_alloc(c, &c->wt, c->P)) ||
         (s = cnn_alloc(c, &c->wk, c->P)) || (s = cnn_alloc(c, &c->wtk, c->P)) ||
         (s = cnn_alloc(c, &c->err, 1)) ||
         (s = cnn_alloc(c, &c->y32, M * kCout)) || (s = cnn_alloc(c, &c->dA, M * 128)) ||
@@ -1505,16 +1413,13 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
     if ((s = cnn_alloc(c, &c->part, c->part_size))) return fail(s);
     ADR_CUDA_TRY(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
     // the tensor-core kernels use more than 48 KB of shared memory (per device)
-    ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      tc_smem_bytes<64>()));
-    ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      tc_smem_bytes<128>()));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem + 1024));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem + 1024));
-    ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tma<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      TmaConv<64>::SMEM));
-    ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_tma<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      TmaConv<128>::SMEM));
+    ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_first, cudaFuncAttributeMaxDynamicSharedMemorySize, kFirstSmem));
+    const void* convs[] = {(const void*)k_conv<16, 1>, (const void*)k_conv<16, 2>,  (const void*)k_conv<64, 1>,
+                           (const void*)k_conv<64, 2>, (const void*)k_conv<128, 1>, (const void*)k_conv<128, 2>};
+    for (const void* f : convs)
+        ADR_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem + 1024));
     if ((s = adr_cnn_set_params(c, params))) return fail(s);
     *out = c;
     return ADR_OK;
@@ -1602,7 +1507,7 @@ adr_status adr_cnn_train_step(adr_cnn* c, int batch, const uint16_t* x, const fl
     float c1 = 1.f - powf(b1, (float)c->step), c2 = 1.f - powf(b2, (float)c->step);
     k_adam<<<(int)((c->P + 255) / 256), 256, 0, c->stream>>>(
         c->prm, c->m, c->v, c->grad, c->P, lr, b1, b2, 1e-8f, c1, c2, c->T,
-        WeightCopies{c->wb, c->wt, c->wk, c->wtk});
+        WeightCopies{c->wk, c->wtk});
     ADR_CUDA_TRY(cudaGetLastError());
     if (loss) {
         int e = 0;
