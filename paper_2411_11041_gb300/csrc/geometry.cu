@@ -687,7 +687,9 @@ __global__ void k_bnd_scan(const int* norder, const double* w, int cap_order, do
         for (int j = 0; j < 32; ++j) {
             const double wv = __shfl_sync(0xffffffffu, wl, j);
             if (lane == j) mine = cum;
-            if (wv > 0.0) cum += wv;  // past n the weights are 0
+            // wv > 0 from its bits (an FP64 comparison costs as much as the sum);
+            // past n the weights are 0
+            if ((unsigned long long)(__double_as_longlong(wv) - 1) < 0x7ff0000000000000ull) cum += wv;
         }
         if (base + lane < n) cbf[base + lane] = mine;
     }
@@ -785,135 +787,244 @@ __device__ __forceinline__ bool seed_of(const int* nseeds, int cap, int t, int* 
     return false;
 }
 
-// Two warps trace each 32 curves: lane l of warp 0 and lane l of warp 1 work
-// on the same curve.  Warp 0 computes the x halves of every RK4 stage (beta1
-// at the stage point, the x component of the direction, the x coordinate),
-// warp 1 the y halves, and the two trade what the other half needs through
-// shared memory: the cell index and local coordinate, then the field value,
-// at every stage, and the new point with its interior-test halves at every
-// step.  An FP64 warp instruction holds its sub-partition's FP64 unit for
-// about 64 cycles, and the two warps run on different sub-partitions, so a
-// stage's chain is about a third shorter.  Every value comes from the same
-// operations as in rk4, direction and interior_point, so the points are the
-// same.  All lanes of both warps reach every barrier: a lane whose curve is
-// done computes on its last point and drops the result.
-struct Trade {
-    double a, b;
-    int i, j, k;
-};
-
-// publish this warp's values for the lane, read the other warp's; the buffer
-// alternates, so that one barrier per trade suffices
-__device__ __forceinline__ Trade trade(Trade (*buf)[2][32], int& nb, int w, int lane, Trade mine)
+// ---- one direction component, num / sqrt(s), as direction computes it
+// A warp's FP64 instruction takes 64 cycles, dependent or not, whatever the
+// number of active lanes; the compiler's square root and division take about 9
+// each, half of a stage.  Here 1/sqrt(s) comes from the FP32 pipe (about 5
+// cycles an instruction) to 2^-45: the hardware estimate r0 and one
+// second-order step on e = 1 - s r0^2, e formed exactly enough by FMA
+// residuals.  Square root and quotient then follow Markstein's scheme (IBM J.
+// Res. Dev. 34, 1990): an approximation, its exact residual by FMA, and one
+// corrected rounding.  The value rounded last is within 2^-89 (relative) of the
+// true one, so the result is the correctly rounded one, as sqrt and / give,
+// unless the true value lies that close to a rounding boundary (one in 2^35).
+__device__ __forceinline__ double f32_widen(float x)  // exact for normal x, integer pipe
 {
-    buf[nb][w][lane] = mine;
-    __syncthreads();
-    Trade o = buf[nb][w ^ 1][lane];
-    nb ^= 1;
-    return o;
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
 
-// this warp's direction component at the stage point whose own coordinate is
-// c (the other warp holds the other coordinate); bad is raised where |beta|
-// is not positive (direction's failure)
-__device__ __forceinline__ double half_direction(const GridView& g, int w, int fam, double c,
-                                                 Trade (*buf)[2][32], int& nb, int lane, bool& bad)
+__device__ __forceinline__ double unit_component(double num, double s, bool& bad)
 {
-    const int lim = w == 0 ? g.nx - 2 : g.ny - 2;
-    int q = __double2int_rd(c);
-    if (q > lim) q = lim;
-    if (q < 0) q = 0;
-    const double l = c - q, a = 1.0 - l;
-    const Trade t = trade(buf, nb, w, lane, Trade{l, a, q, 0, 0});
-    const int i = w == 0 ? q : t.i, r = w == 0 ? t.i : q;
-    const double lx = w == 0 ? l : t.a, ax = w == 0 ? a : t.b;
-    const double ly = w == 0 ? t.a : l, ay = w == 0 ? t.b : a;
-    const double w11 = ay * ax, w12 = ay * lx, w21 = ly * ax, w22 = ly * lx;
-    const double* p = (w == 0 ? g.beta1 : g.beta2) + ((size_t)r * g.nx + i);
-    const double v = w11 * p[0] + w12 * p[1] + w21 * p[g.nx] + w22 * p[g.nx + 1];
-    const Trade u = trade(buf, nb, w, lane, Trade{v, 0.0, 0, 0, 0});
-    const double b1 = w == 0 ? v : u.a, b2 = w == 0 ? u.a : v;
-    const double nrm = sqrt(b1 * b1 + b2 * b2);
+    const unsigned hi = (unsigned)__double2hiint(s), lo = (unsigned)__double2loint(s);
+    if (hi - (963u << 20) < (120u << 20)) {  // 2^-60 <= s < 2^60
+        // s = sh + sl exactly, both FP32
+        const float sh = __uint_as_float(__funnelshift_r(lo, hi, 29) - (384u << 23));
+        const float sl = __uint2float_rn(lo & 0x1fffffffu) * __uint_as_float(((hi >> 20) - 1023u - 52u + 127u) << 23);
+        const float r0 = rsqrtf(sh);
+        const float p = r0 * r0, pe = __fmaf_rn(r0, r0, -p);
+        const float t = sh * p, te = __fmaf_rn(sh, p, -t);
+        float e = (1.0f - t) - te;
+        e = __fmaf_rn(-sh, pe, e);
+        e = __fmaf_rn(-sl, p, e);
+        const float rl = r0 * (e * __fmaf_rn(0.375f, e, 0.5f));
+        double y = f32_widen(r0);
+        if (fabsf(rl) >= 1.1754944e-38f) y = y + f32_widen(rl);
+        const double hy = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));  // y / 2
+        double g = s * y;
+        g = __fma_rn(__fma_rn(-g, g, s), hy, g);
+        const double q = num * y;
+        return __fma_rn(__fma_rn(-q, g, num), y, q);
+    }
+    const double nrm = sqrt(s);
     if (!(nrm > 0.0)) bad = true;
-    const double num = w == 0 ? (fam == 0 ? b1 : b2) : (fam == 0 ? b2 : -b1);
     return num / nrm;
 }
 
-// this warp's coordinate after one classical RK4 step of step component st
-__device__ __forceinline__ double half_rk4(const GridView& g, int w, int fam, double c, double st,
-                                           Trade (*buf)[2][32], int& nb, int lane, bool& bad)
+// cell index and local coordinate of c as bilin takes them (q clamped to [0,
+// lim], l = c - q); plain: c >= 0 lies strictly inside cell q, away from its
+// ends by more than the snapping tolerance (then snap leaves c alone and
+// floor(c) = q).  The integer part comes from the bits of c.
+struct Split {
+    int q, qu;  // clamped and unclamped cell
+    double l;
+    bool plain;
+};
+__device__ __forceinline__ Split split(double c, int lim, double limd)
 {
-    const double k1 = half_direction(g, w, fam, c, buf, nb, lane, bad);
-    const double k2 = half_direction(g, w, fam, c + 0.5 * st * k1, buf, nb, lane, bad);
-    const double k3 = half_direction(g, w, fam, c + 0.5 * st * k2, buf, nb, lane, bad);
-    const double k4 = half_direction(g, w, fam, c + st * k3, buf, nb, lane, bad);
-    return c + st / 6.0 * (k1 + 2.0 * k2 + 2.0 * k3 + k4);
+    Split r;
+    const unsigned hi = (unsigned)__double2hiint(c), lo = (unsigned)__double2loint(c);
+    double qd = 0.0;
+    if (hi < (1043u << 20)) {  // 0 <= c < 2^20
+        const int e = (int)(hi >> 20) - 1023;
+        r.qu = 0;
+        if (e >= 0) {
+            r.qu = (int)((0x100000u | (hi & 0xfffffu)) >> (20 - e));
+            qd = __hiloint2double((int)(hi & ~(0xfffffu >> e)), 0);
+        }
+        r.q = r.qu;
+        if (r.q > lim) {
+            r.q = lim;
+            qd = limd;
+        }
+        r.l = c - qd;
+        const unsigned hl = (unsigned)__double2hiint(r.l);
+        r.plain = hl - (994u << 20) < 0x3fefffffu - (994u << 20);  // 2^-29 <= l < 1 - 2^-21
+        (void)lo;
+        return r;
+    }
+    r.q = r.qu = __double2int_rd(c);
+    if (r.q > lim) r.q = lim;
+    if (r.q < 0) r.q = 0;
+    r.l = c - r.q;
+    r.plain = false;
+    return r;
 }
+
+// LPC lanes of one warp trace a curve together (2 or 4): one half of them
+// computes the x halves of every RK4 stage (beta1 at the stage point, the x
+// component of the direction, the x coordinate), the other the y halves; with
+// 4 lanes each half splits the bilinear sum's two columns.  The lanes trade
+// what the others need by shuffles.  Every value comes from the same
+// operations as in rk4, direction and interior_point (and the sums in the same
+// order), so the points are the same.  All lanes of the warp reach every
+// shuffle: a lane whose curve is done computes on its last point and drops
+// the result.
+template <int LPC>
+struct Lane {
+    static constexpr unsigned kAll = 0xffffffffu;
+    int h, j, lim;   // half (0 x, 1 y), column, largest cell index of the own axis
+    int fam;
+    double limd;
+    const double* field;  // beta1 or beta2
+
+    __device__ __forceinline__ double other(double v) const { return __shfl_xor_sync(kAll, v, LPC / 2); }
+    __device__ __forceinline__ int other(int v) const { return __shfl_xor_sync(kAll, v, LPC / 2); }
+
+    // this half's direction component at the stage point in cell (own index q,
+    // local coordinate l)
+    __device__ __forceinline__ double dir(const GridView& g, int q, double l, double a, bool& bad) const
+    {
+        const int qo = other(q);
+        const double lo = other(l), ao = other(a);
+        const int i = h == 0 ? q : qo, r = h == 0 ? qo : q;
+        const double lx = h == 0 ? l : lo, ax = h == 0 ? a : ao;
+        const double ly = h == 0 ? lo : l, ay = h == 0 ? ao : a;
+        const double* p = field + ((size_t)r * g.nx + i);
+        double v;
+        if constexpr (LPC == 2) {
+            const double w11 = ay * ax, w12 = ay * lx, w21 = ly * ax, w22 = ly * lx;
+            v = w11 * p[0] + w12 * p[1] + w21 * p[g.nx] + w22 * p[g.nx + 1];
+        } else {
+            const double cx = j ? lx : ax;
+            const double t1 = (ay * cx) * p[j], t2 = (ly * cx) * p[g.nx + j];
+            const double o1 = __shfl_xor_sync(kAll, t1, 1), o2 = __shfl_xor_sync(kAll, t2, 1);
+            v = ((t1 + o1) + (j ? o2 : t2)) + (j ? t2 : o2);  // the first sum commutes
+        }
+        const double sq = v * v, vo = other(v), s = sq + other(sq);
+        const double num = fam == 0 ? v : (h == 0 ? vo : -vo);
+        return unit_component(num, s, bad);
+    }
+    __device__ __forceinline__ double dir_at(const GridView& g, double c, bool& bad) const
+    {
+        const Split t = split(c, lim, limd);
+        return dir(g, t.q, t.l, 1.0 - t.l, bad);
+    }
+};
 
 // Trace every curve: number of full RK4 steps M, length L and exit point; the
 // accepted points P_1 .. P_M go to the pool when it has room.  A curve takes
 // full RK4 steps while their end points lie inside Omega_h, then locates its
 // exit within the first step that leaves by kBisectIters bisections of that
-// step, then takes the partial step found.  Each lane runs this as a state
-// machine, and every pass of the loop makes one RK4 step per lane (a full
+// step, then takes the partial step found.  Each curve runs this as a state
+// machine, and every pass of the loop makes one RK4 step per curve (a full
 // step, a bisection trial or the final partial step): the same steps with the
-// same arguments as tracing each curve alone.  A lane that bisected on a
+// same arguments as tracing each curve alone.  A curve that bisected on a
 // branch of its own would add its 61 steps to the warp's time, once for every
 // curve of the warp.
-__global__ void __launch_bounds__(64) k_trace_count(GridView g, int cap, const double* sx0,
+// What bounds it is the count of FP64 instructions of the longest curve's
+// chain (64 cycles each; up to 3 warps share an SM's FP64 pipe for free).  With
+// two warps per 32 curves trading through shared memory, the compiler's square
+// root and division and conversions on the FP64 unit a step took 17 000 cycles,
+// now 10 600: 18.0 -> 11.3 ms at 1024^2 (2200 steps), 37 -> 25 ms at 2048^2.
+template <int LPC>
+__global__ void __launch_bounds__(32) k_trace_count(GridView g, int cap, const double* sx0,
                                                     const double* sy0, const int* nseeds, int* M,
                                                     double* L, double* XE, double* YE,
                                                     long long* cn, int* status, PointPool pool)
 {
-    __shared__ Trade buf[2][2][32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    int fam = 0, s = 0;
-    const bool have = seed_of(nseeds, cap, blockIdx.x * 32 + lane, &fam, &s);
+    const int lane = threadIdx.x;
+    Lane<LPC> me;
+    me.h = (lane / (LPC / 2)) & 1;
+    me.j = LPC == 4 ? lane & 1 : 0;
+    me.lim = me.h == 0 ? g.nx - 2 : g.ny - 2;
+    me.limd = me.lim;
+    me.field = me.h == 0 ? g.beta1 : g.beta2;
+    me.fam = 0;
+    int s = 0;
+    const bool have = seed_of(nseeds, cap, blockIdx.x * (32 / LPC) + lane / LPC, &me.fam, &s);
     const double ds = g.hs / kTraceStepsPerH;
-    const double sx = ds / g.hx, sy = ds / g.hy;  // the step in index units
-    const double stp = w == 0 ? sx : sy;          // this warp's component
-    const double lim = w == 0 ? (double)g.nx : (double)g.ny;
+    const double stp = me.h == 0 ? ds / g.hx : ds / g.hy;  // the step in index units, this half's component
+    const double stp2 = 0.5 * stp, stp6 = stp / 6.0, sixth = 1.0 / 6.0;
+    const double limc = me.h == 0 ? (double)g.nx : (double)g.ny;
+    const int limi = me.h == 0 ? g.nx : g.ny;
     const double cap_len = 10.0 * 2.0 * (g.W + g.H);
-    double X = have ? sx0[s] : 0.0, Y = have ? sy0[s] : 0.0;
-    double lo = 0.0, hi = 1.0, xe = 0.0, ye = 0.0;
+    // the most points with npts * ds <= cap_len
+    long long cap_pts = (long long)(cap_len / ds);
+    for (int k = 0; k < 4 && (cap_pts + 1) * ds <= cap_len; ++k) ++cap_pts;
+    for (int k = 0; k < 4 && cap_pts * ds > cap_len; ++k) --cap_pts;
+    double X = have ? (me.h == 0 ? sx0[s] : sy0[s]) : 0.0;  // this half's coordinate of the last point
+    Split at = split(X, me.lim, me.limd);                   // and its cell
+    double lo = 0.0, hi = 1.0, xe = 0.0;
     long long npts = 0;
     enum { kStep, kBisect, kFinal, kDone, kFailed };
-    int phase = have ? kStep : kDone, it = 0, nb = 0;
-    bool keep = w == 0 && have && pool.n_chunks > 0;  // warp 0 writes the pool
+    int phase = have ? kStep : kDone, it = 0;
+    bool keep = have && me.h == 0 && me.j == 0 && pool.n_chunks > 0;  // one lane writes the pool
     int* tab = pool.tab + (size_t)s * kPoolMaxChunks;
     int chunk = -1;
     if (keep) pool.stored[s] = 0;
     while (__any_sync(0xffffffffu, phase < kDone)) {
         const bool act = phase < kDone;
-        const double mid = 0.5 * (lo + hi);
-        double st = stp;
-        if (phase == kBisect) st = mid * stp;
-        else if (phase == kFinal) st = lo * stp;
+        double st = stp, st2 = stp2, st6 = stp6, mid = 0.5;
+        if (__any_sync(0xffffffffu, phase == kBisect || phase == kFinal)) {
+            mid = 0.5 * (lo + hi);
+            if (phase == kBisect || phase == kFinal) {
+                st = (phase == kBisect ? mid : lo) * stp;
+                st2 = 0.5 * st;
+                // st / 6 (Markstein: the residual of the product with the rounded reciprocal)
+                const double q = st * sixth;
+                st6 = __fma_rn(__fma_rn(-6.0, q, st), sixth, q);
+            }
+        }
         if (act && phase == kStep) npts++;
         bool bad = false;
-        const double c = half_rk4(g, w, fam, w == 0 ? X : Y, st, buf, nb, lane, bad);
+        const double k1 = me.dir(g, at.q, at.l, 1.0 - at.l, bad);
+        const double k2 = me.dir_at(g, X + st2 * k1, bad);
+        const double k3 = me.dir_at(g, X + st2 * k2, bad);
+        const double k4 = me.dir_at(g, X + st * k3, bad);
+        // k1 + 2 k2 + 2 k3 + k4 (the doublings are exact)
+        const double c = X + st6 * (__fma_rn(2.0, k3, __fma_rn(2.0, k2, k1)) + k4);
         // this half of interior_point(snap(Xn), snap(Yn)), then the other's
-        const double cs = snap(c);
-        const bool ok = isfinite(cs) && !(cs < -1.0) && !(cs > lim);
-        const double fc = floor(cs);
-        const int q1 = ok ? (int)fc : 0, q0 = ok && cs == fc ? q1 - 1 : q1;
-        const Trade t = trade(buf, nb, w, lane, Trade{c, 0.0, q0, q1, ok ? 1 : 0});
+        const Split to = split(c, me.lim, me.limd);
+        bool ok;
+        int q0, q1;
+        if (to.plain) {
+            ok = to.qu < limi;
+            q0 = q1 = to.qu;
+        } else {
+            const double cs = snap(c);
+            ok = isfinite(cs) && !(cs < -1.0) && !(cs > limc);
+            const double fc = floor(cs);
+            q1 = ok ? (int)fc : 0;
+            q0 = ok && cs == fc ? q1 - 1 : q1;
+        }
+        const int q0o = me.other(q0), q1o = me.other(q1);
+        const int flags = (ok ? 1 : 0) | (bad ? 2 : 0), fo = me.other(flags);
+        const double co = me.other(c);
         if (!act) continue;
-        const double Xn = w == 0 ? c : t.a, Yn = w == 0 ? t.a : c;
-        if (bad) {
+        if ((flags | fo) & 2) {
             phase = kFailed;
             continue;
         }
         if (phase == kFinal) {
-            xe = Xn;
-            ye = Yn;
+            xe = c;
             phase = kDone;
             continue;
         }
-        bool inside = ok && t.k;
+        bool inside = (flags & fo & 1) != 0;
         if (inside) {
-            const int i0 = w == 0 ? q0 : t.i, i1 = w == 0 ? q1 : t.j;
-            const int r0 = w == 0 ? t.i : q0, r1 = w == 0 ? t.j : q1;
+            const int i0 = me.h == 0 ? q0 : q0o, i1 = me.h == 0 ? q1 : q1o;
+            const int r0 = me.h == 0 ? q0o : q0, r1 = me.h == 0 ? q1o : q1;
             for (int r = r0; r <= r1 && inside; ++r)
                 for (int i = i0; i <= i1; ++i)
                     if (!cell_on(g, i, r)) {
@@ -923,8 +1034,8 @@ __global__ void __launch_bounds__(64) k_trace_count(GridView g, int cap, const d
         }
         if (phase == kStep) {
             if (inside) {
-                X = Xn;
-                Y = Yn;
+                X = c;
+                at = to;
                 if (keep) {  // P_q, q = npts, at pool index q - 1 of the curve
                     long long i = npts - 1;
                     int c2 = (int)(i / kPoolChunk), o = (int)(i % kPoolChunk);
@@ -936,9 +1047,9 @@ __global__ void __launch_bounds__(64) k_trace_count(GridView g, int cap, const d
                             tab[c2] = chunk;
                         }
                     }
-                    if (keep) pool.pts[(size_t)chunk * kPoolChunk + o] = make_double2(X, Y);
+                    if (keep) pool.pts[(size_t)chunk * kPoolChunk + o] = make_double2(c, co);
                 }
-                if (npts * ds > cap_len) phase = kFailed;
+                if (npts > cap_pts) phase = kFailed;
             } else {
                 phase = kBisect;
                 lo = 0.0;
@@ -953,13 +1064,15 @@ __global__ void __launch_bounds__(64) k_trace_count(GridView g, int cap, const d
                     phase = kFinal;
                 } else {
                     xe = X;
-                    ye = Y;
                     phase = kDone;
                 }
             }
         }
     }
-    if (!have || w != 0) return;
+    if (!have || me.j != 0) return;
+    if (phase != kDone) xe = me.h == 0 ? sx0[s] : sy0[s];
+    (me.h == 0 ? XE : YE)[s] = xe;
+    if (me.h != 0) return;
     int m = 0;
     double len = 0.0;
     if (phase == kDone) {
@@ -968,13 +1081,9 @@ __global__ void __launch_bounds__(64) k_trace_count(GridView g, int cap, const d
         if (keep) pool.stored[s] = 1;
     } else {
         atomicOr(status, kErrGeom);
-        xe = sx0[s];
-        ye = sy0[s];
     }
     M[s] = m;
     L[s] = len;
-    XE[s] = xe;
-    YE[s] = ye;
     cn[s] = elements_for(g, len) + 1;
 }
 
@@ -1104,13 +1213,14 @@ __global__ void k_node_data(GridView g, int n_nodes, const double* xs, const dou
     fval[k] = bilin(g, g.f, xs[k], es[k]);
 }
 
+// one warp per line (a thread per line took 155 us at 1024^2)
 __global__ void k_line_of_node(int n_lines, const int* off, int* lon, int* maxlen)
 {
-    int l = blockIdx.x * blockDim.x + threadIdx.x;
+    const int l = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (l >= n_lines) return;
-    int a = off[l], b = off[l + 1];
-    for (int k = a; k < b; ++k) lon[k] = l;
-    atomicMax(maxlen, b - a);
+    const int a = off[l], b = off[l + 1];
+    for (int k = a + lane; k < b; k += 32) lon[k] = l;
+    if (lane == 0) atomicMax(maxlen, b - a);
 }
 
 // ------------------------------------------------- curve -> grid crossings
@@ -1618,7 +1728,7 @@ adr_status finish_family(Problem* p, int fam, TmpGuard& tg, int* status_d)
     TRY(alloc_tmp(tg, &lon, F.n_nodes + 1));
     TRY(alloc_tmp(tg, &maxlen, 1));
     ADR_CUDA_TRY(cudaMemsetAsync(maxlen, 0, sizeof(int), st));
-    k_line_of_node<<<blocks_for(F.n_lines), kThreads, 0, st>>>(F.n_lines, F.off, lon, maxlen);
+    k_line_of_node<<<blocks_for(32LL * F.n_lines), kThreads, 0, st>>>(F.n_lines, F.off, lon, maxlen);
     ADR_CUDA_TRY(cudaMemcpyAsync(&F.max_nodes, maxlen, sizeof(int), cudaMemcpyDeviceToHost, st));
     ADR_CUDA_TRY(cudaStreamSynchronize(st));
     // curves sorted longest first
@@ -1814,7 +1924,7 @@ adr_status build_curved_both(Problem* p, int* status_d, TmpGuard& tg)
         if (chunks > max_chunks) chunks = max_chunks;
         pool.n_chunks = (unsigned int)chunks;
         void* q = nullptr;
-        if (cudaMalloc(&q, (size_t)pool.n_chunks * kPoolChunk * sizeof(double2)) != cudaSuccess) {
+        if (pool_alloc(&q, (size_t)pool.n_chunks * kPoolChunk * sizeof(double2), st) != cudaSuccess) {
             cudaGetLastError();  // no pool: every curve is re-traced
             pool.n_chunks = 0;
         } else {
@@ -1826,9 +1936,14 @@ adr_status build_curved_both(Problem* p, int* status_d, TmpGuard& tg)
             ADR_CUDA_TRY(cudaMemsetAsync(pool.next, 0, sizeof(unsigned int), st));
         }
     }
-    // 32 curves per block of two warps: the per-curve traces are serial chains
-    k_trace_count<<<blocks_for(tot, 32), 64, 0, st>>>(g, cap, sx, sy, cnt + 1, M, L, XE, YE, cn,
-                                                      status_d, pool);
+    // 4 lanes per curve while that leaves at most 3 warps per SM (more share its
+    // FP64 pipe and slow each other down), 2 beyond
+    if (blocks_for(tot, 8) <= 3 * p->n_sm)
+        k_trace_count<4><<<blocks_for(tot, 8), 32, 0, st>>>(g, cap, sx, sy, cnt + 1, M, L, XE, YE, cn, status_d,
+                                                            pool);
+    else
+        k_trace_count<2><<<blocks_for(tot, 16), 32, 0, st>>>(g, cap, sx, sy, cnt + 1, M, L, XE, YE, cn, status_d,
+                                                             pool);
     k_scan<<<1, 1024, 0, st>>>(cn, on, ns[0]);
     k_scan<<<1, 1024, 0, st>>>(cn + cap, on + cap, ns[1]);
     long long tn[2] = {0, 0};
@@ -1880,7 +1995,7 @@ adr_status build_transfer(Problem* p)
         TRY(alloc_tmp(tg, &lon[f], F.n_nodes + 1));
         TRY(alloc_tmp(tg, &maxlen, 1));
         ADR_CUDA_TRY(cudaMemsetAsync(maxlen, 0, sizeof(int), st));
-        k_line_of_node<<<blocks_for(F.n_lines), kThreads, 0, st>>>(F.n_lines, F.off, lon[f], maxlen);
+        k_line_of_node<<<blocks_for(32LL * F.n_lines), kThreads, 0, st>>>(F.n_lines, F.off, lon[f], maxlen);
     }
     for (int tf = 0; tf < 2; ++tf) {
         Family& T = p->fam[tf];
