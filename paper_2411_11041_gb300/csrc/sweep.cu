@@ -7,7 +7,7 @@
 //                 curve nodes (§6.1), right-hand side F - S u, the factored
 //                 elimination, curve values u + dt d out; a block of BS threads
 //                 holds BS/T curves of T threads each.
-//  k_grid_map     one thread per grid node: curve -> grid interpolation through
+//  k_grid_map     tiles of 32 x 8 nodes, one per thread: curve -> grid interpolation through
 //                 the nearest crossings on the node's row and column (§6), with
 //                 the relative-update norms fused in.
 //  k_check        one block: convergence test and the CUDA-graph loop condition.
@@ -1075,39 +1075,32 @@ __device__ __forceinline__ void map_prefetch(const GridArgs& a, long long k, Map
     p.c3 = c[3];
 }
 
-// curve -> grid map over nodes first, first + stride, ... of one problem into
-// out; adds the norms' sums of the calling thread (against prev).  COH: the
-// curve values and the previous state come from this launch, and the first
-// node's tables from pre.
-template <bool NORMS, bool COH>
+// curve -> grid map over nodes first, first + stride, ... into out inside the
+// one-launch iteration, the first node's tables from pre; adds the norms' sums
+// of the calling thread (against prev)
+template <bool NORMS>
 __device__ __forceinline__ void grid_map_nodes(const GridArgs& a, double* __restrict__ out, const double* prev,
                                                long long first, long long stride, double& dd, double& uu,
-                                               const MapPre* pre = nullptr)
+                                               const MapPre& pre)
 {
-    const double* v = a.v;
+    const double* v = a.v;  // written by other blocks of this launch: plain loads
     const long long N = (long long)a.nx * a.ny;
     for (long long k = first; k < N; k += stride) {
         double val = 0.0;
         MapPre q;
-        if (COH && k == first) {
-            q = *pre;
-        } else if (COH) {
-            map_prefetch(a, k, q);
-        } else {
-            q.in = a.ntype[k] == kInterior;
-            if (q.in) map_prefetch(a, k, q);
-        }
+        if (k == first) q = pre;
+        else map_prefetch(a, k, q);
         if (q.in) {
-            val = q.c0.x * ld_state<COH>(v + q.g.x);
-            val = fma(q.c0.y, ld_state<COH>(v + q.g.x + 1), val);
-            val = fma(q.c1.x, ld_state<COH>(v + q.g.y), val);
-            val = fma(q.c1.y, ld_state<COH>(v + q.g.y + 1), val);
-            val = fma(q.c2.x, ld_state<COH>(v + q.g.z), val);
-            val = fma(q.c2.y, ld_state<COH>(v + q.g.z + 1), val);
-            val = fma(q.c3.x, ld_state<COH>(v + q.g.w), val);
-            val = fma(q.c3.y, ld_state<COH>(v + q.g.w + 1), val);
+            val = q.c0.x * v[q.g.x];
+            val = fma(q.c0.y, v[q.g.x + 1], val);
+            val = fma(q.c1.x, v[q.g.y], val);
+            val = fma(q.c1.y, v[q.g.y + 1], val);
+            val = fma(q.c2.x, v[q.g.z], val);
+            val = fma(q.c2.y, v[q.g.z + 1], val);
+            val = fma(q.c3.x, v[q.g.w], val);
+            val = fma(q.c3.y, v[q.g.w + 1], val);
             if (NORMS) {
-                double dlt = val - prev[k];
+                const double dlt = val - prev[k];
                 dd = fma(dlt, dlt, dd);
                 uu = fma(val, val, uu);
             }
@@ -1116,15 +1109,51 @@ __device__ __forceinline__ void grid_map_nodes(const GridArgs& a, double* __rest
     }
 }
 
-// the same into the state buffer of the step's parity
+// The same into the state buffer of the step's parity, block blk of nblk over
+// tiles of 32 x 8 nodes (a warp per row).  What bounds it is the FP64 pipe (8
+// products and, with the norms, 3 more per node: 63 and 87 us at 2048^2) and
+// L1's gather throughput (77 to 81 % busy): a curve that passes a tile is met by
+// several of its rows, so the tile shape decides how many of the 8 curve values
+// L1 already holds.  Measured at 2048^2 / 1024^2, without and with norms: runs
+// of 256 nodes along a row 84.2 and 109.0 / 23.3 and 34.9 us, 64 x 4 79.8 and
+// 98.4, 32 x 8 79.4 and 95.2 / 21.0 and 31.0, 16 x 16 80.2 and 96.4, 8 x 32 82.6
+// and 98.4.
 template <bool NORMS>
-__device__ __forceinline__ void grid_map_body(const GridArgs& a, long long first, long long stride,
-                                              double& dd, double& uu)
+__device__ __forceinline__ void grid_map_tiles(const GridArgs& a, int blk, int nblk, double& dd, double& uu)
 {
-    int it = a.state ? a.state->iter : 0;
-    double* out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
-    const double* prev = (it & 1) ? a.prev_odd : a.prev_even;
-    grid_map_nodes<NORMS, false>(a, out, prev, first, stride, dd, uu);
+    constexpr int TX = 32, TY = kGridThreads / TX;
+    const int it = a.state ? a.state->iter : 0;
+    double* __restrict__ out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
+    const double* __restrict__ prev = (it & 1) ? a.prev_odd : a.prev_even;
+    const double* __restrict__ v = a.v;
+    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+    const int ntx = (a.nx + TX - 1) / TX, nty = (a.ny + TY - 1) / TY;
+    const long long nt = (long long)ntx * nty;
+    for (long long t = blk; t < nt; t += nblk) {
+        const int by = (int)(t / ntx), x = (int)(t - (long long)by * ntx) * TX + tx, y = by * TY + ty;
+        if (x >= a.nx || y >= a.ny) continue;
+        const long long k = (long long)y * a.nx + x;
+        double val = 0.0;
+        if (a.ntype[k] == kInterior) {
+            const int4 g = *reinterpret_cast<const int4*>(a.mg + 4 * k);
+            const double2* c = reinterpret_cast<const double2*>(a.mc + 8 * k);
+            const double2 c0 = c[0], c1 = c[1], c2 = c[2], c3 = c[3];
+            val = c0.x * __ldg(v + g.x);
+            val = fma(c0.y, __ldg(v + g.x + 1), val);
+            val = fma(c1.x, __ldg(v + g.y), val);
+            val = fma(c1.y, __ldg(v + g.y + 1), val);
+            val = fma(c2.x, __ldg(v + g.z), val);
+            val = fma(c2.y, __ldg(v + g.z + 1), val);
+            val = fma(c3.x, __ldg(v + g.w), val);
+            val = fma(c3.y, __ldg(v + g.w + 1), val);
+            if (NORMS) {
+                const double dlt = val - prev[k];
+                dd = fma(dlt, dlt, dd);
+                uu = fma(val, val, uu);
+            }
+        }
+        out[k] = val;
+    }
 }
 
 template <bool NORMS>
@@ -1132,8 +1161,7 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_map(GridArgs a)
 {
     if (a.state && a.state->done) return;
     double dd = 0.0, uu = 0.0;
-    grid_map_body<NORMS>(a, blockIdx.x * (long long)blockDim.x + threadIdx.x,
-                         (long long)gridDim.x * blockDim.x, dd, uu);
+    grid_map_tiles<NORMS>(a, blockIdx.x, gridDim.x, dd, uu);
     if (NORMS) block_sum2(dd, uu, a.partial + 2 * blockIdx.x);
 }
 
@@ -1155,8 +1183,7 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_map_batch(const GridArgs*
         const GridArgs& a = table[2 * p + fam];
         if (a.state->done) continue;  // uniform per block
         double dd = 0.0, uu = 0.0;
-        grid_map_body<NORMS>(a, (long long)lb * blockDim.x + threadIdx.x,
-                             (long long)nblk[p] * blockDim.x, dd, uu);
+        grid_map_tiles<NORMS>(a, lb, nblk[p], dd, uu);
         if (NORMS) block_sum2(dd, uu, a.partial + 2 * lb);
         __syncthreads();  // block_sum2's shared arrays are reused
     }
@@ -1724,7 +1751,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_con
         loop_solve<GS, 0, REF>(a, u, hp, sm, corr, w0, pre);
         map_prefetch(a.g[0], first, mp);
         if (!grid_barrier(a.state, epoch)) return;
-        grid_map_nodes<false, true>(a.g[0], a.g[0].out_even, nullptr, first, stride, dd, uu, &mp);
+        grid_map_nodes<false>(a.g[0], a.g[0].out_even, nullptr, first, stride, dd, uu, mp);
         loop_prefetch(a.c[1], w1, pre);
         if (!grid_barrier(a.state, epoch)) return;
         if (REF && blockIdx.x == 0 && threadIdx.x == 0) a.state->corr_loop[(iter + 1) & 1] = 0ull;
@@ -1732,13 +1759,13 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_con
         map_prefetch(a.g[1], first, mp);
         if (!grid_barrier(a.state, epoch)) return;
         if (!a.norms) {
-            grid_map_nodes<false, true>(a.g[1], un, nullptr, first, stride, dd, uu, &mp);
+            grid_map_nodes<false>(a.g[1], un, nullptr, first, stride, dd, uu, mp);
             loop_prefetch(a.c[0], w0, pre);
             if (++iter >= a.max_iter) break;
             if (!grid_barrier(a.state, epoch)) return;
             continue;
         }
-        grid_map_nodes<true, true>(a.g[1], un, u, first, stride, dd, uu, &mp);
+        grid_map_nodes<true>(a.g[1], un, u, first, stride, dd, uu, mp);
         loop_prefetch(a.c[0], w0, pre);
         if (warp < nwarp) {
             const double v = warp_sum2(dd, uu, lane);
