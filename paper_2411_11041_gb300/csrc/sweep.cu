@@ -29,6 +29,11 @@ namespace {
 
 constexpr int kCmax = 16;      // most rows per thread of the curve solve (kept in shared memory)
 constexpr int kGridThreads = 256;
+// 32 x 8-node tiles of one block of a batch's maps: a lone large problem at the
+// batch's end still spreads over every SM.  48 problems / the last one alone
+// (630 000 nodes), a split step: 2 tiles 1565 / 135 us, 4 1526 / 135, 8 1484 /
+// 149, 16 1441 / 192 (a block per tile or two: 1799 / 137)
+constexpr int kBatchTiles = 4;
 
 // ---------------------------------------------------------------- curves
 // The curve systems A = M + theta dt S are fixed for a given (theta, dt,
@@ -921,28 +926,29 @@ struct GridArgs {
     double* partial;   // [2 * gridDim.x] sums of (u - u_prev)^2 and u^2
 };
 
+// (dd, uu) summed over the warp: lane 0 gets dd, lane 16 uu (5 additions, as
+// an FP64 warp instruction costs the same for 1 or 32 lanes)
+__device__ __forceinline__ double warp_sum2(double dd, double uu, int lane)
+{
+    double v = lane < 16 ? dd : uu;
+    const double w = lane < 16 ? uu : dd;
+    v += __shfl_xor_sync(0xffffffffu, w, 16);
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
 // block sum of (dd, uu) into dst[0..1]
 __device__ __forceinline__ void block_sum2(double dd, double uu, double* dst)
 {
-    __shared__ double sd[kGridThreads / 32], su[kGridThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        dd += __shfl_down_sync(0xffffffffu, dd, o);
-        uu += __shfl_down_sync(0xffffffffu, uu, o);
-    }
-    int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
-        sd[w] = dd;
-        su[w] = uu;
-    }
+    __shared__ double red[2][kGridThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double v = warp_sum2(dd, uu, lane);
+    if ((lane & 15) == 0) red[lane >> 4][w] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double td = 0, tu = 0;
-        for (int q = 0; q < kGridThreads / 32; ++q) {
-            td += sd[q];
-            tu += su[q];
-        }
-        dst[0] = td;
-        dst[1] = tu;
+    if (threadIdx.x < 2) {  // both sums in one warp's instructions
+        double t = 0.0;
+        for (int q = 0; q < kGridThreads / 32; ++q) t += red[threadIdx.x][q];
+        dst[threadIdx.x] = t;
     }
 }
 
@@ -1165,8 +1171,48 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_map(GridArgs a)
     if (NORMS) block_sum2(dd, uu, a.partial + 2 * blockIdx.x);
 }
 
+// A batch's map blocks (problem, local block): a persistent block walks the
+// active ones, the next one's indices loaded while it works on the current one
+struct BlockWalk {
+    const int *list, *prob, *local;
+    int n, ii, bk_next, p, lb;
+    __device__ __forceinline__ BlockWalk(const int* l, int n_act, const int* pr, const int* lo)
+        : list(l), prob(pr), local(lo), n(n_act), ii(blockIdx.x), bk_next(-1), p(0), lb(0)
+    {
+        if (ii < n) {
+            const int bk = list[ii];
+            p = prob[bk];
+            lb = local[bk];
+            if (ii + (int)gridDim.x < n) bk_next = list[ii + gridDim.x];
+        }
+    }
+    __device__ __forceinline__ bool valid() const { return ii < n; }
+    // issue the loads of the next block's problem (call before the work)
+    int p_next, lb_next, bk_next2;
+    __device__ __forceinline__ void ahead()
+    {
+        bk_next2 = -1;
+        if (bk_next >= 0) {
+            p_next = prob[bk_next];
+            lb_next = local[bk_next];
+            if (ii + 2 * (int)gridDim.x < n) bk_next2 = list[ii + 2 * gridDim.x];
+        }
+    }
+    __device__ __forceinline__ void next()
+    {
+        p = p_next;
+        lb = lb_next;
+        bk_next = bk_next2;
+        ii += gridDim.x;
+    }
+};
+
 // batched map: block b works for problem blk_prob[b] as its local block
-// blk_local[b] of nblk[p] (table entries 2p + fam); partial sums per local block
+// blk_local[b] of nblk[p] (table entries 2p + fam); partial sums per local block.
+// A problem has a block per kBatchTiles tiles: with a block per tile or two (608
+// a problem) the norms' block sums alone took 116 us of SM time a step for 48
+// problems of 13 M nodes (10 FP64 additions a warp, 24 000 blocks), 551 us in
+// all.
 template <bool NORMS>
 __global__ void __launch_bounds__(kGridThreads) k_grid_map_batch(const GridArgs* __restrict__ table,
                                                                 int fam, const int* blk_prob,
@@ -1175,17 +1221,16 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_map_batch(const GridArgs*
                                                                 const int* act_count, const int* sel)
 {
     const int cur = *sel;
-    const int* list = act_blocks[cur];
-    const int n_act = act_count[cur * 7 + 6];
-    for (int ii = blockIdx.x; ii < n_act; ii += gridDim.x) {
-        int bk = list[ii];
-        int p = blk_prob[bk], lb = blk_local[bk];
-        const GridArgs& a = table[2 * p + fam];
+    for (BlockWalk w(act_blocks[cur], act_count[cur * 7 + 6], blk_prob, blk_local); w.valid(); w.next()) {
+        w.ahead();
+        const GridArgs& a = table[2 * w.p + fam];
         if (a.state->done) continue;  // uniform per block
         double dd = 0.0, uu = 0.0;
-        grid_map_tiles<NORMS>(a, lb, nblk[p], dd, uu);
-        if (NORMS) block_sum2(dd, uu, a.partial + 2 * lb);
-        __syncthreads();  // block_sum2's shared arrays are reused
+        grid_map_tiles<NORMS>(a, w.lb, nblk[w.p], dd, uu);
+        if (NORMS) {
+            block_sum2(dd, uu, a.partial + 2 * w.lb);
+            __syncthreads();  // its shared array is reused
+        }
     }
 }
 
@@ -1208,15 +1253,13 @@ __global__ void __launch_bounds__(256) k_gather_batch(const GatherArgs* __restri
                                                       const int* act_count, const int* sel)
 {
     const int cur = *sel;
-    const int* list = act_blocks[cur];
-    const int n_act = act_count[cur * 7 + 6];
-    for (int ii = blockIdx.x; ii < n_act; ii += gridDim.x) {
-        const int bk = list[ii], pr = blk_prob[bk], lb = blk_local[bk];
-        const GatherArgs& g = table[2 * pr + fam];
+    for (BlockWalk w(act_blocks[cur], act_count[cur * 7 + 6], blk_prob, blk_local); w.valid(); w.next()) {
+        w.ahead();
+        const GatherArgs& g = table[2 * w.p + fam];
         if (g.state->done) continue;
         const double* __restrict__ u = (g.state->iter & 1) ? g.u_odd : g.u_even;
-        const long long stride = (long long)nblk[pr] * blockDim.x;
-        for (long long k = (long long)lb * blockDim.x + threadIdx.x; k < g.n; k += stride) {
+        const long long stride = (long long)nblk[w.p] * blockDim.x;
+        for (long long k = (long long)w.lb * blockDim.x + threadIdx.x; k < g.n; k += stride) {
             const int c = __ldg(g.ncell + k);
             double v = 0.0;
             if (c >= 0) {
@@ -1703,17 +1746,6 @@ __device__ __forceinline__ void loop_solve(const LoopArgs& a, const double* u, b
         use = false;
         if (q < units) loop_unit<GS, FAM>(a, q, gt, w);
     }
-}
-
-// (dd, uu) summed over the warp: lane 0 gets dd, lane 16 uu (5 additions, as
-// an FP64 warp instruction costs the same for 1 or 32 lanes)
-__device__ __forceinline__ double warp_sum2(double dd, double uu, int lane)
-{
-    double v = lane < 16 ? dd : uu;
-    const double w = lane < 16 ? uu : dd;
-    v += __shfl_xor_sync(0xffffffffu, w, 16);
-    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
 }
 
 template <int GS, bool REF>
@@ -2697,7 +2729,10 @@ adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const 
         // work items of both families share the item lists (the B and G
         // curves of a problem differ, so items are per family): the batch
         // keeps one list per family and set
-        nb[i] = grid_map_blocks(p);
+        {
+            const long long tiles = (long long)((p->grid.nx + 31) / 32) * ((p->grid.ny + 7) / 8);
+            nb[i] = (int)std::min<long long>(grid_map_blocks(p), (tiles + kBatchTiles - 1) / kBatchTiles);
+        }
         for (int q = 0; q < nb[i]; ++q) {
             bp.push_back(i);
             bl.push_back(q);
