@@ -100,6 +100,7 @@ __device__ __forceinline__ void aa_dots_body(const AaArgs& a, long long start, l
 template <int M>
 __global__ void __launch_bounds__(kAaThreads) k_aa_dots(AaArgs a)
 {
+    step_entry();
     if (a.state->done || a.state->iter < 1) return;
     aa_dots_body<M>(a, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x,
                     blockIdx.x);
@@ -183,6 +184,7 @@ __device__ void aa_solve_body(const AaArgs& a, int nblocks)
 
 __global__ void k_aa_solve(AaArgs a, int nblocks)
 {
+    step_entry();
     if (a.state->done || a.state->iter < 1) return;
     aa_solve_body(a, nblocks);
 }
@@ -213,6 +215,7 @@ __device__ __forceinline__ void aa_update_body(const AaArgs& a, long long start,
 template <int M>
 __global__ void __launch_bounds__(kAaThreads) k_aa_update(AaArgs a)
 {
+    step_entry();
     if (a.state->done || a.state->iter < 1) return;
     aa_update_body<M>(a, blockIdx.x * (long long)blockDim.x + threadIdx.x, (long long)gridDim.x * blockDim.x);
 }
@@ -225,6 +228,7 @@ __global__ void __launch_bounds__(kAaThreads) k_aa_update(AaArgs a)
 template <int M>
 __global__ void __launch_bounds__(kAaThreads) k_aa_dots_batch(const AaArgs* __restrict__ table, AaBatchView v)
 {
+    step_entry();
     const int cur = *v.sel;
     const int* list = v.act_blocks[cur];
     const int n_act = v.act_count[cur * 7 + 6];
@@ -239,6 +243,7 @@ __global__ void __launch_bounds__(kAaThreads) k_aa_dots_batch(const AaArgs* __re
 
 __global__ void k_aa_solve_batch(const AaArgs* __restrict__ table, AaBatchView v)
 {
+    step_entry();
     const AaArgs& a = table[blockIdx.x];
     if (a.m == 0 || a.state->done || a.state->iter < 1) return;
     aa_solve_body(a, v.nblk[blockIdx.x]);
@@ -247,6 +252,7 @@ __global__ void k_aa_solve_batch(const AaArgs* __restrict__ table, AaBatchView v
 template <int M>
 __global__ void __launch_bounds__(kAaThreads) k_aa_update_batch(const AaArgs* __restrict__ table, AaBatchView v)
 {
+    step_entry();
     const int cur = *v.sel;
     const int* list = v.act_blocks[cur];
     const int n_act = v.act_count[cur * 7 + 6];
@@ -298,9 +304,9 @@ adr_status launch_anderson(Problem* p)
     switch (m) {
 #define ADR_AA_CASE(M_)                                        \
     case M_:                                                   \
-        k_aa_dots<M_><<<nb, kAaThreads, 0, st>>>(a);           \
-        k_aa_solve<<<1, 32 * (kAaMax + 1), 0, st>>>(a, nb);    \
-        k_aa_update<M_><<<nb, kAaThreads, 0, st>>>(a);         \
+        launch_step(k_aa_dots<M_>, nb, kAaThreads, 0, st, a);           \
+        launch_step(k_aa_solve, 1, 32 * (kAaMax + 1), 0, st, a, nb);    \
+        launch_step(k_aa_update<M_>, nb, kAaThreads, 0, st, a);         \
         break;
         ADR_AA_CASE(1)
         ADR_AA_CASE(2)
@@ -371,9 +377,9 @@ adr_status launch_anderson_batch(const AaBatchView& v, cudaStream_t st)
     switch (v.mmax) {
 #define ADR_AA_CASE(M_)                                                   \
     case M_:                                                              \
-        k_aa_dots_batch<M_><<<v.grid, kAaThreads, 0, st>>>(t, v);         \
-        k_aa_solve_batch<<<v.n, 32 * (kAaMax + 1), 0, st>>>(t, v);        \
-        k_aa_update_batch<M_><<<v.grid, kAaThreads, 0, st>>>(t, v);       \
+        launch_step(k_aa_dots_batch<M_>, v.grid, kAaThreads, 0, st, t, v);         \
+        launch_step(k_aa_solve_batch, v.n, 32 * (kAaMax + 1), 0, st, t, v);        \
+        launch_step(k_aa_update_batch<M_>, v.grid, kAaThreads, 0, st, t, v);       \
         break;
         ADR_AA_CASE(1)
         ADR_AA_CASE(2)

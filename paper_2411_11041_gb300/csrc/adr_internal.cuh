@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "adr.h"
@@ -244,6 +245,38 @@ adr_status dev_alloc(Problem* p, T** ptr, size_t count)
     *ptr = static_cast<T*>(q);
     return ADR_OK;
 }
+
+// Programmatic dependent launch of the split step's kernels: a kernel is put
+// on the SMs as soon as its predecessor's last block has left, its launch
+// work done before that, and waits there until the predecessor has finished
+// and its writes are visible (step_entry, the first statement of every such
+// kernel, before anything is read or any thread returns).  About 0.7 us a
+// kernel: 513^2 74.5 -> 71.7 us a step, 1024^2 146 -> 143, direct transfer at
+// 257^2 32.2 -> 30.1.  Letting the successor in earlier (launch_dependents at
+// its predecessor's start) costs 25 to 40 %: the blocks that wait hold shared
+// memory that is the running kernel's L1.
+#ifdef __CUDACC__
+__device__ __forceinline__ void step_entry()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline void launch_step(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);  // an error is the caller's cudaGetLastError
+}
+#endif
 
 // setup (geometry.cu)
 adr_status build_geometry(Problem* p, const uint8_t* mask);

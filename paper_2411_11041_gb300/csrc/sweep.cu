@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(256) k_gather_grid(long long n, const int* __r
                                                      const double* u_even, const double* u_odd,
                                                      const IterState* state, double* __restrict__ out)
 {
+    step_entry();
     if (state && state->done) return;
     const double* __restrict__ u = (state && (state->iter & 1)) ? u_odd : u_even;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
@@ -807,6 +808,7 @@ __global__ void __launch_bounds__(BS, BS == 256 ? 4 : (BS == 512 ? 2 : 1)) k_cur
                                                     const int* item_curve, const double* lanec,
                                                     const float* lanec32)
 {
+    step_entry();
     if (a.state && a.state->done) return;
     extern __shared__ __align__(16) unsigned char smem[];
     const int T = item_T[blockIdx.x];
@@ -848,6 +850,7 @@ __global__ void __launch_bounds__(BS, BS == 256 ? 4 : (BS == 512 ? 2 : 1)) k_cur
                                                     const int* item_curve, const double* lanec,
                                                     const float* lanec32)
 {
+    step_entry();
     if (a.state && a.state->done) return;
     extern __shared__ __align__(16) unsigned char smem[];
     const size_t lo = (size_t)blockIdx.x * Items<BS>::NF * BS;
@@ -868,6 +871,7 @@ __global__ void __launch_bounds__(GS, 1024 / GS) k_curve_solve_slice(CurveArgs a
                                                                      const int* item_curve, const double* lanec,
                                                                      const float* lanec32)
 {
+    step_entry();
     if (a.state && a.state->done) return;
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int PER = 256 / GS, NF = Items<256>::NF;
@@ -892,6 +896,7 @@ __global__ void __launch_bounds__(BS) k_curve_solve_batch(const CurveArgs* __res
                                                           const BatchItem* __restrict__ items,
                                                           ActiveLists act, int set)
 {
+    step_entry();
     extern __shared__ __align__(16) unsigned char smem[];
     const int cur = *act.sel;
     const int* list = act.items[cur][FAM][set];
@@ -974,6 +979,7 @@ struct XferArgs {
 template <bool NORMS>
 __global__ void __launch_bounds__(kGridThreads) k_curve_xfer(XferArgs a)
 {
+    step_entry();
     if (a.state && a.state->done) return;
     const int it = a.state ? a.state->iter : 0;
     double* __restrict__ out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
@@ -1165,6 +1171,7 @@ __device__ __forceinline__ void grid_map_tiles(const GridArgs& a, int blk, int n
 template <bool NORMS>
 __global__ void __launch_bounds__(kGridThreads) k_grid_map(GridArgs a)
 {
+    step_entry();
     if (a.state && a.state->done) return;
     double dd = 0.0, uu = 0.0;
     grid_map_tiles<NORMS>(a, blockIdx.x, gridDim.x, dd, uu);
@@ -1220,6 +1227,7 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_map_batch(const GridArgs*
                                                                 const int* const* act_blocks,
                                                                 const int* act_count, const int* sel)
 {
+    step_entry();
     const int cur = *sel;
     for (BlockWalk w(act_blocks[cur], act_count[cur * 7 + 6], blk_prob, blk_local); w.valid(); w.next()) {
         w.ahead();
@@ -1252,6 +1260,7 @@ __global__ void __launch_bounds__(256) k_gather_batch(const GatherArgs* __restri
                                                       const int* nblk, const int* const* act_blocks,
                                                       const int* act_count, const int* sel)
 {
+    step_entry();
     const int cur = *sel;
     for (BlockWalk w(act_blocks[cur], act_count[cur * 7 + 6], blk_prob, blk_local); w.valid(); w.next()) {
         w.ahead();
@@ -1282,6 +1291,7 @@ __global__ void __launch_bounds__(256) k_gather_batch(const GatherArgs* __restri
 __global__ void k_batch_compact(ActiveLists act, const BatchItem* const* items, const int* n_items,
                                 const int* blk_prob, int n_blk, IterState* const* states)
 {
+    step_entry();
     if (!*act.changed) return;
     const int cur = *act.sel, nxt = cur ^ 1;
     long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -1312,6 +1322,7 @@ __global__ void k_batch_compact(ActiveLists act, const BatchItem* const* items, 
 // make the rebuilt lists current and clear the other buffer's counters
 __global__ void k_batch_flip(ActiveLists act)
 {
+    step_entry();
     if (!*act.changed) return;
     int nxt = *act.sel ^ 1;
     for (int q = 0; q < kCountPerBuf; ++q) act.count[(nxt ^ 1) * kCountPerBuf + q] = 0;
@@ -1347,6 +1358,7 @@ __global__ void k_check_batch(IterState* const* states, const double* const* par
                               const int* nblk, int n_prob, const double* tols, const int* max_iters,
                               unsigned int* ticket, cudaGraphConditionalHandle handle, int* changed)
 {
+    step_entry();
     int p = blockIdx.x;
     IterState* st = states[p];
     const double tol = tols[p];
@@ -1407,6 +1419,7 @@ __global__ void k_check_batch(IterState* const* states, const double* const* par
 __global__ void k_check(IterState* st, const double* partial, int nblocks, double tol,
                         int max_iter, cudaGraphConditionalHandle handle, int use_cond)
 {
+    step_entry();
     if (st->done) {
         if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(handle, 0);
         return;
@@ -2270,11 +2283,11 @@ adr_status launch_line_solve(Problem* p, int fam, double dt, const double* u_eve
     if (I_.count) {                                                                                \
         const size_t sm = solve_smem<BS_>(R);                                                      \
         if (ref) {                                                                                 \
-            if (fam == 0) k_curve_solve<BS_, 0, true><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
-            else k_curve_solve<BS_, 1, true><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
+            if (fam == 0) launch_step(k_curve_solve<BS_, 0, true>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
+            else launch_step(k_curve_solve<BS_, 1, true>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
         } else {                                                                                   \
-            if (fam == 0) k_curve_solve<BS_, 0, false><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
-            else k_curve_solve<BS_, 1, false><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
+            if (fam == 0) launch_step(k_curve_solve<BS_, 0, false>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
+            else launch_step(k_curve_solve<BS_, 1, false>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
         }                                                                                          \
     }
     ADR_SOLVE(1024, F.iset[2])
@@ -2314,11 +2327,11 @@ adr_status launch_line_solve_dir(Problem* p, int fam, double dt, const double* u
     if (I_.count) {                                                                                \
         const size_t sm = solve_smem<BS_>(R);                                                      \
         if (ref) {                                                                                 \
-            if (fam == 0) k_curve_solve_dir<BS_, 0, true><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
-            else k_curve_solve_dir<BS_, 1, true><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
+            if (fam == 0) launch_step(k_curve_solve_dir<BS_, 0, true>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
+            else launch_step(k_curve_solve_dir<BS_, 1, true>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
         } else {                                                                                   \
-            if (fam == 0) k_curve_solve_dir<BS_, 0><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
-            else k_curve_solve_dir<BS_, 1><<<I_.count, BS_, sm, st>>>(a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
+            if (fam == 0) launch_step(k_curve_solve_dir<BS_, 0>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32); \
+            else launch_step(k_curve_solve_dir<BS_, 1>, I_.count, BS_, sm, st, a, I_.T, I_.curve, I_.lanec, I_.lanec32);         \
         }                                                                                          \
     }
     ADR_SOLVE_DIR(1024, F.iset[2])
@@ -2330,11 +2343,11 @@ adr_status launch_line_solve_dir(Problem* p, int fam, double dt, const double* u
         const size_t sm = solve_smem<GS_>(R);                                                      \
         const int nb = I0.count * (256 / GS_);                                                     \
         if (ref) {                                                                                 \
-            if (fam == 0) k_curve_solve_slice<GS_, 0, true><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32); \
-            else k_curve_solve_slice<GS_, 1, true><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32);         \
+            if (fam == 0) launch_step(k_curve_solve_slice<GS_, 0, true>, nb, GS_, sm, st, a, I0.T, I0.curve, I0.lanec, I0.lanec32); \
+            else launch_step(k_curve_solve_slice<GS_, 1, true>, nb, GS_, sm, st, a, I0.T, I0.curve, I0.lanec, I0.lanec32);         \
         } else {                                                                                   \
-            if (fam == 0) k_curve_solve_slice<GS_, 0, false><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32); \
-            else k_curve_solve_slice<GS_, 1, false><<<nb, GS_, sm, st>>>(a, I0.T, I0.curve, I0.lanec, I0.lanec32);         \
+            if (fam == 0) launch_step(k_curve_solve_slice<GS_, 0, false>, nb, GS_, sm, st, a, I0.T, I0.curve, I0.lanec, I0.lanec32); \
+            else launch_step(k_curve_solve_slice<GS_, 1, false>, nb, GS_, sm, st, a, I0.T, I0.curve, I0.lanec, I0.lanec32);         \
         }                                                                                          \
     }
     if (gs == 32) ADR_SLICE(32)
@@ -2366,7 +2379,7 @@ adr_status launch_substep_solve(Problem* p, int fam, double dt, const double* u_
     if (!F.ug) return launch_line_solve(p, fam, dt, u_even, u_odd, use_state, 0);
     const long long n = F.n_nodes;
     const int blocks = gather_blocks(F);
-    k_gather_grid<<<blocks, 256, 0, p->stream>>>(n, F.ncell, F.nw, p->grid.nx, u_even, u_odd,
+    launch_step(k_gather_grid, blocks, 256, 0, p->stream, n, F.ncell, F.nw, p->grid.nx, u_even, u_odd,
                                                  use_state ? p->state : nullptr, F.ug);
     ADR_CUDA_TRY(cudaGetLastError());
     return launch_line_solve_dir(p, fam, dt, F.ug, F.ug, use_state);
@@ -2377,7 +2390,7 @@ adr_status launch_gather_pass(Problem* p, int fam, const double* u)
 {
     Family& F = p->fam[fam];
     if (!F.ug) return ADR_OK;
-    k_gather_grid<<<gather_blocks(F), 256, 0, p->stream>>>(F.n_nodes, F.ncell, F.nw, p->grid.nx, u, u,
+    launch_step(k_gather_grid, gather_blocks(F), 256, 0, p->stream, F.n_nodes, F.ncell, F.nw, p->grid.nx, u, u,
                                                              nullptr, F.ug);
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
@@ -2411,8 +2424,8 @@ adr_status launch_xfer(Problem* p, int to_fam, const double* v, double* out_even
     a.parity_shift = shift;
     a.partial = p->partial;
     const int blocks = grid_map_blocks(p);  // the check kernel reads this many partial sums
-    if (norms) k_curve_xfer<true><<<blocks, kGridThreads, 0, p->stream>>>(a);
-    else k_curve_xfer<false><<<blocks, kGridThreads, 0, p->stream>>>(a);
+    if (norms) launch_step(k_curve_xfer<true>, blocks, kGridThreads, 0, p->stream, a);
+    else launch_step(k_curve_xfer<false>, blocks, kGridThreads, 0, p->stream, a);
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
 }
@@ -2467,8 +2480,8 @@ adr_status launch_grid_map_ex(Problem* p, int fam, double* out_even, double* out
     a.parity_shift = parity_shift;
     a.partial = p->partial;
     int blocks = grid_map_blocks(p);
-    if (norms) k_grid_map<true><<<blocks, kGridThreads, 0, p->stream>>>(a);
-    else k_grid_map<false><<<blocks, kGridThreads, 0, p->stream>>>(a);
+    if (norms) launch_step(k_grid_map<true>, blocks, kGridThreads, 0, p->stream, a);
+    else launch_step(k_grid_map<false>, blocks, kGridThreads, 0, p->stream, a);
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
 }
@@ -2561,7 +2574,7 @@ int grid_map_blocks(const Problem* p)
 adr_status launch_check_ex(Problem* p, double tol, int max_iter,
                            cudaGraphConditionalHandle handle, bool use_cond)
 {
-    k_check<<<1, 256, 0, p->stream>>>(p->state, p->partial, grid_map_blocks(p), tol, max_iter,
+    launch_step(k_check, 1, 256, 0, p->stream, p->state, p->partial, grid_map_blocks(p), tol, max_iter,
                                       handle, use_cond ? 1 : 0);
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
@@ -2879,15 +2892,15 @@ adr_status batch_dev_step(BatchDev* b, cudaStream_t st, cudaGraphConditionalHand
     const bool dir = b->gath != nullptr;  // gather passes, then solves from the node values
 #define ADR_BATCH_SOLVE_BS(BS_, FAM_, IT, G)                                                        \
     if (b->ref) {                                                                                  \
-        if (dir) k_curve_solve_batch<BS_, FAM_, true, true><<<G[k], BS_, solve_smem<BS_>(R), st>>>(b->ctab, IT[k], b->act, k); \
-        else k_curve_solve_batch<BS_, FAM_, true><<<G[k], BS_, solve_smem<BS_>(R), st>>>(b->ctab, IT[k], b->act, k);          \
+        if (dir) launch_step(k_curve_solve_batch<BS_, FAM_, true, true>, G[k], BS_, solve_smem<BS_>(R), st, b->ctab, IT[k], b->act, k); \
+        else launch_step(k_curve_solve_batch<BS_, FAM_, true>, G[k], BS_, solve_smem<BS_>(R), st, b->ctab, IT[k], b->act, k);          \
     } else {                                                                                       \
-        if (dir) k_curve_solve_batch<BS_, FAM_, false, true><<<G[k], BS_, solve_smem<BS_>(R), st>>>(b->ctab, IT[k], b->act, k); \
-        else k_curve_solve_batch<BS_, FAM_, false><<<G[k], BS_, solve_smem<BS_>(R), st>>>(b->ctab, IT[k], b->act, k);          \
+        if (dir) launch_step(k_curve_solve_batch<BS_, FAM_, false, true>, G[k], BS_, solve_smem<BS_>(R), st, b->ctab, IT[k], b->act, k); \
+        else launch_step(k_curve_solve_batch<BS_, FAM_, false>, G[k], BS_, solve_smem<BS_>(R), st, b->ctab, IT[k], b->act, k);          \
     }
 #define ADR_BATCH_SOLVE(FAM_, IT, N, G)                                                            \
     if (dir)                                                                                       \
-        k_gather_batch<<<b->map_grid, 256, 0, st>>>(b->gath, FAM_, b->blk_prob, b->blk_local, b->nblk, \
+        launch_step(k_gather_batch, b->map_grid, 256, 0, st, b->gath, FAM_, b->blk_prob, b->blk_local, b->nblk, \
                                                     b->act.blocks_dev, b->act.count, b->act.sel);    \
     for (int k = kItemSets - 1; k >= 0; --k) {                                                     \
         if (!N[k]) continue;                                                                       \
@@ -2901,16 +2914,16 @@ adr_status batch_dev_step(BatchDev* b, cudaStream_t st, cudaGraphConditionalHand
         }                                                                                          \
     }
     ADR_BATCH_SOLVE(0, itB, nB, gB)
-    k_grid_map_batch<false><<<b->map_grid, kGridThreads, 0, st>>>(b->gtab, 0, b->blk_prob, b->blk_local,
+    launch_step(k_grid_map_batch<false>, b->map_grid, kGridThreads, 0, st, b->gtab, 0, b->blk_prob, b->blk_local,
                                                                  b->nblk, b->act.blocks_dev, b->act.count,
                                                                  b->act.sel);
     ADR_BATCH_SOLVE(1, itG, nG, gG)
-    k_grid_map_batch<true><<<b->map_grid, kGridThreads, 0, st>>>(b->gtab, 1, b->blk_prob, b->blk_local,
+    launch_step(k_grid_map_batch<true>, b->map_grid, kGridThreads, 0, st, b->gtab, 1, b->blk_prob, b->blk_local,
                                                                 b->nblk, b->act.blocks_dev, b->act.count,
                                                                 b->act.sel);
 #undef ADR_BATCH_SOLVE
 #undef ADR_BATCH_SOLVE_BS
-    k_check_batch<<<b->n, 256, 0, st>>>(b->states, (const double* const*)b->partials, b->nblk, b->n,
+    launch_step(k_check_batch, b->n, 256, 0, st, b->states, (const double* const*)b->partials, b->nblk, b->n,
                                         b->tol, b->max_iter, b->ticket, cond, b->act.changed);
     if (b->aa_table) {
         // the extrapolated next states of the problems that go on
@@ -2918,9 +2931,9 @@ adr_status batch_dev_step(BatchDev* b, cudaStream_t st, cudaGraphConditionalHand
                       b->act.blocks_dev, b->act.count, b->act.sel};
         TRY_S(launch_anderson_batch(v, st));
     }
-    k_batch_compact<<<b->map_grid, 256, 0, st>>>(b->act, b->d_items, b->d_n_items, b->blk_prob,
+    launch_step(k_batch_compact, b->map_grid, 256, 0, st, b->act, b->d_items, b->d_n_items, b->blk_prob,
                                                  b->n_blk, b->states);
-    k_batch_flip<<<1, 1, 0, st>>>(b->act);
+    launch_step(k_batch_flip, 1, 1, 0, st, b->act);
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
 }
