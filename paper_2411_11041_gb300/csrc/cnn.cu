@@ -82,6 +82,20 @@ constexpr long long kWaitLimit = 1LL << 22;  // default bound: blocking polls (a
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
 
+// one lane of a converged warp.  The issuing loops below are run by whole warps
+// (uniform values, waits included) and only the issue itself is elected: an MMA
+// issued from a branch that one thread took by its index cost about 170 cycles
+// whatever its shape, as its operands have to reach uniform registers.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
+// the warp's index as a value the compiler knows to be the same in all lanes
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0); }
+
 __device__ __forceinline__ void umma(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
@@ -127,6 +141,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* er
     return false;
 }
 
+// a wait of a whole warp: it goes on or gives up together
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, int* err, long long spin)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, spin) ? 1 : 0) != 0;
+}
+
 // 16 BF16 values set to 0 where the mask's are not positive (sign set, zero or NaN)
 __device__ __forceinline__ void relu_mask16(uint32_t (&v)[8], const bf16* mask)
 {
@@ -158,16 +178,65 @@ __device__ __forceinline__ void relu_mask16(uint32_t (&v)[8], const bf16* mask)
 // roundings of the stored activations (0.4 % of the output); the order kept
 // here is tap by tap.
 // Measured, forward of 128 problems (all eight layers): 1.06 ms with two CTAs
-// of one tile each per SM and mma.sync for the last layer, 0.83 ms here; the
-// 128 -> 128 layer at dilation 8 runs at 0.95 PFLOP/s, the last layer took 125
-// us of 64 problems and takes 43.
+// of one tile each per SM and mma.sync for the last layer, 0.83 ms with this
+// kernel for all layers but the first, 0.68 ms with the issue elected and
+// k_conv_win; the 128 -> 128 layer at dilation 8 runs at 1.1 PFLOP/s and 12.6
+// TB/s from L2 (64 problems).
 template <int N, int MT>
 struct ConvWs {
     static constexpr int WH = 8 * MT, THREADS = 64 + 128 * MT, COLS = 2 * MT * N;
 };
 constexpr int kConvMaxStages = 8;
+constexpr int kWinDil = 2;             // largest dilation of k_conv_win (its windows and weights fit)
 constexpr int kFirstSmem = 2 * (128 * 128 + 64 * 128) + 1024;  // k_conv_first's two stages
 constexpr int kConvSmem = 224 * 1024;  // stages, without the alignment slack
+
+// one accumulator row (tensor-memory address src, the calling warp's lanes) to
+// pixel m of the output: bias, ReLU or ReLU mask, BF16; the last layer (N =
+// 16): bias, 8 FP32 channels
+template <int N>
+__device__ __forceinline__ void conv_output(const ConvArgs& a, uint32_t src, long long m)
+{
+#pragma unroll
+    for (int c0 = 0; c0 < N; c0 += 16) {
+        uint32_t v[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+              "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+              "=r"(v[15])
+            : "r"(src + (uint32_t)c0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        if constexpr (N == 16) {  // the last layer: 8 FP32 channels
+            float f[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[j]) + a.bias[j];
+            float4* dst = reinterpret_cast<float4*>(a.y32 + m * kCout);
+            dst[0] = make_float4(f[0], f[1], f[2], f[3]);
+            dst[1] = make_float4(f[4], f[5], f[6], f[7]);
+        } else {
+            uint32_t packed[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                float f0 = __uint_as_float(v[2 * j]), f1 = __uint_as_float(v[2 * j + 1]);
+                if (a.bias) {
+                    f0 += a.bias[c0 + 2 * j];
+                    f1 += a.bias[c0 + 2 * j + 1];
+                }
+                if (a.relu) {
+                    f0 = fmaxf(f0, 0.f);
+                    f1 = fmaxf(f1, 0.f);
+                }
+                __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
+                packed[j] = *reinterpret_cast<uint32_t*>(&h);
+            }
+            if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
+            uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
+            dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+            dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+        }
+    }
+}
 
 // the (tap, channel block) steps of a tile in order, both for the loads and for
 // the MMAs: f(tap, cb, window y, window x); stops when f returns false
@@ -195,7 +264,7 @@ __global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid
     __shared__ uint64_t full[kConvMaxStages], empty[kConvMaxStages], tfull[2], tempty[2];
     __shared__ uint32_t tmem_base;
     __shared__ int s_issued, s_consumed;
-    const int tid = threadIdx.x, warp = tid >> 5, S = a.stages;
+    const int tid = threadIdx.x, warp = warp_index(), S = a.stages;
     const int tiles_x = a.W / 16, per_img = tiles_x * (a.H / WH);
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
@@ -220,7 +289,7 @@ __global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = tmem_base;
     bool ok = true;
-    if (tid == 0) {
+    if (warp == 0) {
         // producer
         const uint64_t pa = reinterpret_cast<uint64_t>(&ta), pw = reinterpret_cast<uint64_t>(&tw);
         int k = 0;
@@ -230,8 +299,10 @@ __global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid
             ok = conv_steps<WH>(a, y0, x0, [&](int tap, int cb, int y, int x) {
                 const int s = k % S;
                 // slot s was last read by the MMAs of step k - S
-                if (k >= S && !mbar_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin)) return false;
+                if (k >= S && !warp_wait(smem_u32(&empty[s]), ((k / S) - 1) & 1, err, a.spin)) return false;
                 const uint32_t sa = sbase + s * STAGE, bar = smem_u32(&full[s]);
+                ++k;
+                if (!elect_one()) return true;
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(STAGE)
                              : "memory");
                 asm volatile(
@@ -244,45 +315,48 @@ __global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid
                     "[%4];\n" ::"r"(sa + A_BYTES),
                     "l"(pw), "r"(tap * a.kc + cb * 64), "r"(0), "r"(bar)
                     : "memory");
-                ++k;
                 return true;
             });
         }
-        s_issued = k;
-    } else if (tid == 32) {
-        // MMA issuer
+        if (tid == 0) s_issued = k;
+    } else if (warp == 1) {
+        // MMA issuer (the whole warp; the same lane is elected throughout)
         const uint32_t idesc = umma_idesc(128, N);
         int k = 0, i = 0;
         for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++i) {
             const int b = t / per_img, r = t - b * per_img;
             const int y0 = (r / tiles_x) * WH, x0 = (r - (r / tiles_x) * tiles_x) * 16;
             const int buf = i & 1;
-            if (i >= 2 && !(ok = mbar_wait(smem_u32(&tempty[buf]), ((i >> 1) - 1) & 1, err, a.spin))) break;
+            if (i >= 2 && !(ok = warp_wait(smem_u32(&tempty[buf]), ((i >> 1) - 1) & 1, err, a.spin))) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n");
             const uint32_t d = tmem + (uint32_t)(buf * MT * N);
             uint32_t acc = 0u;
             ok = conv_steps<WH>(a, y0, x0, [&](int, int, int, int) {
                 const int s = k % S;
-                if (!mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin)) return false;
+                if (!warp_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin)) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint32_t al = desc_lo(sbase + s * STAGE, 16), bl = al + A_BYTES / 16;
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {  // 16 channels: 32 bytes of the swizzled rows
+                    for (int ks = 0; ks < 4; ++ks)  // 16 channels: 32 bytes of the swizzled rows
 #pragma unroll
-                    for (int m = 0; m < MT; ++m)
-                        umma(d + (uint32_t)(m * N), al + m * (128 * 128 / 16) + ks * 2, bl + ks * 2, idesc, acc);
-                    acc = 1u;
+                        for (int m = 0; m < MT; ++m)
+                            umma(d + (uint32_t)(m * N), al + m * (128 * 128 / 16) + ks * 2, bl + ks * 2, idesc,
+                                 ks > 0 ? 1u : acc);
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                        smem_u32(&empty[s])));
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                    smem_u32(&empty[s])));
+                __syncwarp();
+                acc = 1u;
                 ++k;
                 return true;
             });
-            if (ok)
+            if (ok && elect_one())
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                     smem_u32(&tfull[buf])));
+            __syncwarp();
         }
-        s_consumed = k;
+        if (tid == 32) s_consumed = k;
     } else if (warp >= 2) {
         // output: warp w reads lanes 32 (w % 4) .. of accumulator (w - 2) / 4;
         // accumulator row r of window q is the pixel (y0 + 8 q + r / 16, x0 + r % 16)
@@ -300,45 +374,7 @@ __global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid
             const int y0 = (rr / tiles_x) * WH, x0 = (rr - (rr / tiles_x) * tiles_x) * 16;
             const long long m = ((long long)b * a.H + y0 + 8 * q + (r >> 4)) * a.W + x0 + (r & 15);
             const uint32_t src = tmem + lane + (uint32_t)(buf * MT * N);
-#pragma unroll
-            for (int c0 = 0; c0 < N; c0 += 16) {
-                uint32_t v[16];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                      "=r"(v[15])
-                    : "r"(src + (uint32_t)c0));
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-                if constexpr (N == 16) {  // the last layer: 8 FP32 channels
-                    float f[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) f[j] = __uint_as_float(v[j]) + a.bias[j];
-                    float4* dst = reinterpret_cast<float4*>(a.y32 + m * kCout);
-                    dst[0] = make_float4(f[0], f[1], f[2], f[3]);
-                    dst[1] = make_float4(f[4], f[5], f[6], f[7]);
-                } else {
-                    uint32_t packed[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float f0 = __uint_as_float(v[2 * j]), f1 = __uint_as_float(v[2 * j + 1]);
-                        if (a.bias) {
-                            f0 += a.bias[c0 + 2 * j];
-                            f1 += a.bias[c0 + 2 * j + 1];
-                        }
-                        if (a.relu) {
-                            f0 = fmaxf(f0, 0.f);
-                            f1 = fmaxf(f1, 0.f);
-                        }
-                        __nv_bfloat162 h = __floats2bfloat162_rn(f0, f1);
-                        packed[j] = *reinterpret_cast<uint32_t*>(&h);
-                    }
-                    if (a.mask) relu_mask16(packed, a.mask + m * N + c0);
-                    uint4* dst = reinterpret_cast<uint4*>(a.y + m * N + c0);
-                    dst[0] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                    dst[1] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
-                }
-            }
+            conv_output<N>(a, src, m);
             asm volatile("tcgen05.fence::before_thread_sync;\n");
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&tempty[buf])) : "memory");
         }
@@ -356,6 +392,165 @@ __global__ void __launch_bounds__(ConvWs<N, MT>::THREADS, 1) k_conv(const __grid
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(C::COLS));
+}
+
+// The same for 64 input channels and dilations 1 and 2, where a tile of 8 x 16
+// pixels shares most of its taps' pixels: the tile's three windows (one per tap
+// column, 8 + 2 dil rows of 16 pixels; a row is 2 KB, so the taps of a column
+// are 1024-byte aligned offsets of its window) are loaded once, two tiles'
+// worth of windows deep, and all nine taps' weights stay in shared memory for
+// the whole launch.  A tile then takes 60 or 72 KB from L2 instead of 9 x (16 +
+// N / 8) KB.  The taps are summed in k_conv's order.
+// Measured, 64 problems, cold: 64 -> 64 channels 46 us and the last layer 43 us
+// on k_conv, 32 and 27 here.
+template <int N>
+__global__ void __launch_bounds__(192, 1) k_conv_win(const __grid_constant__ CUtensorMap ta,
+                                                     const __grid_constant__ CUtensorMap tw, ConvArgs a, int* err)
+{
+    constexpr int WH = 8, SLOTS = 6, B_BYTES = N * 128, COLS = 2 * N;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t wbase = (smem_u32(smem_raw) + 1023u) & ~1023u, sbase = wbase + 9 * B_BYTES;
+    __shared__ uint64_t full[SLOTS], empty[SLOTS], tfull[2], tempty[2], wfull, done;
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_issued, s_landed, s_mma;
+    const int tid = threadIdx.x, warp = warp_index();
+    const int tiles_x = a.W / 16, per_img = tiles_x * (a.H / WH);
+    const int win = (WH + 2 * a.dil) * 2048;
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                         smem_u32(&tmem_base)),
+                     "r"(COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < SLOTS; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&full[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&empty[s])));
+        }
+        for (int k = 0; k < 2; ++k) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&tfull[k])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 128;\n" ::"r"(smem_u32(&tempty[k])));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&wfull)));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&done)));
+        asm volatile("fence.mbarrier_init.release.cluster;\n");
+        s_issued = s_landed = s_mma = 0;
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+    const uint32_t tmem = tmem_base;
+    bool ok = true;
+    if (warp == 0) {
+        // producer: the weights, then three windows per tile
+        const uint64_t pa = reinterpret_cast<uint64_t>(&ta), pw = reinterpret_cast<uint64_t>(&tw);
+        if (elect_one()) {
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(&wfull)),
+                         "r"(9 * B_BYTES)
+                         : "memory");
+            for (int tap = 0; tap < 9; ++tap)
+                asm volatile(
+                    "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                    "[%4];\n" ::"r"(wbase + tap * B_BYTES),
+                    "l"(pw), "r"(tap * 64), "r"(0), "r"(smem_u32(&wfull))
+                    : "memory");
+        }
+        __syncwarp();
+        int w = 0;
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x) {
+            const int b = t / per_img, r = t - b * per_img;
+            const int y0 = (r / tiles_x) * WH, x0 = (r - (r / tiles_x) * tiles_x) * 16;
+            for (int kx = 0; kx < 3; ++kx, ++w) {
+                const int s = w % SLOTS;
+                // slot s was last read by the MMAs of window w - SLOTS
+                if (w >= SLOTS && !(ok = warp_wait(smem_u32(&empty[s]), ((w / SLOTS) - 1) & 1, err, a.spin))) break;
+                const uint32_t bar = smem_u32(&full[s]);
+                if (!elect_one()) continue;
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(win)
+                             : "memory");
+                asm volatile(
+                    "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+                    "%4, %5}], [%6];\n" ::"r"(sbase + s * win),
+                    "l"(pa), "r"(0), "r"(x0 + (kx - 1) * a.dil), "r"(y0 - a.dil), "r"(b), "r"(bar)
+                    : "memory");
+            }
+        }
+        __syncwarp();
+        if (tid == 0) s_issued = w;
+    } else if (warp == 1) {
+        // MMA issuer
+        const uint32_t idesc = umma_idesc(128, N);
+        int w0 = 0, i = 0, landed = 0, mma = 0;
+        ok = warp_wait(smem_u32(&wfull), 0, err, a.spin);
+        for (int t = blockIdx.x; t < a.tiles && ok; t += gridDim.x, ++i, w0 += 3) {
+            const int buf = i & 1;
+            if (i >= 2 && !(ok = warp_wait(smem_u32(&tempty[buf]), ((i >> 1) - 1) & 1, err, a.spin))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const uint32_t d = tmem + (uint32_t)(buf * N);
+            for (int tap = 0; tap < 9 && ok; ++tap) {
+                const int ky = tap / 3, kx = tap - 3 * ky, w = w0 + kx, s = w % SLOTS;
+                if (ky == 0) {
+                    if (!(ok = warp_wait(smem_u32(&full[s]), (w / SLOTS) & 1, err, a.spin))) break;
+                    landed = w + 1;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n");
+                }
+                const uint32_t al = desc_lo(sbase + s * win, 16) + ky * a.dil * (2048 / 16);
+                const uint32_t bl = desc_lo(wbase + tap * B_BYTES, 16);
+                if (elect_one()) {
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks)
+                        umma(d, al + ks * 2, bl + ks * 2, idesc, (tap > 0 || ks > 0) ? 1u : 0u);
+                    if (ky == 2)
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                                smem_u32(&empty[s])));
+                }
+                __syncwarp();
+                mma = 1;
+            }
+            if (ok && elect_one())
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                    smem_u32(&tfull[buf])));
+            __syncwarp();
+        }
+        if (mma && elect_one())
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                smem_u32(&done)));
+        __syncwarp();
+        if (tid == 32) {
+            s_landed = landed;
+            s_mma = mma;
+        }
+    } else if (warp >= 2) {
+        const int r = ((warp & 3) << 5) + (tid & 31);
+        const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
+        int i = 0;
+        for (int t = blockIdx.x; t < a.tiles; t += gridDim.x, ++i) {
+            const int buf = i & 1;
+            const bool w = mbar_wait(smem_u32(&tfull[buf]), (i >> 1) & 1, err, a.spin);
+            ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;  // the loads below are warp-collective
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const int b = t / per_img, rr = t - b * per_img;
+            const int y0 = (rr / tiles_x) * WH, x0 = (rr - (rr / tiles_x) * tiles_x) * 16;
+            conv_output<N>(a, tmem + lane + (uint32_t)(buf * N),
+                           ((long long)b * a.H + y0 + (r >> 4)) * a.W + x0 + (r & 15));
+            asm volatile("tcgen05.fence::before_thread_sync;\n");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&tempty[buf])) : "memory");
+        }
+    }
+    const bool all_ok = __syncthreads_and(ok ? 1 : 0) != 0;
+    if (!all_ok && tid == 0) {
+        // a wait gave up: the loads land and the MMAs finish before the memories
+        // are released (the default bound)
+        mbar_wait(smem_u32(&wfull), 0, err);
+        for (int w = s_landed; w < s_issued; ++w) mbar_wait(smem_u32(&full[w % SLOTS]), (w / SLOTS) & 1, err);
+        if (s_mma) mbar_wait(smem_u32(&done), 0, err);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(COLS));
 }
 
 // The first layer (40 channels): im2col rows of the 360 features of a pixel
@@ -559,7 +754,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     __shared__ int consumed, used;
     __shared__ float sbias[128];
     const bool bias = blockIdx.y == 0;  // these CTAs' warps 2 and 3 sum dy from its staged tiles
-    const int tid = threadIdx.x, warp = tid >> 5, S = a.stages;
+    const int tid = threadIdx.x, warp = warp_index(), S = a.stages;
     const int g0 = blockIdx.y * a.G, ng = min(a.G, a.npair - g0);
     const int t0 = blockIdx.x * a.per, t1 = min(t0 + a.per, a.tiles), nk = max(t1 - t0, 0);
     const int stage = (2 * a.G + NB) * kWgPlane;
@@ -642,7 +837,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
             issued = k + 1;
             next_window();
         }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         // FP32 accumulator, BF16 operands, both MN-major
         const uint32_t idesc = umma_idesc(128, N) | (1u << 15) | (1u << 16);
         unsigned have = 0u;  // pairs accumulated into
@@ -651,27 +846,33 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
             const int s = k % S;
             const unsigned mk = live(y0, x0);
             next_window();
-            if (!(ok = mbar_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin))) break;
+            if (!(ok = warp_wait(smem_u32(&full[s]), (k / S) & 1, err, a.spin))) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n");
             const uint32_t al = desc_lo(sbase + s * stage, kWgPlane);
             const uint32_t bl = desc_lo(sbase + s * stage + 2 * a.G * kWgPlane, kWgPlane);
-            for (int g = 0; g < ng; ++g) {
-                if (!((mk >> g) & 1u)) continue;
-                const uint32_t first = (have >> g) & 1u;
+            if (elect_one()) {
+                for (int g = 0; g < ng; ++g) {
+                    if (!((mk >> g) & 1u)) continue;
+                    const uint32_t first = (have >> g) & 1u;
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)  // 16 pixels each
-                    umma(tmem + (uint32_t)(g * N), al + (2 * g * kWgPlane + ks * 2048) / 16, bl + ks * (2048 / 16),
-                         idesc, ks > 0 ? 1u : first);
+                    for (int ks = 0; ks < 4; ++ks)  // 16 pixels each
+                        umma(tmem + (uint32_t)(g * N), al + (2 * g * kWgPlane + ks * 2048) / 16, bl + ks * (2048 / 16),
+                             idesc, ks > 0 ? 1u : first);
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                    smem_u32(&empty[s])));
             }
+            __syncwarp();
             have |= mk;
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                smem_u32(&empty[s])));
         }
-        if (k > 0)
+        if (k > 0 && elect_one())
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                 smem_u32(&done)));
-        consumed = k;
-        used = (int)have;
+        __syncwarp();
+        if (tid == 32) {
+            consumed = k;
+            used = (int)have;
+        }
     } else if (warp >= 2 && bias) {
         // two channels a lane: warp w takes dy plane w - 2 (N = 128) or half of
         // the rows of the one plane
@@ -1182,17 +1383,35 @@ adr_status launch_conv_t(const adr_cnn* c, cudaStream_t st, ConvArgs a, const bf
     return ADR_OK;
 }
 
+template <int N>
+adr_status launch_conv_win(const adr_cnn* c, cudaStream_t st, ConvArgs a, const bf16* x, const bf16* wk, int cout)
+{
+    const int rows = 8 + 2 * a.dil;
+    a.tiles = a.B * (a.H / 8) * (a.W / 16);
+    CUtensorMap ta, tw;
+    if (!act_map(&ta, x, a.B, a.H, a.W, 64, rows) || !weight_map(&tw, wk, 9 * 64, cout, N)) {
+        adr::set_error("the driver refused a tensor map of a convolution");
+        return ADR_ECUDA;
+    }
+    const int smem = 6 * rows * 2048 + 9 * N * 128 + 1024;
+    k_conv_win<N><<<std::min(c->n_sm, a.tiles), 192, smem, st>>>(ta, tw, a, c->err);
+    return ADR_OK;
+}
+
 // tiles of 16 x 16 pixels, or of 8 x 16 where the larger ones would leave SMs
 // without one (fewer than about 10 problems)
 adr_status launch_conv(const adr_cnn* c, cudaStream_t st, const ConvArgs& a, const bf16* x, int cin, const bf16* wk,
                        int cout)
 {
+    if (cin == 64 && a.dil <= kWinDil && cout <= 64)  // 64 or 8 output channels
+        return cout == 64 ? launch_conv_win<64>(c, st, a, x, wk, cout) : launch_conv_win<16>(c, st, a, x, wk, cout);
     const bool big = a.B * (a.H / 16) * (a.W / 16) >= c->n_sm;
     if (cout == 128)
         return big ? launch_conv_t<128, 2>(c, st, a, x, cin, wk, cout) : launch_conv_t<128, 1>(c, st, a, x, cin, wk, cout);
     if (cout == 64)
         return big ? launch_conv_t<64, 2>(c, st, a, x, cin, wk, cout) : launch_conv_t<64, 1>(c, st, a, x, cin, wk, cout);
-    return big ? launch_conv_t<16, 2>(c, st, a, x, cin, wk, cout) : launch_conv_t<16, 1>(c, st, a, x, cin, wk, cout);
+    adr::set_error("internal: no convolution kernel for this layer");
+    return ADR_EINVAL;
 }
 
 // forward of a batch: act[0..6] bf16, y32 of the last layer
@@ -1416,8 +1635,10 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem + 1024));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_wgrad_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem + 1024));
     ADR_CUDA_TRY(cudaFuncSetAttribute(k_conv_first, cudaFuncAttributeMaxDynamicSharedMemorySize, kFirstSmem));
-    const void* convs[] = {(const void*)k_conv<16, 1>, (const void*)k_conv<16, 2>,  (const void*)k_conv<64, 1>,
-                           (const void*)k_conv<64, 2>, (const void*)k_conv<128, 1>, (const void*)k_conv<128, 2>};
+    for (const void* f : {(const void*)k_conv_win<16>, (const void*)k_conv_win<64>})
+        ADR_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem + 1024));
+    const void* convs[] = {(const void*)k_conv<64, 1>, (const void*)k_conv<64, 2>, (const void*)k_conv<128, 1>,
+                           (const void*)k_conv<128, 2>};
     for (const void* f : convs)
         ADR_CUDA_TRY(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem + 1024));
     if ((s = adr_cnn_set_params(c, params))) return fail(s);
