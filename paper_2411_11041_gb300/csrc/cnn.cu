@@ -171,7 +171,7 @@ __device__ __forceinline__ void relu_mask16(uint32_t (&v)[8], const bf16* mask)
 // lies outside the image altogether is left out (of 9 taps 6.25 on average are
 // left at dilation 16 and 4 at 32).  The last layer's 8 channels run as N = 16
 // with zero-filled weight rows.
-// What bounds it is the operands' traffic from L2 (8 to 11 TB/s into all SMs).
+// What bounds it is the operands' traffic from L2 (8 to 13 TB/s into all SMs).
 // Loading a window once for the three taps above each other (2 KB rows, so the
 // taps are 1024-byte aligned offsets of it) was 20 % faster in the layers of
 // small dilation, but sums the taps in another order, which flips BF16
@@ -557,8 +557,10 @@ __global__ void __launch_bounds__(192, 1) k_conv_win(const __grid_constant__ CUt
 // staged by cp.async in 64-wide K tiles that run across taps, two stages deep,
 // one CTA of 128 threads per 128 output pixels.  (On k_conv with the channels
 // padded to 64 the K tiles would fall differently and the stored BF16
-// activations would round differently.)  As in k_conv every wait is bounded;
-// the decision to give up is the block's.
+// activations would round differently.)  Bound by the 16-byte copies, 1536 a K
+// tile with their bounds: 60 us for 64 problems, the same with loads two tiles
+// ahead of the MMAs.  As in k_conv every wait is bounded; the decision to give
+// up is the block's.
 __device__ __forceinline__ uint32_t sw128(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
 
 __global__ void __launch_bounds__(128) k_conv_first(ConvArgs a, const bf16* __restrict__ x,
@@ -717,8 +719,10 @@ __global__ void __launch_bounds__(128) k_conv_first(ConvArgs a, const bf16* __re
 // serving all G pairs; partial sums per CTA are reduced in a fixed order
 // afterwards, so the gradient is deterministic.  What bounds it is the planes'
 // traffic from L2: (2 G + N / 64) 8 KB per 4 G MMAs of 128 x N x 16.
-// Measured for a 64-problem batch: 128 -> 128 channels 672 us on mma.sync, 103
-// us here (0.75 PFLOP/s); 64 -> 64 channels 201 -> 60 us.
+// Measured for a 64-problem batch: 128 -> 128 channels 672 us on mma.sync, 80
+// us here at dilation 8 (0.96 PFLOP/s); 64 -> 64 channels 201 -> 38 us.  The
+// bias sums came from a pass of their own (176 us per layer); here two idle warps
+// add them up from the staged dy tiles.
 struct WgradArgs {
     int B, H, W, Cin, Cout, dil;
     float* part;       // [splits][9 Cin][Cout]

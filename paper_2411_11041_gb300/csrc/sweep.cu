@@ -165,7 +165,7 @@ __device__ __forceinline__ double ld_state(const double* p)
 
 // bilinear gather at a row's node from its cell and corner weights (slot sl)
 template <bool COH>
-__device__ __forceinline__ double gather_w(const double* __restrict__ u, int nx, int cell,
+__device__ __forceinline__ double gather_w(const double* u, int nx, int cell,
                                            const double* __restrict__ w, size_t NS, int sl)
 {
     const double* r0 = u + cell;
@@ -590,7 +590,7 @@ struct GroupSync {
 // precision E and v = u + dt x accumulated in FP64 (u is parked in v between
 // the passes) and corr (nullable) keeps the largest |dt x|.  The rows' rp
 // values live in shared memory [R][BS] between the passes.
-template <int BS, int LS, int FAM, bool RES, typename E, bool DIR, bool COH, class Sync>
+template <int BS, int LS, int FAM, bool RES, typename E, bool DIR, class Sync>
 __device__ __forceinline__ void curve_solve_group(const CurveArgs& a, const double* __restrict__ u, int Titem,
                                                   const int* curves, const E* __restrict__ Lc,
                                                   const E* __restrict__ fac, unsigned char* smem, int tid,
@@ -636,9 +636,9 @@ __device__ __forceinline__ void curve_solve_group(const CurveArgs& a, const doub
         if (cnt > 0) {
             const double kap = (FAM == 1) ? __ldg(a.kap + b.line) : 0.0;
             const double* __restrict__ un = u + base + s;
-            double u0 = paper ? 0.0 : ld_state<COH>(un), u1 = paper ? 0.0 : ld_state<COH>(un + 1);
+            double u0 = paper ? 0.0 : __ldg(un), u1 = paper ? 0.0 : __ldg(un + 1);
             for (int j = 0; j < cnt; ++j) {
-                const double u2 = paper ? 0.0 : ld_state<COH>(un + j + 2);
+                const double u2 = paper ? 0.0 : __ldg(un + j + 2);
                 row(j, so + j * T + lt, kap, u0, u1, u2);
                 u0 = u1;
                 u1 = u2;
@@ -646,7 +646,7 @@ __device__ __forceinline__ void curve_solve_group(const CurveArgs& a, const doub
         }
     } else if (cnt > 0) {
         const double kap = (FAM == 1) ? __ldg(a.kap + b.line) : 0.0;
-        auto uslot = [&](int sl) -> double { return gather_w<COH>(u, a.nx, __ldg(a.gcell + sl), a.gw, NS, sl); };
+        auto uslot = [&](int sl) -> double { return gather_w<false>(u, a.nx, __ldg(a.gcell + sl), a.gw, NS, sl); };
         double u0 = 0.0, u1 = 0.0;
         if (!paper) {
             u0 = (s == 0) ? 0.0 : uslot(so + (b.c - 1) * T + (lt - 1));
@@ -675,10 +675,10 @@ __device__ __forceinline__ void curve_solve_group(const CurveArgs& a, const doub
             double u2 = 0.0;
             if (nsl >= 0) {
                 const double* r0 = u + ncell;
-                u2 = nw0 * ld_state<COH>(r0);
-                u2 = fma(nw1, ld_state<COH>(r0 + 1), u2);
-                u2 = fma(nw2, ld_state<COH>(r0 + a.nx), u2);
-                u2 = fma(nw3, ld_state<COH>(r0 + a.nx + 1), u2);
+                u2 = nw0 * __ldg(r0);
+                u2 = fma(nw1, __ldg(r0 + 1), u2);
+                u2 = fma(nw2, __ldg(r0 + a.nx), u2);
+                u2 = fma(nw3, __ldg(r0 + a.nx + 1), u2);
             }
             nsl = next_slot(j + 1);
             if (nsl >= 0) load_desc();
@@ -742,7 +742,7 @@ __device__ __forceinline__ void curve_solve_group(const CurveArgs& a, const doub
             if constexpr (sizeof(E) == 4) x64 = f32_to_f64(x);
             else x64 = x;
             // v = u + dt d in FP64 (u parked in v, or the node values themselves)
-            const double ub = DIR ? ld_state<COH>(u + node) : v[node];
+            const double ub = DIR ? __ldg(u + node) : v[node];
             v[node] = paper ? x64 : fma(a.dt, x64, ub);
             xmax = fmaxf(xmax, fabsf(as_f32(x)));
         } else {
@@ -772,7 +772,7 @@ __device__ __forceinline__ void curve_solve_body(const CurveArgs& a, int Titem, 
                                                  unsigned char* smem)
 {
     const double* u = (a.state && (a.state->iter & 1)) ? a.u_odd : a.u_even;
-    curve_solve_group<BS, BS, FAM, RES, E, DIR, false>(a, u, Titem, curves, Lc, fac, smem, threadIdx.x,
+    curve_solve_group<BS, BS, FAM, RES, E, DIR>(a, u, Titem, curves, Lc, fac, smem, threadIdx.x,
                                                        BlockSync(),
                                                        a.state ? const_cast<unsigned long long*>(&a.state->corr_bits)
                                                                : nullptr);
@@ -882,10 +882,10 @@ __global__ void __launch_bounds__(GS, 1024 / GS) k_curve_solve_slice(CurveArgs a
     const double* u = (a.state && (a.state->iter & 1)) ? a.u_odd : a.u_even;
     unsigned long long* corr = a.state ? const_cast<unsigned long long*>(&a.state->corr_bits) : nullptr;
     if (REF && !(a.state && a.state->hp))
-        curve_solve_group<GS, 256, FAM, true, float, true, false>(a, u, T, cv, lanec32 + lo, a.fac32, smem,
+        curve_solve_group<GS, 256, FAM, true, float, true>(a, u, T, cv, lanec32 + lo, a.fac32, smem,
                                                                   threadIdx.x, BlockSync(), corr);
     else
-        curve_solve_group<GS, 256, FAM, REF, double, true, false>(a, u, T, cv, lanec + lo, a.fac, smem, threadIdx.x,
+        curve_solve_group<GS, 256, FAM, REF, double, true>(a, u, T, cv, lanec + lo, a.fac, smem, threadIdx.x,
                                                                   BlockSync(), corr);
 }
 
@@ -1479,8 +1479,9 @@ __global__ void k_check(IterState* st, const double* partial, int nblocks, doubl
 // where T = GS), dealt to the SMs before it is dealt to an SM's groups, so
 // that every SM's FP64 pipe gets its share of the curves.
 // Data that other blocks write during the launch (the grid states, the curve
-// values, the partial sums) is read from L2 (ld.global.cg); the static tables
-// may stay in L1 from step to step.  Barrier waits are bounded: a block that
+// values) is read by plain loads, which the barrier's acquire orders; the partial
+// sums come from L2.  (All of it from L2: a map at 513^2 24 instead of 17
+// thousand cycles, neighbouring nodes share their lines in L1.)  Barrier waits are bounded: a block that
 // gives up flags IterState::timeout and leaves, and so do the others.
 constexpr int kLoopThreads = 256;
 constexpr size_t kLoopSmem = 224 * 1024;  // dynamic shared memory of a block

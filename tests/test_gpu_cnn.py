@@ -309,3 +309,17 @@ def test_gradient_of_a_batch_is_the_mean_of_its_samples(torch_cuda, batch):
         for lo, hi in ((CNN.offset(l), CNN.offset(l, True)), (CNN.offset(l, True), CNN.offset(l + 1))):
             a, r = g[lo:hi].double(), mean[lo:hi]
             assert (a - r).norm() <= 1e-3 * r.norm(), (l, lo)
+
+
+@pytest.mark.parametrize("batch", [4, 5, 9, 10, 19])
+def test_a_sample_is_the_same_in_every_batch(batch, torch_cuda):
+    """The convolutions' tile follows the batch (tiles per SM) while the order of
+    a pixel's sums does not, so a sample's output is bit for bit that of the
+    sample alone."""
+    torch = torch_cuda
+    from paper_2411_11041_gb300 import Network
+    net = Network(batch, W.cnn_init_params(5, last_scale=1.0))
+    x, _, _, _ = _rand_inputs(batch, 100 + batch, torch)
+    y = net.forward(x).clone()
+    for b in sorted({0, batch // 2, batch - 1}):
+        assert torch.equal(net.forward(x[b:b + 1].contiguous())[0], y[b])
