@@ -2504,7 +2504,9 @@ static cudaError_t loop_launch(const LoopArgs& a, int R, int blocks, cudaStream_
     // as many groups as fit the block's threads and an SM's shared memory
     const int groups = std::min(kLoopThreads / GS, (int)(kLoopSmem / loop_smem<GS, REF>(R)));
     const size_t sm = (size_t)groups * loop_smem<GS, REF>(R);
-    cudaError_t e = cudaFuncSetAttribute(k_solve_loop<GS, REF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    // the same limit at every call: another thread may be between its own two calls
+    cudaError_t e =
+        cudaFuncSetAttribute(k_solve_loop<GS, REF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLoopSmem);
     if (e != cudaSuccess) return e;
     void* args[] = {const_cast<LoopArgs*>(&a)};
     return cudaLaunchCooperativeKernel((const void*)k_solve_loop<GS, REF>, dim3(blocks), dim3(groups * GS), args, sm,

@@ -90,3 +90,31 @@ def test_two_streams_solve_at_once():
     torch.cuda.synchronize()
     for u, r in zip(out, ref):
         assert torch.equal(u, r)
+
+
+def test_threads_with_different_launch_shapes():
+    """Handles whose launches want different amounts of shared memory (rows per
+    thread 4 and 16), solved from two threads at once, many short solves each."""
+    import threading
+
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    ps = [_problem(60, 60, "sheared", "square", seed=3), _problem(240, 240, "sheared", "square", seed=4)]
+    rows = (4, 16)
+    ref = [Solver(p, tol=0.0, max_iter=2, rows_per_thread=r).solve_stationary()[0].clone() for p, r in zip(ps, rows)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in ps]
+    bad = [None, None]
+
+    def work(i):
+        try:
+            with torch.cuda.stream(streams[i]):
+                s = Solver(ps[i], tol=0.0, max_iter=2, rows_per_thread=rows[i], stream=streams[i])
+                bad[i] = sum(not torch.equal(s.solve_stationary()[0], ref[i]) for _ in range(100))
+        except Exception as e:  # reported by the assertion below
+            bad[i] = e
+
+    th = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    [t.start() for t in th]
+    [t.join() for t in th]
+    assert bad == [0, 0]
