@@ -1320,22 +1320,21 @@ adr_status cnn_alloc(adr_cnn* c, T** p, size_t n)
     return ADR_OK;
 }
 
-// the driver's tensor-map encoder, looked up once through the runtime
+// the driver's tensor-map encoder, looked up once through the runtime (the
+// first caller looks it up, others wait for it: C++'s rule for local statics);
+// null when the driver has none
 PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder()
 {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
         void* q = nullptr;
         cudaDriverEntryPointQueryResult res = cudaDriverEntryPointSymbolNotFound;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &q, 12000, cudaEnableDefault, &res) ==
                 cudaSuccess &&
             res == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(q);
-        else
-            cudaGetLastError();
-    }
+            return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(q);
+        cudaGetLastError();
+        return nullptr;
+    }();
     return fn;
 }
 
@@ -1599,6 +1598,10 @@ adr_status adr_cnn_create(int max_batch, const float* params, void* stream, adr_
         return ADR_EINVAL;
     }
     *out = nullptr;
+    if (!tmap_encoder()) {
+        adr::set_error("adr_cnn_create: the driver has no tensor-map encoder (cuTensorMapEncodeTiled)");
+        return ADR_ECUDA;
+    }
     adr_cnn* c = new (std::nothrow) adr_cnn;
     if (!c) return ADR_ENOMEM;
     c->max_batch = max_batch;

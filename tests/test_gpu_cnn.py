@@ -323,3 +323,59 @@ def test_a_sample_is_the_same_in_every_batch(batch, torch_cuda):
     y = net.forward(x).clone()
     for b in sorted({0, batch // 2, batch - 1}):
         assert torch.equal(net.forward(x[b:b + 1].contiguous())[0], y[b])
+
+
+# delays the driver's answer to the first lookup, so that the callers meet in it
+SLOW_LOOKUP = """
+#define _GNU_SOURCE
+#include <dlfcn.h>
+#include <string.h>
+#include <unistd.h>
+int cudaGetDriverEntryPointByVersion(const char* name, void** fn, unsigned version, unsigned long long flags, int* res)
+{
+    int (*next)(const char*, void**, unsigned, unsigned long long, int*) =
+        dlsym(RTLD_NEXT, "cudaGetDriverEntryPointByVersion");
+    if (strcmp(name, "cuTensorMapEncodeTiled") == 0) usleep(500000);
+    return next(name, fn, version, flags, res);
+}
+"""
+FIRST_CALLS = """
+import threading
+import torch
+from paper_2411_11041_gb300 import Network
+N = 4
+x = torch.zeros((1, 64, 64, 40), dtype=torch.bfloat16, device="cuda:0")
+torch.cuda.synchronize()
+start, failed, done = threading.Barrier(N), [], []
+def work():
+    try:
+        with torch.cuda.stream(torch.cuda.Stream()):
+            net = Network(1)
+            start.wait()
+            net.forward(x)
+            done.append(net.sync())
+    except Exception as e:
+        failed.append(repr(e))
+        start.abort()
+ts = [threading.Thread(target=work) for _ in range(N)]
+[t.start() for t in ts]
+[t.join() for t in ts]
+assert not failed, failed
+assert done == [0] * N, done
+"""
+
+
+def test_first_network_calls_from_several_threads(torch_cuda, tmp_path):
+    """The first network calls of a process, from four threads with a network
+    each: the driver's tensor-map encoder is looked up once, and a thread that
+    comes while another looks it up waits for it."""
+    import os
+    import subprocess
+    import sys
+    src, so = tmp_path / "slow.c", tmp_path / "slow.so"
+    src.write_text(SLOW_LOOKUP)
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src), "-ldl"], check=True)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=root, capture_output=True, text=True,
+                       timeout=300, env=dict(os.environ, LD_PRELOAD=str(so)))
+    assert r.returncode == 0, r.stderr[-2000:]
