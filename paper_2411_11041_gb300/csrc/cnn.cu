@@ -889,13 +889,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
             ok = __all_sync(0xffffffffu, w ? 1 : 0) != 0;
             if (!ok) break;
             const uint32_t base = sbase + s * stage + (2 * a.G + plane) * kWgPlane + (lane & 3) * 4;
+            float w0 = 0.f, w1 = 0.f;  // a window's sum first: chains of ROWS and of the windows
 #pragma unroll 8
             for (int r = row0; r < row0 + ROWS; ++r) {
                 uint32_t v;
                 asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(base + r * 128 + (((lane >> 2) ^ (r & 7)) << 4)));
-                s0 += __uint_as_float(v << 16);
-                s1 += __uint_as_float(v & 0xffff0000u);
+                w0 += __uint_as_float(v << 16);
+                w1 += __uint_as_float(v & 0xffff0000u);
             }
+            s0 += w0;
+            s1 += w1;
             __syncwarp();
             if (lane == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(&empty[s])) : "memory");

@@ -379,3 +379,36 @@ def test_first_network_calls_from_several_threads(torch_cuda, tmp_path):
     r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=root, capture_output=True, text=True,
                        timeout=300, env=dict(os.environ, LD_PRELOAD=str(so)))
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_bias_gradient_keeps_small_terms(torch_cuda):
+    """Bias gradients of a large batch against their 64-bit sums, where one pixel
+    of every image outweighs the others by 2^25: added to it one by one in FP32
+    they would all be lost (1e-4 of the sum).  Identity weights and activations
+    of 1 carry the output gradient to every layer exactly.  A sum's chain has at
+    most 64 pixels of a window, 82 windows of a split, 19 splits and 9 partial
+    sums, each step rounding by 2^-24 of the running sum."""
+    torch = torch_cuda
+    from paper_2411_11041_gb300 import Network
+    B = 64
+    prm = np.zeros(CNN.offset(CNN.LAYERS), np.float32)
+    for l in range(1, CNN.LAYERS):
+        cin, cout = W.CNN_CHANNELS[l], W.CNN_CHANNELS[l + 1]
+        w = prm[CNN.offset(l):CNN.offset(l, True)].reshape(9, cin, cout)
+        if l < CNN.LAYERS - 1:
+            w[4, :64, :64] = np.eye(64)
+        else:
+            w[4, :, 0] = 1.0
+    prm[CNN.offset(0, True):CNN.offset(0, True) + 64] = 1.0  # activations of 1, output 64 - 64
+    prm[CNN.offset(CNN.LAYERS - 1, True)] = -64.0
+    net = Network(B, prm)
+    x = torch.zeros((B, 64, 64, 40), dtype=torch.bfloat16, device="cuda:0")
+    t = torch.full((B, 64, 64), -2.0 ** -19, dtype=torch.float32, device="cuda:0")
+    t[:, 0, 0] = -64.0
+    assert not net.forward(x)[..., 0].any()
+    g = net.loss_grad(x, t)[1].double().cpu().numpy()
+    want = B * 64.0 * (1.0 + 4095 * 2.0 ** -25) / (B * 4096)
+    for l in range(CNN.LAYERS - 1):
+        gb = g[CNN.offset(l, True):CNN.offset(l + 1)]
+        assert np.abs(gb[:64] - want).max() <= 174 * 2.0 ** -24 * want, (l, np.abs(gb[:64] - want).max() / want)
+        assert not gb[64:].any()
