@@ -301,7 +301,7 @@ adr_status ensure_iteration_active(Problem* p);
 constexpr int kLoopMaxNodes = 1 << 18;
 bool loop_applies(const Problem* p);
 adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
-                             double* half, double tol, int max_iter, bool norms);
+                             double* half, double tol, int max_iter);
 // Anderson extrapolation (accel.cu)
 adr_status launch_anderson(Problem* p);
 adr_status alloc_anderson(Problem* p);

@@ -226,7 +226,7 @@ adr_status run_iteration(adr_problem* h, double theta, double dt, double sig,
         TRY(prepare_family(p, 1, theta * dt, dt, sig, 0));
         TRY(load_family(p, fextra, fx_scale));
         if (!accel && loop_applies(p)) {
-            TRY(launch_solve_loop(p, dt, p->ubuf[0], p->ubuf[1], p->ubuf[0], p->ubuf[2], tol, max_iter, true));
+            TRY(launch_solve_loop(p, dt, p->ubuf[0], p->ubuf[1], p->ubuf[0], p->ubuf[2], tol, max_iter));
         } else {
         if (!h->exec || h->g_theta != theta || h->g_dt != dt || h->g_sig != sig ||
             h->g_fextra != fextra || h->g_scale != fx_scale || h->g_tol != tol ||
@@ -636,17 +636,6 @@ adr_status adr_split_step(adr_problem* h, double dt, const double* u, double* u_
         TRY(launch_xfer(p, 1, p->fam[0].v, p->xuG, p->xuG, 0, nullptr, nullptr, false, false));
         TRY(launch_line_solve_dir(p, 1, dt, p->xuG, p->xuG, false));
         TRY(launch_grid_map_ex(p, 1, u_next, u_next, 0, nullptr, nullptr, false, false));
-    } else if (loop_applies(p)) {
-        TRY(launch_state_reset(p));
-        TRY(launch_solve_loop(p, dt, u, u_next, u_next, half, -1.0, 1, false));
-        IterState st;
-        ADR_CUDA_TRY(cudaMemcpyAsync(&st, p->state, sizeof st, cudaMemcpyDeviceToHost, p->stream));
-        ADR_CUDA_TRY(cudaStreamSynchronize(p->stream));
-        if (st.timeout) {
-            set_error("the split step gave up waiting at a grid barrier; its outputs are not valid");
-            return ADR_ETIMEOUT;
-        }
-        return ADR_OK;
     } else {
         TRY(launch_substep_solve(p, 0, dt, u, u, false));
         TRY(launch_grid_map_ex(p, 0, half, half, 0, nullptr, nullptr, false, false));

@@ -1499,7 +1499,6 @@ struct LoopArgs {
     double* partial;  // [2][2 * gridDim.x] by the step's parity
     double tol;
     int max_iter;
-    int norms;        // 0: exactly max_iter steps, no norms (a split step of a caller's own loop)
 };
 
 // all blocks of the (cooperative) launch; *epoch counts the barriers passed
@@ -1792,7 +1791,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_con
     for (;;) {
         const double* u = (iter & 1) ? a.c[0].u_odd : a.c[0].u_even;
         double* un = (iter & 1) ? a.g[1].out_even : a.g[1].out_odd;
-        unsigned long long* corr = REF && a.norms ? &a.state->corr_loop[iter & 1] : nullptr;
+        unsigned long long* corr = REF ? &a.state->corr_loop[iter & 1] : nullptr;
         double dd = 0.0, uu = 0.0;
         loop_solve<GS, 0, REF>(a, u, hp, sm, corr, w0, pre);
         map_prefetch(a.g[0], first, mp);
@@ -1804,13 +1803,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_con
         loop_solve<GS, 1, REF>(a, a.c[1].u_even, hp, sm, corr, w1, pre);
         map_prefetch(a.g[1], first, mp);
         if (!grid_barrier(a.state, epoch)) return;
-        if (!a.norms) {
-            grid_map_nodes<false>(a.g[1], un, nullptr, first, stride, dd, uu, mp);
-            loop_prefetch(a.c[0], w0, pre);
-            if (++iter >= a.max_iter) break;
-            if (!grid_barrier(a.state, epoch)) return;
-            continue;
-        }
         grid_map_nodes<true>(a.g[1], un, u, first, stride, dd, uu, mp);
         loop_prefetch(a.c[0], w0, pre);
         if (warp < nwarp) {
@@ -1867,7 +1859,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_con
         st->converged = conv;
         st->hp = hp;
         st->fp32_steps = fp32;
-        if (REF && a.norms)  // the last step's corrections are behind its barriers
+        if (REF)  // the last step's corrections are behind its barriers
             st->corr = __longlong_as_double((long long)__ldcg(&st->corr_loop[(iter - 1) & 1]));
         st->done = 1;
     }
@@ -2514,9 +2506,9 @@ static cudaError_t loop_launch(const LoopArgs& a, int R, int blocks, cudaStream_
 }
 
 // steps from u_even (the state buffers by the step's parity; the first step
-// reads u_even), u_{j+1/2} in half; norms = false: exactly max_iter steps
+// reads u_even), u_{j+1/2} in half
 adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
-                             double* half, double tol, int max_iter, bool norms)
+                             double* half, double tol, int max_iter)
 {
     LoopArgs a{};
     int tmax = 32;
@@ -2553,7 +2545,6 @@ adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double
     a.partial = p->partial;
     a.tol = tol;
     a.max_iter = max_iter;
-    a.norms = norms ? 1 : 0;
     const int blocks = std::min(p->n_sm, p->n_loop_blocks);
     const bool ref = p->opts.prec == ADR_FP32_REFINE;
     cudaError_t e = cudaSuccess;

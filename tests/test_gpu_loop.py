@@ -118,3 +118,32 @@ def test_threads_with_different_launch_shapes():
     [t.start() for t in th]
     [t.join() for t in th]
     assert bad == [0, 0]
+
+
+def _beside_a_busy_stream(call, mine):
+    """call() on stream mine while another stream keeps one block of the device
+    busy for about 50 ms; whether it came back before that stream was done."""
+    import torch
+    other = torch.cuda.Stream()
+    with torch.cuda.stream(mine):
+        call()  # first use: buffers, factors, kernels
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(100_000_000)
+    with torch.cuda.stream(mine):
+        call()  # returns when its results are there
+    first = not other.query()
+    torch.cuda.synchronize()
+    return first
+
+
+@pytest.mark.parametrize("n", [33, 129, 300])
+def test_split_step_does_not_wait_for_other_streams(n):
+    """A split step needs no empty device: it runs beside another stream's kernel."""
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    mine = torch.cuda.Stream()
+    s = Solver(_problem(n, n, "sheared", "square"), stream=mine)
+    u = torch.rand((n, n), dtype=torch.float64, device="cuda:0")
+    torch.cuda.synchronize()
+    assert _beside_a_busy_stream(lambda: s.split_step(u, 0.05), mine)
