@@ -158,7 +158,6 @@ struct Problem {
     int n_interior = 0;
     int n_sm = 0;
     bool coop = false;     // the device takes cooperative launches
-    int n_loop_blocks = 0; // blocks of the one-launch iteration the partial sums have room for
     int rows_per_thread = 16;   // launch shape of the curve solve (<= 16 rows per thread)
     int map_blocks_per_sm = 4;  // launch shape of the curve -> grid map
     bool const_beta = false;
@@ -296,9 +295,12 @@ adr_status launch_mask_copy(Problem* p, const double* in, double* out);
 // batch reads the active buffers once, when it is built
 adr_status ensure_iteration_active(Problem* p);
 // the outer iteration in one cooperative launch (sweep.cu), measured faster up
-// to about 500^2 nodes; larger grids take the graph of separate kernels, whose
-// blocks fill the chip by themselves
-constexpr int kLoopMaxNodes = 1 << 18;
+// to about 400^2 nodes (385^2 45.0 us a step, the graph 48.9; 420^2 55 and 56);
+// larger grids take the graph of separate kernels, whose blocks fill the chip
+// by themselves.  Near the limit two handles on two streams gain as well (385^2
+// 70 us for both, graphs 84), four or more would be better off as graphs (141
+// and 112)
+constexpr int kLoopMaxNodes = 400 * 400;
 bool loop_applies(const Problem* p);
 adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
                              double* half, double tol, int max_iter);

@@ -488,8 +488,8 @@ adr_status adr_create(const adr_grid* grid, const uint8_t* mask, double mu, doub
             return fail(cuda_fail(e, "cudaMemsetAsync"));
     }
     if ((s = alloc_anderson(p))) return fail(s);
-    p->n_loop_blocks = p->n_sm;  // the one-launch iteration keeps two steps' partial sums
-    if ((s = dev_alloc(p, &p->partial, 2 * (size_t)std::max(p->n_partial_blocks, 2 * p->n_loop_blocks))) ||
+    // the one-launch iteration keeps two steps' partial sums of at most a block per SM
+    if ((s = dev_alloc(p, &p->partial, 2 * (size_t)std::max(p->n_partial_blocks, 2 * p->n_sm))) ||
         (s = dev_alloc(p, &p->state, 1)) || (s = dev_alloc(p, &p->fextra, N)) ||
         (s = dev_alloc(p, &p->pivmin, 2)))
         return fail(s);

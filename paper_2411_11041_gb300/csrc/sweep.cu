@@ -1462,19 +1462,26 @@ __global__ void k_check(IterState* st, const double* partial, int nblocks, doubl
 
 // ---------------------------------------------------- one-launch iteration
 // The whole outer iteration of a small or medium problem as one cooperative
-// launch: one block per SM stays resident and walks the phases of every split
-// step (B solve with its gather, B map, G solve with its gather, G map with
-// the norms) with a grid barrier after each, and every block evaluates the
-// convergence test from the same partial sums in the same order.  The
-// arithmetic per row and node is the separate kernels', in the same order.
+// launch: its blocks stay resident and walk the phases of every split step (B
+// solve with its gather, B map, G solve with its gather, G map with the norms)
+// with a grid barrier after each, and every block evaluates the convergence
+// test from the same partial sums in the same order.  The arithmetic per row
+// and node is the separate kernels', in the same order.
 // What bounds these sizes is latency, not a pipe: a graph node costs about 4 us
 // from its predecessor's last block to its own, seven times a step; here a
 // barrier costs 1.3 us, four times a step, and a warp's FP64 instruction 64
-// cycles (31 ns), dependent or not.  Measured per split step (sheared
-// problem, FP64, graph of kernels -> one launch): 33^2 25.6 -> 13.0 us,
-// 64^2 28.4 -> 13.6, 129^2 32.7 -> 19.3, 257^2 40.4 -> 28.6, 385^2 52.1 -> 39.4,
-// 500^2 75 -> 72; at 700^2 one block of 256 threads per SM no longer hides the
-// tables' latency (110 -> 129 us), hence kLoopMaxNodes.
+// cycles (31 ns), dependent or not.
+// The blocks take half an SM's registers (128 threads of 254: with 128 registers
+// each thread spills, 64^2 13.8 -> 18.6 us a step), one per SM at most and fewer
+// where the work is little (loop_blocks), so that solves on several streams and
+// other kernels share the device: a cooperative launch starts only when all its
+// blocks fit.  Measured per split step (sheared problem, FP64), graph of
+// kernels -> one launch: 33^2 27.1 -> 12.9 us, 64^2 27.8 -> 14.2, 129^2 34.1 ->
+// 20.7, 200^2 38.0 -> 27.3, 257^2 39.9 -> 31.6, 300^2 42.9 -> 34.9, 385^2 48.9 ->
+// 45.0, 420^2 56.0 -> 55.  Blocks of 256 threads on every SM took 13.9, 19.5,
+// 29.0 and 40 at 64^2, 129^2, 257^2 and 385^2, but handles on several streams
+// then took turns: eight of 64^2 109 us a step for all (the graphs 47, now 18),
+// eight of 129^2 156 (58, 45), four of 257^2 116 (75, 67).
 // A group of GS threads owns one slice of a 256-thread work item (one curve
 // where T = GS), dealt to the SMs before it is dealt to an SM's groups, so
 // that every SM's FP64 pipe gets its share of the curves.
@@ -1483,8 +1490,7 @@ __global__ void k_check(IterState* st, const double* partial, int nblocks, doubl
 // sums come from L2.  (All of it from L2: a map at 513^2 24 instead of 17
 // thousand cycles, neighbouring nodes share their lines in L1.)  Barrier waits are bounded: a block that
 // gives up flags IterState::timeout and leaves, and so do the others.
-constexpr int kLoopThreads = 256;
-constexpr size_t kLoopSmem = 224 * 1024;  // dynamic shared memory of a block
+constexpr int kLoopThreads = 128;
 constexpr int kLoopSpin = 1 << 23;  // polls of one barrier wait (several seconds)
 
 struct LoopArgs {
@@ -1762,7 +1768,7 @@ __device__ __forceinline__ void loop_solve(const LoopArgs& a, const double* u, b
 }
 
 template <int GS, bool REF>
-__global__ void __launch_bounds__(kLoopThreads, 1) k_solve_loop(const __grid_constant__ LoopArgs a)
+__global__ void __launch_bounds__(kLoopThreads, 2) k_solve_loop(const __grid_constant__ LoopArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double red[2][kLoopThreads / 32];
@@ -2479,30 +2485,47 @@ adr_status launch_grid_map_ex(Problem* p, int fam, double* out_even, double* out
     return ADR_OK;
 }
 
+// blocks of the one-launch iteration: a group for every slice of the work items
+// and a warp for every run of 32 nodes, but more than half the SMs only where a
+// warp would have more than two runs.  Measured, us a step at 8/16/25/38/76/152
+// blocks: 64^2 32.2/20.6/15.8/14.2/14.2/13.8 (32 taken), 129^2
+// 86.6/48.7/36.5/28.7/20.6/19.5 (76), 257^2 264/144/97/71/43/31.7 (152).
+static int loop_blocks(const Problem* p)
+{
+    constexpr int kWarps = kLoopThreads / 32;
+    const int items = std::max(p->fam[0].iset[0].count, p->fam[1].iset[0].count), runs = (p->N + 31) / 32;
+    const int solve = items * (256 / kLoopThreads);
+    const int map = std::max(std::min((runs + kWarps - 1) / kWarps, p->n_sm / 2), (runs + 2 * kWarps - 1) / (2 * kWarps));
+    return std::min(std::max(solve, map), p->n_sm);
+}
+
 // one-launch iteration: problems through the grid whose curves take at most
-// 64 threads (their groups' tables fit an SM's shared memory) and whose step
-// is bound by latency
+// 64 threads (the groups' tables fit shared memory) and whose step is bound by
+// latency: few enough nodes, and at most three slices a group.  Many short
+// curves take longer here than as blocks of their own (17 x 4000 nodes, 5.5
+// slices a group: 37.9 us a step, the graph 35.2; 4000 x 17 38.7 and 32.3; 17 x
+// 2000, 2.7 slices: 22.5 and 29.4)
 bool loop_applies(const Problem* p)
 {
     if (p->opts.transfer || p->N > kLoopMaxNodes || p->n_sm <= 0 || !p->coop) return false;
     for (const Family& F : p->fam)
-        if (!F.iset[0].count || F.iset[1].count || F.iset[2].count || F.tmax > 64) return false;
+        if (!F.iset[0].count || F.iset[1].count || F.iset[2].count || F.tmax > 64 ||
+            F.iset[0].count * (256 / kLoopThreads) > 3 * p->n_sm)
+            return false;
     return true;
 }
 
 template <int GS, bool REF>
 static cudaError_t loop_launch(const LoopArgs& a, int R, int blocks, cudaStream_t st)
 {
-    // as many groups as fit the block's threads and an SM's shared memory
-    const int groups = std::min(kLoopThreads / GS, (int)(kLoopSmem / loop_smem<GS, REF>(R)));
-    const size_t sm = (size_t)groups * loop_smem<GS, REF>(R);
+    constexpr int groups = kLoopThreads / GS;
     // the same limit at every call: another thread may be between its own two calls
-    cudaError_t e =
-        cudaFuncSetAttribute(k_solve_loop<GS, REF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLoopSmem);
+    cudaError_t e = cudaFuncSetAttribute(k_solve_loop<GS, REF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(groups * loop_smem<GS, REF>(kCmax)));
     if (e != cudaSuccess) return e;
     void* args[] = {const_cast<LoopArgs*>(&a)};
-    return cudaLaunchCooperativeKernel((const void*)k_solve_loop<GS, REF>, dim3(blocks), dim3(groups * GS), args, sm,
-                                       st);
+    return cudaLaunchCooperativeKernel((const void*)k_solve_loop<GS, REF>, dim3(blocks), dim3(kLoopThreads), args,
+                                       groups * loop_smem<GS, REF>(R), st);
 }
 
 // steps from u_even (the state buffers by the step's parity; the first step
@@ -2545,7 +2568,7 @@ adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double
     a.partial = p->partial;
     a.tol = tol;
     a.max_iter = max_iter;
-    const int blocks = std::min(p->n_sm, p->n_loop_blocks);
+    const int blocks = loop_blocks(p);
     const bool ref = p->opts.prec == ADR_FP32_REFINE;
     cudaError_t e = cudaSuccess;
 #define ADR_LOOP(GS_) e = ref ? loop_launch<GS_, true>(a, R, blocks, p->stream) : loop_launch<GS_, false>(a, R, blocks, p->stream)

@@ -147,3 +147,62 @@ def test_split_step_does_not_wait_for_other_streams(n):
     u = torch.rand((n, n), dtype=torch.float64, device="cuda:0")
     torch.cuda.synchronize()
     assert _beside_a_busy_stream(lambda: s.split_step(u, 0.05), mine)
+
+
+@pytest.mark.parametrize("n", [33, 129, 300])
+def test_solve_does_not_wait_for_other_streams(n):
+    """The one launch takes part of an SM's registers: it starts beside another
+    stream's kernel."""
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    mine = torch.cuda.Stream()
+    s = Solver(_problem(n, n, "sheared", "square"), tol=0.0, max_iter=10, stream=mine)
+    torch.cuda.synchronize()
+    assert _beside_a_busy_stream(lambda: s.solve_stationary(), mine)
+
+
+@pytest.mark.parametrize("n,k", [(64, 4), (129, 4), (257, 2)])
+def test_small_solves_overlap(n, k):
+    """k handles of one size on k streams: their launches fit the device side by
+    side, so all of them take little longer than one (below 1.5 of it; one
+    after the other k of it)."""
+    import threading
+    import time
+
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    streams = [torch.cuda.Stream() for _ in range(k)]
+    hs = [Solver(_problem(n, n, "sheared", "square", seed=i), tol=0.0, max_iter=2000, stream=streams[i])
+          for i in range(k)]
+    torch.cuda.synchronize()
+
+    def seconds(m):
+        go = threading.Barrier(m + 1)
+
+        def work(i):
+            with torch.cuda.stream(streams[i]):
+                go.wait()
+                hs[i].solve_stationary()
+
+        th = [threading.Thread(target=work, args=(i,)) for i in range(m)]
+        [t.start() for t in th]
+        go.wait()
+        t0 = time.perf_counter()
+        [t.join() for t in th]
+        return time.perf_counter() - t0
+
+    seconds(k)
+    one, all_ = min(seconds(1) for _ in range(3)), min(seconds(k) for _ in range(3))
+    assert all_ < 1.5 * one, (one, all_)
+
+
+@pytest.mark.parametrize("nx,ny,field", [
+    (400, 400, "sheared"),               # the largest grid of the one launch
+    (401, 400, "sheared"),               # the first of the separate kernels
+    (17, 2200, (0.8, 0.6)),              # near three slices a group
+    (17, 2400, (0.8, 0.6)),              # past them: separate kernels
+    (600, 260, (1.0, 0.0)),              # 64 threads a curve, two groups a block
+])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_fixed_steps_match_oracle_at_the_rules_edges(nx, ny, field, prec):
+    test_fixed_steps_match_oracle(nx, ny, field, "square", prec)
