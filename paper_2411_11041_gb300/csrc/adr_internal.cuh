@@ -158,6 +158,7 @@ struct Problem {
     int n_interior = 0;
     int n_sm = 0;
     bool coop = false;     // the device takes cooperative launches
+    int stream_sms = 0;    // SMs the stream's kernels may use (fewer than n_sm on a partition)
     int rows_per_thread = 16;   // launch shape of the curve solve (<= 16 rows per thread)
     int map_blocks_per_sm = 4;  // launch shape of the curve -> grid map
     bool const_beta = false;
@@ -302,8 +303,10 @@ adr_status ensure_iteration_active(Problem* p);
 // and 112)
 constexpr int kLoopMaxNodes = 400 * 400;
 bool loop_applies(const Problem* p);
+// *launched = false: the runtime refused the launch, nothing was enqueued and
+// the handle takes the graph from now on
 adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
-                             double* half, double tol, int max_iter);
+                             double* half, double tol, int max_iter, bool* launched);
 // Anderson extrapolation (accel.cu)
 adr_status launch_anderson(Problem* p);
 adr_status alloc_anderson(Problem* p);

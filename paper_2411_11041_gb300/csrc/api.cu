@@ -1,6 +1,8 @@
 // C ABI of the directional splitting solver: handle lifecycle, the outer
 // iteration as one CUDA graph with a device-side WHILE loop, and the
 // parabolic time stepping.  See include/adr.h for the contract.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -195,6 +197,37 @@ adr_status finish_direct(Problem* p, int max_iter, double* out, double* iter_out
     return ADR_OK;
 }
 
+// SMs that kernels on a stream may use: all of the device's, unless the stream
+// belongs to a partition of them (a green context)
+int stream_sm_count(cudaStream_t st, int n_sm)
+{
+    struct Api {
+        PFN_cuStreamGetCtx_v9020 ctx = nullptr;
+        PFN_cuCtxGetDevResource_v12040 res = nullptr;
+    };
+    static const Api api = [] {
+        Api a;
+        auto get = [](const char* name, unsigned version) -> void* {
+            void* q = nullptr;
+            cudaDriverEntryPointQueryResult r = cudaDriverEntryPointSymbolNotFound;
+            if (cudaGetDriverEntryPointByVersion(name, &q, version, cudaEnableDefault, &r) == cudaSuccess &&
+                r == cudaDriverEntryPointSuccess)
+                return q;
+            cudaGetLastError();
+            return nullptr;
+        };
+        a.ctx = reinterpret_cast<PFN_cuStreamGetCtx_v9020>(get("cuStreamGetCtx", 9020));
+        a.res = reinterpret_cast<PFN_cuCtxGetDevResource_v12040>(get("cuCtxGetDevResource", 12040));
+        return a;
+    }();
+    CUcontext ctx = nullptr;
+    CUdevResource r{};
+    if (!api.ctx || !api.res || api.ctx(st, &ctx) != CUDA_SUCCESS ||
+        api.res(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS || r.sm.smCount < 1)
+        return n_sm;
+    return std::min(n_sm, (int)r.sm.smCount);
+}
+
 // the handle's capture stream and timing events, on first use
 adr_status ensure_stream_events(adr_problem* h)
 {
@@ -225,14 +258,15 @@ adr_status run_iteration(adr_problem* h, double theta, double dt, double sig,
         TRY(prepare_family(p, 0, theta * dt, dt, sig, 0));
         TRY(prepare_family(p, 1, theta * dt, dt, sig, 0));
         TRY(load_family(p, fextra, fx_scale));
-        if (!accel && loop_applies(p)) {
-            TRY(launch_solve_loop(p, dt, p->ubuf[0], p->ubuf[1], p->ubuf[0], p->ubuf[2], tol, max_iter));
-        } else {
-        if (!h->exec || h->g_theta != theta || h->g_dt != dt || h->g_sig != sig ||
-            h->g_fextra != fextra || h->g_scale != fx_scale || h->g_tol != tol ||
-            h->g_max_iter != max_iter || h->g_accel != accel)
-            TRY(build_graph(h, theta, dt, sig, fextra, fx_scale, tol, max_iter, accel));
-        ADR_CUDA_TRY(cudaGraphLaunch(h->exec, p->stream));
+        bool launched = false;
+        if (!accel && loop_applies(p))
+            TRY(launch_solve_loop(p, dt, p->ubuf[0], p->ubuf[1], p->ubuf[0], p->ubuf[2], tol, max_iter, &launched));
+        if (!launched) {
+            if (!h->exec || h->g_theta != theta || h->g_dt != dt || h->g_sig != sig ||
+                h->g_fextra != fextra || h->g_scale != fx_scale || h->g_tol != tol ||
+                h->g_max_iter != max_iter || h->g_accel != accel)
+                TRY(build_graph(h, theta, dt, sig, fextra, fx_scale, tol, max_iter, accel));
+            ADR_CUDA_TRY(cudaGraphLaunch(h->exec, p->stream));
         }
     }
     if (p->opts.transfer) TRY(finish_direct(p, max_iter, out, iter_out, midpoint));
@@ -453,6 +487,7 @@ adr_status adr_create(const adr_grid* grid, const uint8_t* mask, double mu, doub
         int coop = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
         p->coop = coop != 0;
+        p->stream_sms = stream_sm_count(p->stream, p->n_sm);
     }
     adr_status s = ADR_OK;
     auto fail = [&](adr_status st) {

@@ -2495,8 +2495,9 @@ static int loop_blocks(const Problem* p)
     constexpr int kWarps = kLoopThreads / 32;
     const int items = std::max(p->fam[0].iset[0].count, p->fam[1].iset[0].count), runs = (p->N + 31) / 32;
     const int solve = items * (256 / kLoopThreads);
-    const int map = std::max(std::min((runs + kWarps - 1) / kWarps, p->n_sm / 2), (runs + 2 * kWarps - 1) / (2 * kWarps));
-    return std::min(std::max(solve, map), p->n_sm);
+    const int map =
+        std::max(std::min((runs + kWarps - 1) / kWarps, p->stream_sms / 2), (runs + 2 * kWarps - 1) / (2 * kWarps));
+    return std::min(std::max(solve, map), p->stream_sms);
 }
 
 // one-launch iteration: problems through the grid whose curves take at most
@@ -2507,10 +2508,12 @@ static int loop_blocks(const Problem* p)
 // 2000, 2.7 slices: 22.5 and 29.4)
 bool loop_applies(const Problem* p)
 {
-    if (p->opts.transfer || p->N > kLoopMaxNodes || p->n_sm <= 0 || !p->coop) return false;
+    if (p->opts.transfer || p->n_sm <= 0 || !p->coop) return false;
+    // on a partition of the SMs (it has to hold all blocks at once) its share of the nodes
+    if ((long long)p->N * p->n_sm > (long long)kLoopMaxNodes * p->stream_sms) return false;
     for (const Family& F : p->fam)
         if (!F.iset[0].count || F.iset[1].count || F.iset[2].count || F.tmax > 64 ||
-            F.iset[0].count * (256 / kLoopThreads) > 3 * p->n_sm)
+            F.iset[0].count * (256 / kLoopThreads) > 3 * p->stream_sms)
             return false;
     return true;
 }
@@ -2531,8 +2534,9 @@ static cudaError_t loop_launch(const LoopArgs& a, int R, int blocks, cudaStream_
 // steps from u_even (the state buffers by the step's parity; the first step
 // reads u_even), u_{j+1/2} in half
 adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double* u_odd, double* out_even,
-                             double* half, double tol, int max_iter)
+                             double* half, double tol, int max_iter, bool* launched)
 {
+    *launched = false;
     LoopArgs a{};
     int tmax = 32;
     int R = 1;
@@ -2575,6 +2579,14 @@ adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double
     if (tmax <= 32) ADR_LOOP(32);
     else ADR_LOOP(64);
 #undef ADR_LOOP
+    *launched = e == cudaSuccess;
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported ||
+        e == cudaErrorInvalidValue) {
+        // the blocks do not fit what the process may use of the device: separate kernels
+        cudaGetLastError();
+        p->coop = false;
+        return ADR_OK;
+    }
     if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel (one-launch iteration)");
     return ADR_OK;
 }

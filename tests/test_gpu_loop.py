@@ -206,3 +206,81 @@ def test_small_solves_overlap(n, k):
 @pytest.mark.parametrize("prec", [0, 1])
 def test_fixed_steps_match_oracle_at_the_rules_edges(nx, ny, field, prec):
     test_fixed_steps_match_oracle(nx, ny, field, "square", prec)
+
+
+REFUSED = """
+import sys
+import numpy as np
+import torch
+from tests.test_gpu_loop import _problem
+from paper_2411_11041_gb300 import Solver
+for prec in (0, 1):
+    s = Solver(_problem(90, 70, "sheared", "square"), tol=0.0, max_iter=7, prec=prec)
+    for _ in range(2):
+        u, _, st, _ = s.solve_stationary()
+        assert st["iters"] == 7
+    np.save(sys.argv[1] + "%d.npy" % prec, u.cpu().numpy())
+"""
+
+
+def test_a_refused_launch_takes_the_graph(tmp_path):
+    """Where the runtime refuses the cooperative launch (the blocks do not fit the
+    part of the device the process may use; here a library in front of the
+    runtime answers so), the solve runs as the graph of separate kernels."""
+    import os
+    import subprocess
+    import sys
+
+    from paper_2411_11041_gb300 import Solver
+    src, so = tmp_path / "refuse.c", tmp_path / "refuse.so"
+    src.write_text("int cudaLaunchCooperativeKernel() { return 720; }\n")  # cudaErrorCooperativeLaunchTooLarge
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", REFUSED, str(tmp_path / "u")], cwd=root, capture_output=True, text=True,
+                       timeout=300, env=dict(os.environ, LD_PRELOAD=str(so)))
+    assert r.returncode == 0, r.stderr[-2000:]
+    for prec in (0, 1):
+        u = Solver(_problem(90, 70, "sheared", "square"), tol=0.0, max_iter=7, prec=prec).solve_stationary()[0]
+        assert np.array_equal(u.cpu().numpy(), np.load(tmp_path / f"u{prec}.npy"))
+
+
+def _partition_stream(sms):
+    """A stream on a partition of about sms SMs (a green context of this process)."""
+    import ctypes as C
+
+    import torch
+    torch.zeros(1, device="cuda:0")  # the primary context
+    cu = C.CDLL("libcuda.so.1")
+
+    def ok(code, what):
+        if code:
+            pytest.skip(f"no partition of the SMs here: {what} gave {code}")
+
+    size = 4 + 92 + 48  # CUdevResource; the SM count is the first word of its union
+    whole, part, rest = (C.create_string_buffer(size) for _ in range(3))
+    groups, desc, ctx, st = C.c_uint(1), C.c_void_p(), C.c_void_p(), C.c_void_p()
+    ok(cu.cuDeviceGetDevResource(0, whole, 1), "cuDeviceGetDevResource")
+    ok(cu.cuDevSmResourceSplitByCount(part, C.byref(groups), whole, rest, 0, C.c_uint(sms)), "cuDevSmResourceSplitByCount")
+    ok(cu.cuDevResourceGenerateDesc(C.byref(desc), part, 1), "cuDevResourceGenerateDesc")
+    ok(cu.cuGreenCtxCreate(C.byref(ctx), desc, 0, 1), "cuGreenCtxCreate")
+    ok(cu.cuGreenCtxStreamCreate(C.byref(st), ctx, 1, 0), "cuGreenCtxStreamCreate")
+    return torch.cuda.ExternalStream(st.value), int.from_bytes(part.raw[96:100], "little")
+
+
+@pytest.mark.parametrize("n", [64, 129, 300])
+def test_solve_on_a_partition_of_the_sms(n):
+    """A stream that has a few of the SMs: as many blocks as those hold, or the
+    graph, and the same states as on the whole device."""
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    p = _problem(n, n, "sheared", "square")
+    ref = Solver(p, tol=0.0, max_iter=20).solve_stationary()[0].clone()
+    st, sms = _partition_stream(16)
+    assert 1 <= sms < torch.cuda.get_device_properties(0).multi_processor_count
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        s = Solver(p, tol=0.0, max_iter=20, stream=st)
+        for _ in range(2):
+            u, _, stats, _ = s.solve_stationary()
+    torch.cuda.synchronize()
+    assert stats["iters"] == 20 and torch.equal(u, ref)
