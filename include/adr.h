@@ -272,10 +272,12 @@ adr_status adr_time_kernels(adr_problem* prob, int reps, double* ms_out);
 /*
  * adr_autotune -- choose the launch shapes of a handle by measurement (no
  * counterpart in the paper; the result does not change the solution).  Each
- * candidate (rows_per_thread in {4, 8, 16}, map_blocks_per_sm in {2, 4, 8}) is
- * applied and one split step's kernels are timed reps times with CUDA events
- * on the handle's stream; the fastest is kept.  Outputs (host, nullable): the
- * chosen rows_per_thread and map_blocks_per_sm and its ms per split step.
+ * candidate (rows_per_thread in {4, 8, 16}, map_blocks_per_sm in {2, 4, 8}; the
+ * one launch of small grids has no map blocks: 4) is applied and reps steps of
+ * the stationary iteration are timed from u = 0 as a solve runs them, with CUDA
+ * events on the handle's stream; the fastest is kept.  Outputs (host,
+ * nullable): the chosen rows_per_thread and map_blocks_per_sm and its ms per
+ * split step.  The handle's work buffers are overwritten.
  * The handle's curve groups are rebuilt for every candidate, so a batch built
  * over the handle before the call must be destroyed and built again (or
  * tuned with adr_batch_autotune, which rebuilds its own).  Errors:

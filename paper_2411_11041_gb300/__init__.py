@@ -127,11 +127,13 @@ EXPORTED = ["adr_default_opts", "adr_create", "adr_solve_stationary", "adr_step_
 
 def tune_key(prob, prec, transfer=0):
     """Cache key of a problem's launch shapes: grid, domain, field kind, precision
-    (and the direct transfer, which times other kernels)."""
+    (and the direct transfer, which runs other kernels).  The version changes with
+    the routes that a choice stands for: v2 choices were timed kernel by kernel,
+    also for the grids that solve in one launch."""
     b1, b2 = np.asarray(prob.beta1), np.asarray(prob.beta2)
     const = bool(np.all(b1 == b1.flat[0]) and np.all(b2 == b2.flat[0]))
     mask = np.asarray(prob.mask)
-    key = f"v2:{prob.nx}x{prob.ny}:{int(mask.sum())}:{'const' if const else 'curved'}:p{int(prec)}"
+    key = f"v3:{prob.nx}x{prob.ny}:{int(mask.sum())}:{'const' if const else 'curved'}:p{int(prec)}"
     return key + (":direct" if transfer else "")
 
 

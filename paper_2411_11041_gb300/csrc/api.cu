@@ -765,7 +765,25 @@ adr_status adr_autotune(adr_problem* h, int reps, int* rows_out, int* blocks_out
     const int rows[3] = {4, 8, 16}, blocks[3] = {2, 4, 8};
     double best = 1e300;
     int bR = p->rows_per_thread, bM = p->map_blocks_per_sm;
-    double ms[6];
+    const adr_opts& o = p->opts;
+    const double dt = o.dt > 0 ? o.dt : default_dt(*p, p->sigma);
+    // ms per step of reps steps of the iteration as a solve runs it (its graph,
+    // or the one launch where that applies), from u = 0: the second of two runs
+    // on, as the first factors the systems and builds the graph
+    auto measure = [&](double* ms) -> adr_status {
+        *ms = 1e300;
+        for (int k = 0; k < 4; ++k) {
+            adr_stats st;
+            clear_stats(&st);
+            bool conv = false;
+            TRY(init_state(h, ADR_INIT_ZERO, nullptr));
+            TRY(run_iteration(h, o.theta, dt, p->sigma, nullptr, 0.0, 0.0, reps, o.theta == 0.5, p->fextra, nullptr,
+                              &st, &conv));
+            h->diverged = false;
+            if (k > 0 && st.iters > 0) *ms = std::min(*ms, st.ms / st.iters);
+        }
+        return ADR_OK;
+    };
     for (int R : rows) {
         p->rows_per_thread = R;
         drop_graph(h);
@@ -773,10 +791,13 @@ adr_status adr_autotune(adr_problem* h, int reps, int* rows_out, int* blocks_out
             release_groups(p, fam);
             TRY(setup_groups(p, fam, h->offs[fam]));
         }
+        const bool loop = !o.anderson && loop_applies(p);
         for (int M : blocks) {
+            if (loop && M != 4) continue;  // the one launch has no map blocks of its own
             p->map_blocks_per_sm = M;
-            TRY(adr_time_kernels(h, reps, ms));
-            double t = ms[0] + ms[1] + ms[2] + ms[3] + ms[4] + ms[5];
+            drop_graph(h);
+            double t = 0.0;
+            TRY(measure(&t));
             if (t < best) {
                 best = t;
                 bR = R;

@@ -284,3 +284,23 @@ def test_solve_on_a_partition_of_the_sms(n):
             u, _, stats, _ = s.solve_stationary()
     torch.cuda.synchronize()
     assert stats["iters"] == 20 and torch.equal(u, ref)
+
+
+@pytest.mark.parametrize("n", [64, 257, 385])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_tuned_handle_is_no_slower(n, prec):
+    """The shapes adr_autotune keeps are the fastest of what a solve then runs:
+    a tuned handle takes at most the untuned one's time per step, and 8 % for
+    the spread of single runs."""
+    from paper_2411_11041_gb300 import Solver
+    s = Solver(_problem(n, n, "sheared", "square"), tol=0.0, max_iter=200, prec=prec)
+
+    def us_per_step():
+        s.solve_stationary()
+        return min(s.solve_stationary()[2]["ms"] for _ in range(5)) / 200 * 1e3
+
+    before = us_per_step()
+    rows, blocks, ms = s.autotune()
+    assert rows in (4, 8, 16) and blocks in (2, 4, 8)
+    after = us_per_step()
+    assert after <= 1.08 * before, (before, after, rows, blocks)
