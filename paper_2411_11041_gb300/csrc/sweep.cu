@@ -929,6 +929,7 @@ struct GridArgs {
     const IterState* state;
     int parity_shift;  // output buffer = parity(iter + shift)
     double* partial;   // [2 * gridDim.x] sums of (u - u_prev)^2 and u^2
+    int ltx;           // the tiles' width is 2^ltx nodes (map_tile)
 };
 
 // (dd, uu) summed over the warp: lane 0 gets dd, lane 16 uu (5 additions, as
@@ -1122,27 +1123,27 @@ __device__ __forceinline__ void grid_map_nodes(const GridArgs& a, double* __rest
 }
 
 // The same into the state buffer of the step's parity, block blk of nblk over
-// tiles of 32 x 8 nodes (a warp per row).  What bounds it is the FP64 pipe (8
-// products and, with the norms, 3 more per node: 63 and 87 us at 2048^2) and
-// L1's gather throughput (77 to 81 % busy): a curve that passes a tile is met by
-// several of its rows, so the tile shape decides how many of the 8 curve values
-// L1 already holds.  Measured at 2048^2 / 1024^2, without and with norms: runs
-// of 256 nodes along a row 84.2 and 109.0 / 23.3 and 34.9 us, 64 x 4 79.8 and
-// 98.4, 32 x 8 79.4 and 95.2 / 21.0 and 31.0, 16 x 16 80.2 and 96.4, 8 x 32 82.6
-// and 98.4.
+// tiles of 32 x 8 nodes (a warp per row; narrower where those would be mostly
+// padding: map_tile).  What bounds it is the FP64 pipe (8 products and, with the
+// norms, 3 more per node: 63 and 87 us at 2048^2) and L1's gather throughput
+// (77 to 81 % busy): a curve that passes a tile is met by several of its rows,
+// so the tile shape decides how many of the 8 curve values L1 already holds.
+// Measured at 2048^2 / 1024^2, without and with norms: runs of 256 nodes along a
+// row 84.2 and 109.0 / 23.3 and 34.9 us, 64 x 4 79.8 and 98.4, 32 x 8 79.4 and 95.2
+// / 21.0 and 31.0, 16 x 16 80.2 and 96.4, 8 x 32 82.6 and 98.4.
 template <bool NORMS>
 __device__ __forceinline__ void grid_map_tiles(const GridArgs& a, int blk, int nblk, double& dd, double& uu)
 {
-    constexpr int TX = 32, TY = kGridThreads / TX;
+    const int LX = a.ltx, TX = 1 << LX, TY = kGridThreads >> LX;
     const int it = a.state ? a.state->iter : 0;
     double* __restrict__ out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
     const double* __restrict__ prev = (it & 1) ? a.prev_odd : a.prev_even;
     const double* __restrict__ v = a.v;
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    const int ntx = (a.nx + TX - 1) / TX, nty = (a.ny + TY - 1) / TY;
+    const int tx = threadIdx.x & (TX - 1), ty = threadIdx.x >> LX;
+    const int ntx = (a.nx + TX - 1) >> LX, nty = (a.ny + TY - 1) / TY;
     const long long nt = (long long)ntx * nty;
     for (long long t = blk; t < nt; t += nblk) {
-        const int by = (int)(t / ntx), x = (int)(t - (long long)by * ntx) * TX + tx, y = by * TY + ty;
+        const int by = (int)(t / ntx), x = ((int)(t - (long long)by * ntx) << LX) + tx, y = by * TY + ty;
         if (x >= a.nx || y >= a.ny) continue;
         const long long k = (long long)y * a.nx + x;
         double val = 0.0;
@@ -2459,6 +2460,33 @@ adr_status launch_map_coef(Problem* p, int fam)
     return ADR_OK;
 }
 
+// tiles of 2^ltx x (256 / 2^ltx) nodes that cover the grid
+static long long map_tiles(int nx, int ny, int ltx)
+{
+    const int tx = 1 << ltx, ty = kGridThreads >> ltx;
+    return (long long)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty);
+}
+
+// width of the map's tiles (log2): 32, or the widest of 16, 8 and 4 that pads the
+// grid by at most an eighth, or the one that pads it least.  The padding's
+// threads are idle; otherwise the width makes little difference (1025^2: 4 21.3
+// and 27.1 us, 8 19.4 and 26.9, 32 20.0 and 27.7).  Measured, width 32 -> the one
+// taken, without and with norms: 5 x 60000 nodes 29.1 and 42.3 -> 9.3 and 14.3 us
+// (8), 9 x 40000 20.4 and 29.8 -> 7.7 and 11.6 (4), 33 x 12000 13.4 and 19.7 -> 8.8
+// and 13.2 (4), 48 x 8000 9.9 and 14.9 -> 8.1 and 12.7 (16), 60000 x 5 6.5 and 8.5
+// (32; 16: 9.3 and 11.5)
+static int map_tile(int nx, int ny)
+{
+    const long long N = (long long)nx * ny;
+    int best = 5;
+    for (int l = 5; l >= 2; --l) {
+        const long long pad = map_tiles(nx, ny, l) * kGridThreads - N;
+        if (8 * pad <= N) return l;
+        if (pad < map_tiles(nx, ny, best) * kGridThreads - N) best = l;
+    }
+    return best;
+}
+
 adr_status launch_grid_map_ex(Problem* p, int fam, double* out_even, double* out_odd,
                               int parity_shift, const double* prev_even, const double* prev_odd,
                               bool use_state, bool norms, const double* vin)
@@ -2478,6 +2506,7 @@ adr_status launch_grid_map_ex(Problem* p, int fam, double* out_even, double* out
     a.state = use_state ? p->state : nullptr;
     a.parity_shift = parity_shift;
     a.partial = p->partial;
+    a.ltx = map_tile(p->grid.nx, p->grid.ny);
     int blocks = grid_map_blocks(p);
     if (norms) launch_step(k_grid_map<true>, blocks, kGridThreads, 0, p->stream, a);
     else launch_step(k_grid_map<false>, blocks, kGridThreads, 0, p->stream, a);
@@ -2756,6 +2785,7 @@ adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const 
             g.v = p->fam[fam].v;
             g.state = p->state;
             g.partial = p->partial;
+            g.ltx = map_tile(p->grid.nx, p->grid.ny);
             if (fam == 0) {
                 g.out_even = g.out_odd = p->ubuf[2];
                 g.parity_shift = 0;
@@ -2772,7 +2802,7 @@ adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const 
         // curves of a problem differ, so items are per family): the batch
         // keeps one list per family and set
         {
-            const long long tiles = (long long)((p->grid.nx + 31) / 32) * ((p->grid.ny + 7) / 8);
+            const long long tiles = map_tiles(p->grid.nx, p->grid.ny, map_tile(p->grid.nx, p->grid.ny));
             nb[i] = (int)std::min<long long>(grid_map_blocks(p), (tiles + kBatchTiles - 1) / kBatchTiles);
         }
         for (int q = 0; q < nb[i]; ++q) {
