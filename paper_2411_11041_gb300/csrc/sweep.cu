@@ -29,10 +29,11 @@ namespace {
 
 constexpr int kCmax = 16;      // most rows per thread of the curve solve (kept in shared memory)
 constexpr int kGridThreads = 256;
-// 32 x 8-node tiles of one block of a batch's maps: a lone large problem at the
-// batch's end still spreads over every SM.  48 problems / the last one alone
-// (630 000 nodes), a split step: 2 tiles 1565 / 135 us, 4 1526 / 135, 8 1484 /
-// 149, 16 1441 / 192 (a block per tile or two: 1799 / 137)
+// tiles (of 256 nodes) of one block of a large batch's maps: a lone large problem
+// at the batch's end still spreads over every SM.  48 problems / the last one
+// alone (630 000 nodes), a split step: 2 tiles 1565 / 135 us, 4 1526 / 135, 8 1484
+// / 149, 16 1441 / 192 (a block per tile or two: 1799 / 137).  Small batches take
+// fewer (batch_tiles).
 constexpr int kBatchTiles = 4;
 
 // ---------------------------------------------------------------- curves
@@ -2723,6 +2724,16 @@ void batch_dev_destroy(BatchDev* b)
 static adr_status batch_dev_items(BatchDev* b, Problem* const* ps, int fam, BatchItem** items_out,
                                   int* counts, int* grids);
 
+// tiles of a block of a batch's maps and gathers, by the tiles of all problems:
+// with four a block a small batch leaves SMs idle.  Measured with 1/2/4 tiles, us a
+// step: two of 64^2 (32 tiles) 37.6/42.1/49.6, four of 129^2 (340) 48.4/49.7/53.9,
+// two of 257^2 (594) 57.2/55.5/61.1, six of 200 x 150 (798) 72.1/68.9/75.8, eight of
+// 257^2 (2376) 131/127/115
+static int batch_tiles(long long tiles, int n_sm)
+{
+    return tiles <= 3LL * n_sm ? 1 : (tiles <= 10LL * n_sm ? 2 : kBatchTiles);
+}
+
 // Build the device tables of a batch.  dts[i]: pseudo step of problem i.
 adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const double* tols,
                             const int* max_iters, BatchDev** out)
@@ -2748,6 +2759,10 @@ adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const 
     bool split = true;  // every problem has its gather pass
     for (int i = 0; i < n; ++i) split = split && ps[i]->fam[0].ug && ps[i]->fam[1].ug;
     std::vector<int> bp, bl, nb(n);
+    long long all_tiles = 0;
+    for (int i = 0; i < n; ++i)
+        all_tiles += map_tiles(ps[i]->grid.nx, ps[i]->grid.ny, map_tile(ps[i]->grid.nx, ps[i]->grid.ny));
+    const int per_block = batch_tiles(all_tiles, ps[0]->n_sm);
     std::vector<IterState*> sts(n);
     std::vector<double*> parts(n);
     for (int i = 0; i < n; ++i) {
@@ -2803,7 +2818,7 @@ adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const 
         // keeps one list per family and set
         {
             const long long tiles = map_tiles(p->grid.nx, p->grid.ny, map_tile(p->grid.nx, p->grid.ny));
-            nb[i] = (int)std::min<long long>(grid_map_blocks(p), (tiles + kBatchTiles - 1) / kBatchTiles);
+            nb[i] = (int)std::min<long long>(grid_map_blocks(p), (tiles + per_block - 1) / per_block);
         }
         for (int q = 0; q < nb[i]; ++q) {
             bp.push_back(i);

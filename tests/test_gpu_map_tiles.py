@@ -60,3 +60,18 @@ def test_thin_grids_cost_no_more_than_wide_ones():
 
     tall, wide = maps(5, 60000), maps(60000, 5)
     assert tall < 2.5 * wide, (tall, wide)
+
+
+@pytest.mark.parametrize("count,nx,ny", [(2, 64, 64), (6, 200, 150), (8, 257, 257)])  # 1, 2 and 4 tiles a block
+@pytest.mark.parametrize("prec", [0, 1])
+def test_batches_of_every_block_size_match_single_solves(count, nx, ny, prec):
+    import torch
+    from paper_2411_11041_gb300 import Batch, Solver
+    hs = [Solver(_problem(nx, ny, seed=k), tol=0.0, max_iter=5, prec=prec) for k in range(count)]
+    one = [h.solve_stationary() for h in hs]
+    ref = [(r[0].clone(), r[2]["rel_update"]) for r in one]
+    outs, stats, _ = Batch(hs).solve()
+    for u, (r, rel), st in zip(outs, ref, stats):
+        assert st["iters"] == 5 and torch.equal(u, r)
+        # the same squares summed in another order: n - 1 additions each rounding by 2^-53 at most
+        assert abs(st["rel_update"] - rel) <= nx * ny * 2.0 ** -53 * rel
