@@ -287,6 +287,16 @@ adr_status adr_autotune(adr_problem* prob, int reps, int* rows_per_thread,
                         int* map_blocks_per_sm, double* ms_per_step);
 
 /*
+ * adr_set_wait_limit -- bound of the grid-barrier waits of small grids' one-
+ * launch iteration: polls > 0, or 0 the default bound (several seconds).  A
+ * block whose wait reaches the bound gives up and leaves, and so do the others;
+ * the solve or step then reports ADR_ETIMEOUT, its outputs are not valid, and
+ * the handle can be used again.  A bound of one poll makes the waits give up,
+ * which is how that path is tested.  Errors: ADR_EINVAL.
+ */
+adr_status adr_set_wait_limit(adr_problem* prob, int polls);
+
+/*
  * Batches (many independent problems of uneven size and shape): every split
  * step of all active problems runs as one persistent launch per sweep stage,
  * over one list of work items (curves of all problems, longest first), and the

@@ -109,6 +109,7 @@ def lib():
         L.adr_cnn_initial_state.argtypes = [vp, vp, vp, vp, vp]
         L.adr_cnn_set_wait_limit.argtypes = [vp, C.c_longlong]
         L.adr_cnn_sync.argtypes = [vp]
+        L.adr_set_wait_limit.argtypes = [vp, C.c_int]
         L.adr_set_warm_start.argtypes = [vp, vp]
         _lib = L
     return _lib
@@ -122,7 +123,7 @@ EXPORTED = ["adr_default_opts", "adr_create", "adr_solve_stationary", "adr_step_
             "adr_cnn_num_params", "adr_cnn_create", "adr_cnn_destroy", "adr_cnn_set_params",
             "adr_cnn_get_params", "adr_cnn_features", "adr_cnn_targets", "adr_cnn_forward",
             "adr_cnn_loss_grad", "adr_cnn_train_step", "adr_cnn_initial_state",
-            "adr_cnn_set_wait_limit", "adr_cnn_sync", "adr_set_warm_start"]
+            "adr_cnn_set_wait_limit", "adr_cnn_sync", "adr_set_wait_limit", "adr_set_warm_start"]
 
 
 def tune_key(prob, prec, transfer=0):
@@ -362,6 +363,10 @@ class Solver:
         """Average device ms per launch of [B gather, B solve, B map, G gather,
         G solve, G map] (0 where a stage has no kernel of its own)."""
         return adr_time_kernels(self.h, reps)
+
+    def set_wait_limit(self, polls):
+        """Bound of the one-launch iteration's barrier waits in polls (0: the default)."""
+        _check(lib().adr_set_wait_limit(self.h, int(polls)), "adr_set_wait_limit")
 
     def line_unknowns(self):
         """Unknowns of one sweep of each family (curve nodes minus the ends)."""

@@ -158,6 +158,7 @@ struct Problem {
     int n_interior = 0;
     int n_sm = 0;
     bool coop = false;     // the device takes cooperative launches
+    int loop_spin = 0;     // bound of the one-launch iteration's barrier waits (0: the default)
     int stream_sms = 0;    // SMs the stream's kernels may use (fewer than n_sm on a partition)
     int rows_per_thread = 16;   // launch shape of the curve solve (<= 16 rows per thread)
     int map_blocks_per_sm = 4;  // launch shape of the curve -> grid map

@@ -818,6 +818,17 @@ adr_status adr_autotune(adr_problem* h, int reps, int* rows_out, int* blocks_out
     return ADR_OK;
 }
 
+adr_status adr_set_wait_limit(adr_problem* h, int polls)
+{
+    g_err.clear();
+    if (!h || polls < 0) {
+        set_error("adr_set_wait_limit: NULL handle or negative bound");
+        return ADR_EINVAL;
+    }
+    h->p.loop_spin = polls;
+    return ADR_OK;
+}
+
 adr_status adr_time_kernels(adr_problem* h, int reps, double* ms_out)
 {
     g_err.clear();

@@ -1490,10 +1490,11 @@ __global__ void k_check(IterState* st, const double* partial, int nblocks, doubl
 // Data that other blocks write during the launch (the grid states, the curve
 // values) is read by plain loads, which the barrier's acquire orders; the partial
 // sums come from L2.  (All of it from L2: a map at 513^2 24 instead of 17
-// thousand cycles, neighbouring nodes share their lines in L1.)  Barrier waits are bounded: a block that
-// gives up flags IterState::timeout and leaves, and so do the others.
+// thousand cycles, neighbouring nodes share their lines in L1.)
+// Barrier waits are bounded: a block that gives up flags IterState::timeout and
+// leaves, and so do the others.
 constexpr int kLoopThreads = 128;
-constexpr int kLoopSpin = 1 << 23;  // polls of one barrier wait (several seconds)
+constexpr int kLoopSpin = 1 << 23;  // default bound of a barrier wait in polls (several seconds)
 
 struct LoopArgs {
     CurveArgs c[2];
@@ -1507,10 +1508,11 @@ struct LoopArgs {
     double* partial;  // [2][2 * gridDim.x] by the step's parity
     double tol;
     int max_iter;
+    int spin;         // bound of a barrier wait in polls
 };
 
-// all blocks of the (cooperative) launch; *epoch counts the barriers passed
-__device__ __forceinline__ bool grid_barrier(IterState* st, unsigned& epoch)
+// all blocks of the (cooperative) launch; epoch counts the barriers passed
+__device__ __forceinline__ bool grid_barrier(IterState* st, int spin, unsigned& epoch)
 {
     __shared__ int ok;
     __syncthreads();
@@ -1519,7 +1521,7 @@ __device__ __forceinline__ bool grid_barrier(IterState* st, unsigned& epoch)
         const unsigned target = epoch * gridDim.x;
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&st->bar) : "memory");
         int good = 0;
-        for (int k = 0; k < kLoopSpin; ++k) {
+        for (int k = 0; k < spin; ++k) {
             unsigned c;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(&st->bar) : "memory");
             if ((int)(c - target) >= 0) {
@@ -1803,14 +1805,14 @@ __global__ void __launch_bounds__(kLoopThreads, 2) k_solve_loop(const __grid_con
         double dd = 0.0, uu = 0.0;
         loop_solve<GS, 0, REF>(a, u, hp, sm, corr, w0, pre);
         map_prefetch(a.g[0], first, mp);
-        if (!grid_barrier(a.state, epoch)) return;
+        if (!grid_barrier(a.state, a.spin, epoch)) return;
         grid_map_nodes<false>(a.g[0], a.g[0].out_even, nullptr, first, stride, dd, uu, mp);
         loop_prefetch(a.c[1], w1, pre);
-        if (!grid_barrier(a.state, epoch)) return;
+        if (!grid_barrier(a.state, a.spin, epoch)) return;
         if (REF && blockIdx.x == 0 && threadIdx.x == 0) a.state->corr_loop[(iter + 1) & 1] = 0ull;
         loop_solve<GS, 1, REF>(a, a.c[1].u_even, hp, sm, corr, w1, pre);
         map_prefetch(a.g[1], first, mp);
-        if (!grid_barrier(a.state, epoch)) return;
+        if (!grid_barrier(a.state, a.spin, epoch)) return;
         grid_map_nodes<true>(a.g[1], un, u, first, stride, dd, uu, mp);
         loop_prefetch(a.c[0], w0, pre);
         if (warp < nwarp) {
@@ -1824,7 +1826,7 @@ __global__ void __launch_bounds__(kLoopThreads, 2) k_solve_loop(const __grid_con
             for (int q = 1; q < nwarp; ++q) t += red[threadIdx.x][q];
             part[2 * blockIdx.x + threadIdx.x] = t;
         }
-        if (!grid_barrier(a.state, epoch)) return;
+        if (!grid_barrier(a.state, a.spin, epoch)) return;
         ++iter;
         if (warp == 0) {
             // every block: the same sums in the same order
@@ -2602,6 +2604,7 @@ adr_status launch_solve_loop(Problem* p, double dt, const double* u_even, double
     a.partial = p->partial;
     a.tol = tol;
     a.max_iter = max_iter;
+    a.spin = p->loop_spin > 0 ? p->loop_spin : kLoopSpin;
     const int blocks = loop_blocks(p);
     const bool ref = p->opts.prec == ADR_FP32_REFINE;
     cudaError_t e = cudaSuccess;

@@ -304,3 +304,29 @@ def test_tuned_handle_is_no_slower(n, prec):
     assert rows in (4, 8, 16) and blocks in (2, 4, 8)
     after = us_per_step()
     assert after <= 1.08 * before, (before, after, rows, blocks)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_barrier_timeout_is_reported_and_the_handle_recovers(prec):
+    """A bound of one poll makes the grid barriers of the one-launch iteration give
+    up: the blocks leave, and the solve and the time steps report ADR_ETIMEOUT.
+    With the default bound restored the same handle solves as before, bit for
+    bit."""
+    import torch
+    from paper_2411_11041_gb300 import AdrError, Solver
+    p = _problem(129, 120, "sheared", "square")
+    s = Solver(p, tol=0.0, max_iter=25, prec=prec)
+    u0, _, st0, _ = s.solve_stationary()
+    u0 = u0.clone()
+    s.set_wait_limit(1)
+    with pytest.raises(AdrError, match="ETIMEOUT"):
+        s.solve_stationary()
+    for mode in (0, 1):
+        with pytest.raises(AdrError, match="ETIMEOUT"):
+            s.step_parabolic(u0.clone(), 1e-3, 3, mode)
+    with pytest.raises(AdrError, match="EINVAL"):
+        s.set_wait_limit(-1)
+    s.set_wait_limit(0)
+    u, _, st, _ = s.solve_stationary()
+    assert torch.equal(u, u0)
+    assert (st["iters"], st["rel_update"], st["max_correction"]) == (25, st0["rel_update"], st0["max_correction"])
