@@ -9,6 +9,7 @@
 #include <cstdio>
 
 #include "adr_internal.cuh"
+#include "unit_component.cuh"
 
 namespace adr {
 namespace {
@@ -787,50 +788,6 @@ __device__ __forceinline__ bool seed_of(const int* nseeds, int cap, int t, int* 
     return false;
 }
 
-// ---- one direction component, num / sqrt(s), as direction computes it
-// A warp's FP64 instruction takes 64 cycles, dependent or not, whatever the
-// number of active lanes; the compiler's square root and division take about 9
-// each, half of a stage.  Here 1/sqrt(s) comes from the FP32 pipe (about 5
-// cycles an instruction) to 2^-45: the hardware estimate r0 and one
-// second-order step on e = 1 - s r0^2, e formed exactly enough by FMA
-// residuals.  Square root and quotient then follow Markstein's scheme (IBM J.
-// Res. Dev. 34, 1990): an approximation, its exact residual by FMA, and one
-// corrected rounding.  The value rounded last is within 2^-89 (relative) of the
-// true one, so the result is the correctly rounded one, as sqrt and / give,
-// unless the true value lies that close to a rounding boundary (one in 2^35).
-__device__ __forceinline__ double f32_widen(float x)  // exact for normal x, integer pipe
-{
-    const unsigned b = __float_as_uint(x);
-    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
-}
-
-__device__ __forceinline__ double unit_component(double num, double s, bool& bad)
-{
-    const unsigned hi = (unsigned)__double2hiint(s), lo = (unsigned)__double2loint(s);
-    if (hi - (963u << 20) < (120u << 20)) {  // 2^-60 <= s < 2^60
-        // s = sh + sl exactly, both FP32
-        const float sh = __uint_as_float(__funnelshift_r(lo, hi, 29) - (384u << 23));
-        const float sl = __uint2float_rn(lo & 0x1fffffffu) * __uint_as_float(((hi >> 20) - 1023u - 52u + 127u) << 23);
-        const float r0 = rsqrtf(sh);
-        const float p = r0 * r0, pe = __fmaf_rn(r0, r0, -p);
-        const float t = sh * p, te = __fmaf_rn(sh, p, -t);
-        float e = (1.0f - t) - te;
-        e = __fmaf_rn(-sh, pe, e);
-        e = __fmaf_rn(-sl, p, e);
-        const float rl = r0 * (e * __fmaf_rn(0.375f, e, 0.5f));
-        double y = f32_widen(r0);
-        if (fabsf(rl) >= 1.1754944e-38f) y = y + f32_widen(rl);
-        const double hy = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));  // y / 2
-        double g = s * y;
-        g = __fma_rn(__fma_rn(-g, g, s), hy, g);
-        const double q = num * y;
-        return __fma_rn(__fma_rn(-q, g, num), y, q);
-    }
-    const double nrm = sqrt(s);
-    if (!(nrm > 0.0)) bad = true;
-    return num / nrm;
-}
-
 // cell index and local coordinate of c as bilin takes them (q clamped to [0,
 // lim], l = c - q); plain: c >= 0 lies strictly inside cell q, away from its
 // ends by more than the snapping tolerance (then snap leaves c alone and
@@ -843,7 +800,7 @@ struct Split {
 __device__ __forceinline__ Split split(double c, int lim, double limd)
 {
     Split r;
-    const unsigned hi = (unsigned)__double2hiint(c), lo = (unsigned)__double2loint(c);
+    const unsigned hi = (unsigned)__double2hiint(c);
     double qd = 0.0;
     if (hi < (1043u << 20)) {  // 0 <= c < 2^20
         const int e = (int)(hi >> 20) - 1023;
@@ -860,7 +817,6 @@ __device__ __forceinline__ Split split(double c, int lim, double limd)
         r.l = c - qd;
         const unsigned hl = (unsigned)__double2hiint(r.l);
         r.plain = hl - (994u << 20) < 0x3fefffffu - (994u << 20);  // 2^-29 <= l < 1 - 2^-21
-        (void)lo;
         return r;
     }
     r.q = r.qu = __double2int_rd(c);
