@@ -408,7 +408,7 @@ def run_ours(args):
     # the gathers are passes of their own in FP64 through the grid; + the
     # extrapolation's 3 kernels
     per_step = (5 if direct else 7) + (3 if args.anderson else 0)
-    if one_launch(args.n, direct, args.anderson):
+    if solver.one_launch():
         launches = 4 * len(iters)
     else:
         launches = int(sum(per_step * it + (5 if direct else 3) for it in iters))
@@ -943,11 +943,6 @@ def kernel_units(solver, prob, unknowns, direct=False):
     return [nodes[0], unknowns[0], prob.nx * prob.ny, nodes[1], unknowns[1], prob.nx * prob.ny]
 
 
-def one_launch(n, direct, anderson):
-    """Grids of up to 2^18 nodes run the whole plain iteration in one launch."""
-    return n * n <= 1 << 18 and not direct and not anderson
-
-
 def kernel_roofline(solver, prob, unknowns, direct=False):
     """Dominant sweep kernel of a solver, timed with CUDA events in the
     solve's launch configuration (adr_time_kernels): the roofline object."""
@@ -1054,7 +1049,7 @@ def run_parabolic(args):
                        "step": f"one {nsteps}-step run from the Gaussian blob",
                        "l2": "working set ~250 MB > 129 MB L2"},
             "roofline": roof,
-            "gpu_launches": int((nsteps if one_launch(n, False, args.anderson) else
+            "gpu_launches": int((nsteps if s.one_launch() else
                                  iters[-1] * (7 + (3 if args.anderson else 0)))
                                 + nsteps * 4), "clocks": clk,
             "err_vs_oracle": {"measure": "max |u - u_oracle| / max |u_oracle|",

@@ -287,6 +287,13 @@ adr_status adr_autotune(adr_problem* prob, int reps, int* rows_per_thread,
                         int* map_blocks_per_sm, double* ms_per_step);
 
 /*
+ * adr_one_launch -- whether the handle's stationary solves and implicit time
+ * slices run as the one launch of small grids (*one = 1) or as the graph of
+ * separate kernels (0).  Errors: ADR_EINVAL.
+ */
+adr_status adr_one_launch(adr_problem* prob, int* one);
+
+/*
  * adr_set_wait_limit -- bound of the grid-barrier waits of small grids' one-
  * launch iteration: polls > 0, or 0 the default bound (several seconds).  A
  * block whose wait reaches the bound gives up and leaves, and so do the others;

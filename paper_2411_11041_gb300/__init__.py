@@ -110,6 +110,7 @@ def lib():
         L.adr_cnn_set_wait_limit.argtypes = [vp, C.c_longlong]
         L.adr_cnn_sync.argtypes = [vp]
         L.adr_set_wait_limit.argtypes = [vp, C.c_int]
+        L.adr_one_launch.argtypes = [vp, C.POINTER(C.c_int)]
         L.adr_set_warm_start.argtypes = [vp, vp]
         _lib = L
     return _lib
@@ -123,7 +124,8 @@ EXPORTED = ["adr_default_opts", "adr_create", "adr_solve_stationary", "adr_step_
             "adr_cnn_num_params", "adr_cnn_create", "adr_cnn_destroy", "adr_cnn_set_params",
             "adr_cnn_get_params", "adr_cnn_features", "adr_cnn_targets", "adr_cnn_forward",
             "adr_cnn_loss_grad", "adr_cnn_train_step", "adr_cnn_initial_state",
-            "adr_cnn_set_wait_limit", "adr_cnn_sync", "adr_set_wait_limit", "adr_set_warm_start"]
+            "adr_cnn_set_wait_limit", "adr_cnn_sync", "adr_set_wait_limit", "adr_one_launch",
+            "adr_set_warm_start"]
 
 
 def tune_key(prob, prec, transfer=0):
@@ -363,6 +365,12 @@ class Solver:
         """Average device ms per launch of [B gather, B solve, B map, G gather,
         G solve, G map] (0 where a stage has no kernel of its own)."""
         return adr_time_kernels(self.h, reps)
+
+    def one_launch(self):
+        """Whether solves run as one launch (small grids) or as the graph of kernels."""
+        one = C.c_int()
+        _check(lib().adr_one_launch(self.h, C.byref(one)), "adr_one_launch")
+        return bool(one.value)
 
     def set_wait_limit(self, polls):
         """Bound of the one-launch iteration's barrier waits in polls (0: the default)."""

@@ -818,6 +818,17 @@ adr_status adr_autotune(adr_problem* h, int reps, int* rows_out, int* blocks_out
     return ADR_OK;
 }
 
+adr_status adr_one_launch(adr_problem* h, int* one)
+{
+    g_err.clear();
+    if (!h || !one) {
+        set_error("adr_one_launch: NULL argument");
+        return ADR_EINVAL;
+    }
+    *one = h->p.opts.anderson == 0 && loop_applies(&h->p) ? 1 : 0;
+    return ADR_OK;
+}
+
 adr_status adr_set_wait_limit(adr_problem* h, int polls)
 {
     g_err.clear();

@@ -330,3 +330,26 @@ def test_barrier_timeout_is_reported_and_the_handle_recovers(prec):
     u, _, st, _ = s.solve_stationary()
     assert torch.equal(u, u0)
     assert (st["iters"], st["rel_update"], st["max_correction"]) == (25, st0["rel_update"], st0["max_correction"])
+
+
+@pytest.mark.parametrize("nx,ny,opts,one", [
+    (64, 64, {}, True),
+    (400, 400, {}, True),                          # the largest grid of the one launch
+    (401, 400, {}, False),
+    (64, 64, dict(transfer=1), False),
+    (64, 64, dict(anderson=2), False),
+    (385, 385, dict(rows_per_thread=4), False),    # 128 threads a curve
+    (385, 385, dict(rows_per_thread=16), True),
+])
+def test_route_of_a_solve(nx, ny, opts, one):
+    """What the handle reports is what a solve then does: only the one launch
+    waits at barriers, so a bound of one poll ends it and nothing else."""
+    from paper_2411_11041_gb300 import AdrError, Solver
+    s = Solver(_problem(nx, ny, "sheared", "square"), tol=0.0, max_iter=5, **opts)
+    assert s.one_launch() == one
+    s.set_wait_limit(1)
+    if one:
+        with pytest.raises(AdrError, match="ETIMEOUT"):
+            s.solve_stationary()
+    else:
+        assert s.solve_stationary()[2]["iters"] == 5
