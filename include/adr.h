@@ -435,11 +435,16 @@ adr_status adr_cnn_features(int batch, int n, const double* f, const double* bet
 adr_status adr_cnn_targets(int batch, int n, const double* u, const double* u0,
                            const double* scale, float* t, void* stream);
 /* adr_cnn_forward: y (device float [batch][64][64][8]) <- the network's output.
- * Launch only, on the handle's stream.  Errors: ADR_EINVAL, ADR_ECUDA. */
+ * Launch only, on the handle's stream.  Errors: ADR_EINVAL, ADR_ECUDA.
+ * Parameters and inputs are to be finite: taps outside the image are 0 by being
+ * left out where a whole tile of pixels lies outside, so an infinite or NaN
+ * weight does not reach those pixels (0 times it would be NaN). */
 adr_status adr_cnn_forward(adr_cnn* cnn, int batch, const uint16_t* x, float* y);
 /* adr_cnn_loss_grad: forward and backward without an update.  grad (nullable
  * device float[num_params]) <- d loss / d params; loss (nullable host) <- the
- * loss (the call then waits for the stream). */
+ * loss (the call then waits for the stream).  Output channels 1..7 do not enter
+ * the loss: the gradients of their weights and biases are 0, whatever the
+ * activations hold. */
 adr_status adr_cnn_loss_grad(adr_cnn* cnn, int batch, const uint16_t* x, const float* t,
                              float* grad, double* loss);
 /* adr_cnn_train_step: forward, backward and one Adam step (beta1 0.9, beta2

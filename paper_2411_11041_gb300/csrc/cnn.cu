@@ -767,7 +767,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     // the pairs with a tap whose window meets the image (the others' x is all
     // zero fill): at dilations 16 and 32 a good part of the windows drop out
     auto live = [&](int y0, int x0) -> unsigned {
-        if (!wide) return (1u << ng) - 1u;  // dilations up to 4: every window meets it
+        // dilations up to 4: only the windows of the image's first and last 4 rows
+        // at dilation 4 miss it, 3 taps of 9 each, and zero fill makes them right
+        if (!wide) return (1u << ng) - 1u;
         unsigned mk = 0u;
         for (int g = 0; g < ng; ++g) {
             const int tap = wgrad_tap(g0 + g), y = y0 + (tap / 3 - 1) * a.dil, x = x0 + (tap % 3 - 1) * a.dil;
