@@ -1837,6 +1837,7 @@ __global__ void __launch_bounds__(kLoopThreads, 2) k_solve_loop(const __grid_con
             if (lane == 0) {
                 // the square root and the division (20 FP64 instructions) only where
                 // they decide: a relative update clearly above every threshold goes on
+                // (fixed steps by tol < 0 do them each time: lim^2 is positive there)
                 const double lim = 2.0 * a.tol * (REF && !hp ? kHpSwitch : 1.0);
                 int flag = 0;
                 if (iter >= a.max_iter || !(num > lim * lim * den) || !(den > 0.0) || !isfinite(num) || !isfinite(den)) {
@@ -2534,20 +2535,26 @@ static int loop_blocks(const Problem* p)
 
 // one-launch iteration: problems through the grid whose curves take at most
 // 64 threads (the groups' tables fit shared memory) and whose step is bound by
-// latency: few enough nodes, and at most three slices a group.  Many short
-// curves take longer here than as blocks of their own (17 x 4000 nodes, 5.5
-// slices a group: 37.9 us a step, the graph 35.2; 4000 x 17 38.7 and 32.3; 17 x
-// 2000, 2.7 slices: 22.5 and 29.4)
+// latency: few enough nodes, fewer in proportion where a group has more than one
+// slice, and at most three slices a group.  Where the curves are many and short
+// their slices come in rounds, which take longer than as blocks of their own.
+// Nodes times slices a group, us a step here and as the graph: 1000 x 100 141 000,
+// 37.1 and 37.4; 800 x 140 133 000, 38.0 and 40.1; 700 x 200 156 000, 41.9 and
+// 43.9; 120 x 1000 172 000, 42.0 and 40.8; 800 x 180 177 000, 44.7 and 42.6; 1000 x
+// 150 219 000, 46.2 and 43.4; 80 x 1500 246 000, 43.9 and 39.8; 2000 x 75 405 000,
+// 47.9 and 42.3.  17 x 4000, 5.5 slices: 37.9 and 35.2; 17 x 2000, 2.7 slices: 22.5
+// and 29.4.
 bool loop_applies(const Problem* p)
 {
     if (p->opts.transfer || p->n_sm <= 0 || !p->coop) return false;
+    long long slices = 0;
+    for (const Family& F : p->fam) {
+        if (!F.iset[0].count || F.iset[1].count || F.iset[2].count || F.tmax > 64) return false;
+        slices = std::max(slices, (long long)F.iset[0].count * (256 / kLoopThreads));
+    }
+    const long long sms = p->stream_sms;
     // on a partition of the SMs (it has to hold all blocks at once) its share of the nodes
-    if ((long long)p->N * p->n_sm > (long long)kLoopMaxNodes * p->stream_sms) return false;
-    for (const Family& F : p->fam)
-        if (!F.iset[0].count || F.iset[1].count || F.iset[2].count || F.tmax > 64 ||
-            F.iset[0].count * (256 / kLoopThreads) > 3 * p->stream_sms)
-            return false;
-    return true;
+    return slices <= 3 * sms && p->N * std::max(slices, sms) * p->n_sm <= kLoopMaxNodes * sms * sms;
 }
 
 template <int GS, bool REF>

@@ -340,6 +340,10 @@ def test_barrier_timeout_is_reported_and_the_handle_recovers(prec):
     (64, 64, dict(anderson=2), False),
     (385, 385, dict(rows_per_thread=4), False),    # 128 threads a curve
     (385, 385, dict(rows_per_thread=16), True),
+    (1000, 100, {}, True),                         # 1.5 slices a group
+    (1000, 150, {}, False),                        # as many, and more nodes
+    (80, 1500, {}, False),
+    (2000, 50, {}, False),                         # nearly three
 ])
 def test_route_of_a_solve(nx, ny, opts, one):
     """What the handle reports is what a solve then does: only the one launch
