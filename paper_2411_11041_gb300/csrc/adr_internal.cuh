@@ -296,13 +296,17 @@ adr_status launch_mask_copy(Problem* p, const double* in, double* out);
 // make the iteration's factorisation family 0's active one (sweep.cu); a
 // batch reads the active buffers once, when it is built
 adr_status ensure_iteration_active(Problem* p);
-// the outer iteration in one cooperative launch (sweep.cu), measured faster up
-// to about 400^2 nodes (385^2 45.0 us a step, the graph 48.9; 420^2 55 and 56);
+// the outer iteration in one cooperative launch (sweep.cu), up to 300^2 nodes;
 // larger grids take the graph of separate kernels, whose blocks fill the chip
-// by themselves.  Near the limit two handles on two streams gain as well (385^2
-// 70 us for both, graphs 84), four or more would be better off as graphs (141
-// and 112)
-constexpr int kLoopMaxNodes = 400 * 400;
+// by themselves.  A handle alone gains up to about 400^2 (385^2 44.9 us a step,
+// the graph 49.7; 420^2 55 and 56), but at most two launches share the device:
+// us a step for all of 1 / 2 / 4 / 8 handles on streams of their own, here and as
+// graphs: 257^2 32 / 33 / 66 / 131 and 40 / 47 / 71 / 124, 300^2 35 / 38 / 80 / 158
+// and 42 / 57 / 83 / 140, 340^2 40 / 54 / 111 / 214 and 45 / 70 / 95 / 159, 385^2
+// 45 / 70 / 142 / 282 and 50 / 86 / 111 / 189.
+constexpr int kLoopMaxNodes = 300 * 300;
+// its limit of nodes times slices of curves a group (loop_applies)
+constexpr int kLoopMaxWork = 120000;
 bool loop_applies(const Problem* p);
 // *launched = false: the runtime refused the launch, nothing was enqueued and
 // the handle takes the graph from now on

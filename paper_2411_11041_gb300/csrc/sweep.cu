@@ -2535,15 +2535,15 @@ static int loop_blocks(const Problem* p)
 
 // one-launch iteration: problems through the grid whose curves take at most
 // 64 threads (the groups' tables fit shared memory) and whose step is bound by
-// latency: few enough nodes, fewer in proportion where a group has more than one
-// slice, and at most three slices a group.  Where the curves are many and short
-// their slices come in rounds, which take longer than as blocks of their own.
-// Nodes times slices a group, us a step here and as the graph: 1000 x 100 141 000,
-// 37.1 and 37.4; 800 x 140 133 000, 38.0 and 40.1; 700 x 200 156 000, 41.9 and
-// 43.9; 120 x 1000 172 000, 42.0 and 40.8; 800 x 180 177 000, 44.7 and 42.6; 1000 x
-// 150 219 000, 46.2 and 43.4; 80 x 1500 246 000, 43.9 and 39.8; 2000 x 75 405 000,
-// 47.9 and 42.3.  17 x 4000, 5.5 slices: 37.9 and 35.2; 17 x 2000, 2.7 slices: 22.5
-// and 29.4.
+// latency: few enough nodes, fewer where a group has more than one slice, and at
+// most three slices a group.  Where the curves are many and short their slices
+// come in rounds, which take longer than as blocks of their own.
+// Nodes times slices a group, us a step here and as the graph: 1000 x 60 91 000,
+// 28.2 and 36.4 (eight handles on streams 119 and 112); 1000 x 80 123 000, 33.5 and
+// 40.2 (150 and 127: past the line); 800 x 140 133 000, 38.0 and 40.1; 120 x 1000
+// 172 000, 42.0 and 40.8; 800 x 180 177 000, 44.7 and 42.6; 80 x 1500 246 000, 43.9
+// and 39.8; 2000 x 75 405 000, 47.9 and 42.3.  17 x 4000, 5.5 slices: 37.9 and 35.2;
+// 17 x 2000, 2.7 slices: 22.5 and 29.4.
 bool loop_applies(const Problem* p)
 {
     if (p->opts.transfer || p->n_sm <= 0 || !p->coop) return false;
@@ -2554,7 +2554,8 @@ bool loop_applies(const Problem* p)
     }
     const long long sms = p->stream_sms;
     // on a partition of the SMs (it has to hold all blocks at once) its share of the nodes
-    return slices <= 3 * sms && p->N * std::max(slices, sms) * p->n_sm <= kLoopMaxNodes * sms * sms;
+    return slices <= 3 * sms && (long long)p->N * p->n_sm <= kLoopMaxNodes * sms &&
+           p->N * slices * p->n_sm <= kLoopMaxWork * sms * sms;
 }
 
 template <int GS, bool REF>

@@ -197,8 +197,10 @@ def test_small_solves_overlap(n, k):
 
 
 @pytest.mark.parametrize("nx,ny,field", [
-    (400, 400, "sheared"),               # the largest grid of the one launch
-    (401, 400, "sheared"),               # the first of the separate kernels
+    (300, 300, "sheared"),               # the largest grid of the one launch
+    (301, 300, "sheared"),               # the first of the separate kernels
+    (400, 400, "sheared"),
+    (401, 400, "sheared"),
     (17, 2200, (0.8, 0.6)),              # near three slices a group
     (17, 2400, (0.8, 0.6)),              # past them: separate kernels
     (600, 260, (1.0, 0.0)),              # 64 threads a curve, two groups a block
@@ -334,14 +336,16 @@ def test_barrier_timeout_is_reported_and_the_handle_recovers(prec):
 
 @pytest.mark.parametrize("nx,ny,opts,one", [
     (64, 64, {}, True),
-    (400, 400, {}, True),                          # the largest grid of the one launch
-    (401, 400, {}, False),
+    (300, 300, {}, True),                          # the largest grid of the one launch
+    (301, 300, {}, False),
+    (400, 400, {}, False),
     (64, 64, dict(transfer=1), False),
     (64, 64, dict(anderson=2), False),
-    (385, 385, dict(rows_per_thread=4), False),    # 128 threads a curve
-    (385, 385, dict(rows_per_thread=16), True),
-    (1000, 100, {}, True),                         # 1.5 slices a group
-    (1000, 150, {}, False),                        # as many, and more nodes
+    (290, 290, dict(rows_per_thread=4), False),    # 128 threads a curve
+    (290, 290, dict(rows_per_thread=16), True),
+    (1000, 60, {}, True),                          # 1.5 slices a group
+    (1000, 80, {}, False),                         # as many, and more nodes
+    (1400, 64, {}, False),
     (80, 1500, {}, False),
     (2000, 50, {}, False),                         # nearly three
 ])
@@ -357,3 +361,37 @@ def test_route_of_a_solve(nx, ny, opts, one):
             s.solve_stationary()
     else:
         assert s.solve_stationary()[2]["iters"] == 5
+
+
+def test_large_solves_share_the_device():
+    """Eight handles of 385^2 on eight streams: separate kernels, whose steps take
+    turns at the device's full rate (below five times one handle's time; as
+    single launches, at most two of which fit the device at once, 6.3)."""
+    import threading
+    import time
+
+    import torch
+    from paper_2411_11041_gb300 import Solver
+    streams = [torch.cuda.Stream() for _ in range(8)]
+    hs = [Solver(_problem(385, 385, "sheared", "square", seed=i), tol=0.0, max_iter=1000, stream=streams[i])
+          for i in range(8)]
+    torch.cuda.synchronize()
+
+    def seconds(m):
+        go = threading.Barrier(m + 1)
+
+        def work(i):
+            with torch.cuda.stream(streams[i]):
+                go.wait()
+                hs[i].solve_stationary()
+
+        th = [threading.Thread(target=work, args=(i,)) for i in range(m)]
+        [t.start() for t in th]
+        go.wait()
+        t0 = time.perf_counter()
+        [t.join() for t in th]
+        return time.perf_counter() - t0
+
+    seconds(8)
+    one, all_ = min(seconds(1) for _ in range(3)), min(seconds(8) for _ in range(3))
+    assert all_ < 5.0 * one, (one, all_)
