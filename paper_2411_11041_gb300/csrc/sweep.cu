@@ -29,6 +29,7 @@ namespace {
 
 constexpr int kCmax = 16;      // most rows per thread of the curve solve (kept in shared memory)
 constexpr int kGridThreads = 256;
+constexpr int kWideTile = 5;  // log2 of the widest map tile
 // tiles (of 256 nodes) of one block of a large batch's maps: a lone large problem
 // at the batch's end still spreads over every SM.  48 problems / the last one
 // alone (630 000 nodes), a split step: 2 tiles 1565 / 135 us, 4 1526 / 135, 8 1484
@@ -1132,10 +1133,12 @@ __device__ __forceinline__ void grid_map_nodes(const GridArgs& a, double* __rest
 // Measured at 2048^2 / 1024^2, without and with norms: runs of 256 nodes along a
 // row 84.2 and 109.0 / 23.3 and 34.9 us, 64 x 4 79.8 and 98.4, 32 x 8 79.4 and 95.2
 // / 21.0 and 31.0, 16 x 16 80.2 and 96.4, 8 x 32 82.6 and 98.4.
-template <bool NORMS>
+// WIDE: tiles of 32 x 8, a constant (with the width from a.ltx the map with norms
+// took 88.3 instead of 87.1 us at 2048^2).
+template <bool NORMS, bool WIDE>
 __device__ __forceinline__ void grid_map_tiles(const GridArgs& a, int blk, int nblk, double& dd, double& uu)
 {
-    const int LX = a.ltx, TX = 1 << LX, TY = kGridThreads >> LX;
+    const int LX = WIDE ? kWideTile : a.ltx, TX = 1 << LX, TY = kGridThreads >> LX;
     const int it = a.state ? a.state->iter : 0;
     double* __restrict__ out = ((it + a.parity_shift) & 1) ? a.out_odd : a.out_even;
     const double* __restrict__ prev = (it & 1) ? a.prev_odd : a.prev_even;
@@ -1170,13 +1173,13 @@ __device__ __forceinline__ void grid_map_tiles(const GridArgs& a, int blk, int n
     }
 }
 
-template <bool NORMS>
+template <bool NORMS, bool WIDE>
 __global__ void __launch_bounds__(kGridThreads) k_grid_map(GridArgs a)
 {
     step_entry();
     if (a.state && a.state->done) return;
     double dd = 0.0, uu = 0.0;
-    grid_map_tiles<NORMS>(a, blockIdx.x, gridDim.x, dd, uu);
+    grid_map_tiles<NORMS, WIDE>(a, blockIdx.x, gridDim.x, dd, uu);
     if (NORMS) block_sum2(dd, uu, a.partial + 2 * blockIdx.x);
 }
 
@@ -1222,7 +1225,7 @@ struct BlockWalk {
 // a problem) the norms' block sums alone took 116 us of SM time a step for 48
 // problems of 13 M nodes (10 FP64 additions a warp, 24 000 blocks), 551 us in
 // all.
-template <bool NORMS>
+template <bool NORMS, bool WIDE>
 __global__ void __launch_bounds__(kGridThreads) k_grid_map_batch(const GridArgs* __restrict__ table,
                                                                 int fam, const int* blk_prob,
                                                                 const int* blk_local, const int* nblk,
@@ -1236,7 +1239,7 @@ __global__ void __launch_bounds__(kGridThreads) k_grid_map_batch(const GridArgs*
         const GridArgs& a = table[2 * w.p + fam];
         if (a.state->done) continue;  // uniform per block
         double dd = 0.0, uu = 0.0;
-        grid_map_tiles<NORMS>(a, w.lb, nblk[w.p], dd, uu);
+        grid_map_tiles<NORMS, WIDE>(a, w.lb, nblk[w.p], dd, uu);
         if (NORMS) {
             block_sum2(dd, uu, a.partial + 2 * w.lb);
             __syncthreads();  // its shared array is reused
@@ -2482,8 +2485,8 @@ static long long map_tiles(int nx, int ny, int ltx)
 static int map_tile(int nx, int ny)
 {
     const long long N = (long long)nx * ny;
-    int best = 5;
-    for (int l = 5; l >= 2; --l) {
+    int best = kWideTile;
+    for (int l = kWideTile; l >= 2; --l) {
         const long long pad = map_tiles(nx, ny, l) * kGridThreads - N;
         if (8 * pad <= N) return l;
         if (pad < map_tiles(nx, ny, best) * kGridThreads - N) best = l;
@@ -2512,8 +2515,10 @@ adr_status launch_grid_map_ex(Problem* p, int fam, double* out_even, double* out
     a.partial = p->partial;
     a.ltx = map_tile(p->grid.nx, p->grid.ny);
     int blocks = grid_map_blocks(p);
-    if (norms) launch_step(k_grid_map<true>, blocks, kGridThreads, 0, p->stream, a);
-    else launch_step(k_grid_map<false>, blocks, kGridThreads, 0, p->stream, a);
+    const bool wide = a.ltx == kWideTile;
+    auto* kernel = norms ? (wide ? k_grid_map<true, true> : k_grid_map<true, false>)
+                         : (wide ? k_grid_map<false, true> : k_grid_map<false, false>);
+    launch_step(kernel, blocks, kGridThreads, 0, p->stream, a);
     ADR_CUDA_TRY(cudaGetLastError());
     return ADR_OK;
 }
@@ -2701,6 +2706,7 @@ struct BatchDev {
     const BatchItem** d_items = nullptr;  // [6] item arrays per family and set
     int* d_n_items = nullptr;             // [6]
     int map_grid = 0;
+    bool wide = true;  // every problem's map has tiles of 32 x 8
     // work items per family and set, with their persistent grid sizes
     BatchItem* it[2][kItemSets] = {};
     int nit[2][kItemSets] = {};
@@ -2812,6 +2818,7 @@ adr_status batch_dev_create(Problem* const* ps, int n, const double* dts, const 
             g.state = p->state;
             g.partial = p->partial;
             g.ltx = map_tile(p->grid.nx, p->grid.ny);
+            if (g.ltx != kWideTile) b->wide = false;
             if (fam == 0) {
                 g.out_even = g.out_odd = p->ubuf[2];
                 g.parity_shift = 0;
@@ -2999,13 +3006,11 @@ adr_status batch_dev_step(BatchDev* b, cudaStream_t st, cudaGraphConditionalHand
         }                                                                                          \
     }
     ADR_BATCH_SOLVE(0, itB, nB, gB)
-    launch_step(k_grid_map_batch<false>, b->map_grid, kGridThreads, 0, st, b->gtab, 0, b->blk_prob, b->blk_local,
-                                                                 b->nblk, b->act.blocks_dev, b->act.count,
-                                                                 b->act.sel);
+    launch_step(b->wide ? k_grid_map_batch<false, true> : k_grid_map_batch<false, false>, b->map_grid, kGridThreads, 0,
+                st, b->gtab, 0, b->blk_prob, b->blk_local, b->nblk, b->act.blocks_dev, b->act.count, b->act.sel);
     ADR_BATCH_SOLVE(1, itG, nG, gG)
-    launch_step(k_grid_map_batch<true>, b->map_grid, kGridThreads, 0, st, b->gtab, 1, b->blk_prob, b->blk_local,
-                                                                b->nblk, b->act.blocks_dev, b->act.count,
-                                                                b->act.sel);
+    launch_step(b->wide ? k_grid_map_batch<true, true> : k_grid_map_batch<true, false>, b->map_grid, kGridThreads, 0,
+                st, b->gtab, 1, b->blk_prob, b->blk_local, b->nblk, b->act.blocks_dev, b->act.count, b->act.sel);
 #undef ADR_BATCH_SOLVE
 #undef ADR_BATCH_SOLVE_BS
     launch_step(k_check_batch, b->n, 256, 0, st, b->states, (const double* const*)b->partials, b->nblk, b->n,
