@@ -254,8 +254,9 @@ adr_status dev_alloc(Problem* p, T** ptr, size_t count)
 // kernel, before anything is read or any thread returns).  About 0.7 us a
 // kernel: 513^2 74.5 -> 71.7 us a step, 1024^2 146 -> 143, direct transfer at
 // 257^2 32.2 -> 30.1.  Letting the successor in earlier (launch_dependents at
-// its predecessor's start) costs 25 to 40 %: the blocks that wait hold shared
-// memory that is the running kernel's L1.
+// its predecessor's start) costs 18 to 39 % (2048^2 54.5 -> 64.5 ms a solve, 513^2
+// 7.25 -> 10.09): the blocks that wait hold shared memory that is the running
+// kernel's L1.
 #ifdef __CUDACC__
 __device__ __forceinline__ void step_entry()
 {
